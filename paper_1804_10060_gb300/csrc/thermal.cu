@@ -15,11 +15,11 @@
 //         - theta int_Gamma beta phi_j phi_i
 // The steady problem drops the mass terms and takes theta = 1.
 //
-// Integration: the mass terms use the reference tensors int phi_a phi_b phi_c
-// and int phi_a phi_b, the conduction terms quadrature at every point, the
-// Robin terms the face mass matrix -- all exact for the polynomial degrees
-// involved, from Gauss-Jacobi product (Stroud conical) rules generated here
-// on the host.
+// Integration: every term is a contraction of nodal values with integrals over
+// the reference cell (int phi_a phi_b phi_c, int phi_a lambda_b lambda_c, ...;
+// the cells are affine), the Robin terms use the face mass matrix -- all exact
+// for the polynomial degrees involved, the tables from Gauss-Jacobi product
+// (Stroud conical) rules generated here on the host.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -131,52 +131,34 @@ double face_phi(int deg, int a, const double* m) {
 }
 
 // ---------------------------------------------------------------------------
-// Constant tables (filled once per device by thermal_tables()):
-//   d_T3p2[a][b][c] = int phi_a phi_b phi_c / |K| (P2), d_M2p2 = int phi_a phi_b / |K|,
-//   the same for P1, the face mass matrices int psi_a psi_b / |F|, and the P2
-//   conduction rule (11 points: barycentrics and weights / |K|) with the P2
-//   basis values there.  The P2 tables the kernel indexes per lane live in
-//   global memory (read through L1): constant memory serialises a warp's
-//   accesses to different addresses.
+// Constant tables (filled once per device by thermal_tables()), all integrals
+// divided by the cell's (face's) measure.  P1: int phi_a phi_b phi_c and
+// int phi_a phi_b; faces: int psi_a psi_b.  P2, for the pair index of i <= j
+// below and the moment rows r (0..9: lambda_a lambda_b, a <= b; 10..13:
+// lambda_a; 14: 1):
+//   c_T3s[pair][c]  = int phi_i phi_j phi_c,  c_M2s[pair] = int phi_i phi_j
+//   c_mom[r][c]     = int (row r) phi_c,      c_mom0[r]   = int (row r)
+//   c_gv[j][a][m]   = int phi_j (4 lambda_a - 1) lambda_m   (vertex gradients)
+//   c_ge[j][a][m]   = int phi_j 4 lambda_a lambda_m         (edge gradients)
+// Every access is warp-uniform (a warp works on one entry of 32 cells), which
+// is what constant memory serves in one step.
 // ---------------------------------------------------------------------------
-constexpr int NQ2 = 11;
-__device__ double d_T3p2[10][10][10];
-__device__ double d_M2p2[10][10];
 __constant__ double c_T3p1[4][4][4];
 __constant__ double c_M2p1[4][4];
 __constant__ double c_F2p2[6][6];
 __constant__ double c_F2p1[3][3];
-__device__ double d_qc[NQ2][5];  // l0..l3, weight (sum 1)
+__constant__ double c_T3s[55][10];
+__constant__ double c_M2s[55];
+__constant__ double c_mom[15][10];
+__constant__ double c_mom0[15];
+__constant__ double c_gv[10][4][4];
+__constant__ double c_ge[10][4][4];
 
-// Keast's 11-point rule on the tetrahedron: exact for every polynomial of
-// degree <= 4 (one negative weight); barycentrics and weights normalised to
-// sum 1.  Degree 4 is what the P2 conduction integrands reach (kappa(T_theta)
-// grad phi_i . grad phi_j: 2 + 1 + 1; k1 phi_j grad T_theta . grad phi_i: the same).
-void keast11(std::vector<double>& p, std::vector<double>& w) {
-  p.clear();
-  w.clear();
-  auto add = [&](const double (&l)[4], double wt) {
-    p.insert(p.end(), l, l + 4);
-    w.push_back(wt);
-  };
-  add({0.25, 0.25, 0.25, 0.25}, -6.0 * 74.0 / 5625.0);
-  for (int k = 0; k < 4; ++k) {
-    double l[4] = {1.0 / 14.0, 1.0 / 14.0, 1.0 / 14.0, 1.0 / 14.0};
-    l[k] = 11.0 / 14.0;
-    add(l, 6.0 * 343.0 / 45000.0);
-  }
-  const double a = (1.0 + std::sqrt(5.0 / 14.0)) / 4.0, b = (1.0 - std::sqrt(5.0 / 14.0)) / 4.0;
-  for (int i = 0; i < 4; ++i)
-    for (int j = i + 1; j < 4; ++j) {
-      double l[4] = {b, b, b, b};
-      l[i] = l[j] = a;
-      add(l, 6.0 * 56.0 / 2250.0);
-    }
-}
+// index of the pair i <= j in a symmetric n x n array stored by rows
+__host__ __device__ constexpr int pair_index(int i, int j, int n) { return i * n - i * (i - 1) / 2 + (j - i); }
 
 std::mutex g_tab_mutex;
 bool g_tab_ready[64] = {};
-void thermal_point_values();
 
 void thermal_tables() {
   int dev = 0;
@@ -186,17 +168,35 @@ void thermal_tables() {
   if (g_tab_ready[dev]) return;
   std::vector<double> p, w;
   tet_rule(4, p, w);  // degree 7 >= 6 (three P2 functions)
-  double T3[10][10][10] = {}, M2[10][10] = {}, T3a[4][4][4] = {}, M2a[4][4] = {};
+  double T3[55][10] = {}, M2[55] = {}, T3a[4][4][4] = {}, M2a[4][4] = {};
+  double mom[15][10] = {}, mom0[15] = {}, gv[10][4][4] = {}, ge[10][4][4] = {};
   for (size_t q = 0; q < w.size(); ++q) {
     const double* l = &p[4 * q];
     double f2[10], f1[4];
     for (int a = 0; a < 10; ++a) f2[a] = cell_phi(2, a, l);
     for (int a = 0; a < 4; ++a) f1[a] = cell_phi(1, a, l);
     for (int a = 0; a < 10; ++a)
-      for (int b = 0; b < 10; ++b) {
-        M2[a][b] += w[q] * f2[a] * f2[b];
-        for (int c = 0; c < 10; ++c) T3[a][b][c] += w[q] * f2[a] * f2[b] * f2[c];
+      for (int b = a; b < 10; ++b) {
+        const int pi = pair_index(a, b, 10);
+        M2[pi] += w[q] * f2[a] * f2[b];
+        for (int c = 0; c < 10; ++c) T3[pi][c] += w[q] * f2[a] * f2[b] * f2[c];
       }
+    double row[15];
+    for (int a = 0; a < 4; ++a) {
+      for (int b = a; b < 4; ++b) row[pair_index(a, b, 4)] = l[a] * l[b];
+      row[10 + a] = l[a];
+    }
+    row[14] = 1.0;
+    for (int r = 0; r < 15; ++r) {
+      mom0[r] += w[q] * row[r];
+      for (int c = 0; c < 10; ++c) mom[r][c] += w[q] * row[r] * f2[c];
+    }
+    for (int j = 0; j < 10; ++j)
+      for (int a = 0; a < 4; ++a)
+        for (int m = 0; m < 4; ++m) {
+          gv[j][a][m] += w[q] * f2[j] * (4.0 * l[a] - 1.0) * l[m];
+          ge[j][a][m] += w[q] * f2[j] * 4.0 * l[a] * l[m];
+        }
     for (int a = 0; a < 4; ++a)
       for (int b = 0; b < 4; ++b) {
         M2a[a][b] += w[q] * f1[a] * f1[b];
@@ -213,33 +213,17 @@ void thermal_tables() {
     for (int a = 0; a < 3; ++a)
       for (int b = 0; b < 3; ++b) F1[a][b] += fw[q] * face_phi(1, a, m) * face_phi(1, b, m);
   }
-  keast11(p, w);  // degree 4 (kappa(T_theta) grad phi . grad phi on P2)
-  double qc[NQ2][5];
-  for (int q = 0; q < NQ2; ++q) {
-    for (int k = 0; k < 4; ++k) qc[q][k] = p[4 * q + k];
-    qc[q][4] = w[q];
-  }
-  TAM_CUDA(cudaMemcpyToSymbol(d_T3p2, T3, sizeof(T3)));
-  TAM_CUDA(cudaMemcpyToSymbol(d_M2p2, M2, sizeof(M2)));
+  TAM_CUDA(cudaMemcpyToSymbol(c_T3s, T3, sizeof(T3)));
+  TAM_CUDA(cudaMemcpyToSymbol(c_M2s, M2, sizeof(M2)));
+  TAM_CUDA(cudaMemcpyToSymbol(c_mom, mom, sizeof(mom)));
+  TAM_CUDA(cudaMemcpyToSymbol(c_mom0, mom0, sizeof(mom0)));
+  TAM_CUDA(cudaMemcpyToSymbol(c_gv, gv, sizeof(gv)));
+  TAM_CUDA(cudaMemcpyToSymbol(c_ge, ge, sizeof(ge)));
   TAM_CUDA(cudaMemcpyToSymbol(c_T3p1, T3a, sizeof(T3a)));
   TAM_CUDA(cudaMemcpyToSymbol(c_M2p1, M2a, sizeof(M2a)));
   TAM_CUDA(cudaMemcpyToSymbol(c_F2p2, F2, sizeof(F2)));
   TAM_CUDA(cudaMemcpyToSymbol(c_F2p1, F1, sizeof(F1)));
-  TAM_CUDA(cudaMemcpyToSymbol(d_qc, qc, sizeof(qc)));
-  thermal_point_values();
   g_tab_ready[dev] = true;
-}
-
-// P2 basis values at the conduction points (cell-independent)
-__device__ double d_phic[NQ2][10];
-
-void thermal_point_values() {
-  std::vector<double> p, w;
-  keast11(p, w);
-  double ph[NQ2][10];
-  for (int q = 0; q < NQ2; ++q)
-    for (int a = 0; a < 10; ++a) ph[q][a] = cell_phi(2, a, &p[4 * q]);
-  TAM_CUDA(cudaMemcpyToSymbol(d_phic, ph, sizeof(ph)));
 }
 
 // ---------------------------------------------------------------------------
@@ -326,126 +310,170 @@ __global__ void thermal_p1_kernel(ThArgs A) {
   }
 }
 
-// P2: a warp per cell.  The lanes first evaluate, at the 11 conduction points,
-// the basis gradients, grad T_theta and kappa(T_theta) (into shared memory),
-// then grad T_theta . grad phi_i per point, the symmetric conduction sums
-// once per pair i <= j, and finally the 100 Jacobian and 10 residual entries
-// (FP64 is GB300's slow pipe: the symmetric part and the mass sums are not
-// recomputed per entry).
-constexpr int P2T_WARPS = 4;
+// P2: 32 cells per block, one per lane; the block's warps share out the
+// entries.  The FP64 pipe (2 lanes per cycle and SM) bounds this kernel, so
+// the integrals are contracted instead of summed over quadrature points: with
+// grad phi_a = (4 lambda_a - 1) G_a on vertices, 4 (lambda_q G_p + lambda_p G_q)
+// on the edge (p, q), g_kl = vol G_k . G_l and
+//   m_r      = int kappa(T_theta) (row r of c_mom): 15 moments of kappa,
+//   sig_km   : grad T_theta . G_k vol = sum_m sig_km lambda_m (grad T_theta is linear),
+// the conduction part of an entry is at most four products m g, the
+// non-symmetric part at most eight products sig x table, and F's conduction
+// part is sum_j (conduction_ij) T_theta,j -- with the nodal values taken
+// relative to the first vertex's, which a gradient does not see and which
+// leaves little to cancel.  About 3,300 FP64 operations a cell where an
+// 11-point rule took 13,000: 11.0 -> 1.9 ms on 305,280 cells (floor of the
+// operations at the measured FP64 rate: 1.6 ms).  A warp works on one pair (i, j) for its
+// 32 cells at a time: all lanes busy, table indices warp-uniform, per-cell
+// quantities in shared memory by [quantity][cell] (no bank conflicts).
+constexpr int P2T_WARPS = 8, P2T_CELLS = 32;  // one cell per lane
 
 __global__ void __launch_bounds__(P2T_WARPS * 32) thermal_p2_kernel(ThArgs A) {
-  __shared__ double sg[P2T_WARPS][NQ2][10][3];
-  __shared__ double sq[P2T_WARPS][NQ2][5];   // kappa w vol, k1 w vol, grad T_theta
-  __shared__ double st[P2T_WARPS][2][10];    // T_theta, (T - T_old)/dt
-  __shared__ double stg[P2T_WARPS][NQ2][10]; // grad T_theta . grad phi_i per point
-  __shared__ double ssym[P2T_WARPS][55];     // symmetric conduction part, pairs i <= j
-  __shared__ double sw[P2T_WARPS][10];       // mass weights
-  __shared__ int sv[P2T_WARPS][10];
+  __shared__ double sT[10][32], sD[10][32];     // T_theta, (T - T_old) / dt
+  __shared__ double sg[10][32];                 // vol G_k . G_l, k <= l
+  __shared__ double sm[15][32];                 // moments of kappa
+  __shared__ double ssig[16][32];               // sig_km
+  __shared__ double svol[32];
+  __shared__ double scond[55][32], smass[55][32];  // per pair: conduction part, rho vol int c_v phi_i phi_j
+  __shared__ int sv[10][32];
+  __shared__ unsigned char sok[32];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c = blockIdx.x * P2T_WARPS + wid;
-  if (c >= A.n_cells) return;  // warp-uniform
-  if (lane < 10) sv[wid][lane] = A.cells[(size_t)c * 10 + lane];
-  __syncwarp();
-  double g[4][3], vol;
-  if (!tet_geometry(A.X, sv[wid], g, vol)) {
-    if (lane == 0) atomicExch(A.bad, 1);
-    return;
+  const long long c0 = (long long)blockIdx.x * P2T_CELLS;
+  const int c = (int)min(c0 + lane, (long long)A.n_cells - 1);  // idle lanes repeat the last cell, unscattered
+  for (int t = threadIdx.x; t < 320; t += P2T_WARPS * 32) {
+    const int cl = t / 10;
+    sv[t - cl * 10][cl] = A.cells[min(c0 + cl, (long long)A.n_cells - 1) * 10 + (t - cl * 10)];
   }
-  const double* pr = A.props + 5 * A.mat[c];
-  const double rho = pr[0], c0 = pr[1], c1 = pr[2], k0 = pr[3], k1 = pr[4];
+  __syncthreads();
   const bool steady = A.T_old == nullptr;
   const double th = steady ? 1.0 : A.theta;
-  if (lane < 10) {
-    const int n = sv[wid][lane];
-    const double t = A.T[n];
-    st[wid][0][lane] = steady ? t : (1.0 - th) * A.T_old[n] + th * t;
-    st[wid][1][lane] = steady ? 0.0 : (t - A.T_old[n]) / A.dt;
-  }
-  __syncwarp();
-  if (lane < NQ2) {
-    const int q = lane;
-    const double* l = d_qc[q];
-    double tq = 0.0, gt[3] = {0.0, 0.0, 0.0};
-    for (int a = 0; a < 10; ++a) {
-      double gr[3];
-      if (a < 4) {
-        const double s = 4.0 * l[a] - 1.0;
-        for (int d = 0; d < 3; ++d) gr[d] = s * g[a][d];
-      } else {
-        const int e = a - 4;  // edges 01, 02, 03, 12, 13, 23
-        const int p0 = e < 3 ? 0 : (e < 5 ? 1 : 2), p1 = e < 3 ? e + 1 : (e == 3 ? 2 : 3);
-        for (int d = 0; d < 3; ++d) gr[d] = 4.0 * (l[p1] * g[p0][d] + l[p0] * g[p1][d]);
-      }
-      const double ta = st[wid][0][a];
-      tq += ta * __ldg(&d_phic[q][a]);
-      for (int d = 0; d < 3; ++d) {
-        sg[wid][q][a][d] = gr[d];
-        gt[d] += ta * gr[d];
-      }
+  const double* pr = A.props + 5 * A.mat[c];
+  const double rho = pr[0], c0m = pr[1], c1 = pr[2], k0 = pr[3], k1 = pr[4];
+  if (wid == 0) {
+    int v[4];
+    for (int a = 0; a < 4; ++a) v[a] = sv[a][lane];
+    double g[4][3], vol;
+    const bool ok = tet_geometry(A.X, v, g, vol);
+    if (!ok) atomicExch(A.bad, 1);
+    sok[lane] = ok && c0 + lane < A.n_cells;
+    if (ok) {
+      svol[lane] = vol;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int l = k; l < 4; ++l)
+          sg[pair_index(k, l, 4)][lane] = vol * (g[k][0] * g[l][0] + g[k][1] * g[l][1] + g[k][2] * g[l][2]);
     }
-    const double wv = l[4] * vol;
-    sq[wid][q][0] = (k0 + k1 * tq) * wv;
-    sq[wid][q][1] = k1 * wv;
-    for (int d = 0; d < 3; ++d) sq[wid][q][2 + d] = gt[d];
+  } else {
+    for (int a = wid - 1; a < 10; a += P2T_WARPS - 1) {
+      const int n = sv[a][lane];
+      const double t = A.T[n];
+      sT[a][lane] = steady ? t : (1.0 - th) * A.T_old[n] + th * t;
+      sD[a][lane] = steady ? 0.0 : (t - A.T_old[n]) / A.dt;
+    }
   }
-  __syncwarp();
-  // per point and basis function: tg[q][i] = grad T_theta . grad phi_i
-  for (int e = lane; e < NQ2 * 10; e += 32) {
-    const int q = e / 10, i = e - q * 10;
-    const double* gi = sg[wid][q][i];
-    const double* sp = sq[wid][q];
-    stg[wid][q][i] = sp[2] * gi[0] + sp[3] * gi[1] + sp[4] * gi[2];
+  __syncthreads();
+  double T[10], D[10];
+#pragma unroll
+  for (int a = 0; a < 10; ++a) {
+    T[a] = sT[a][lane];
+    D[a] = sD[a][lane];
   }
-  // mass weights: (T3 is symmetric in its three indices) the mass part of
-  // J_ij is rho vol (c0 M_ij / dt + sum_b T3_ijb w_b), w_b = c1 (theta dT_b/dt + T_theta,b / dt)
-  if (!steady && lane < 10) sw[wid][lane] = c1 * (th * st[wid][1][lane] + st[wid][0][lane] / A.dt);
-  __syncwarp();
-  // the symmetric conduction part, sum_q kappa w vol grad phi_i . grad phi_j, once per pair i <= j
-  for (int e = lane; e < 55; e += 32) {
-    int i = 0, r = e;
+  const double vol = svol[lane];
+  for (int r = wid; r < 15; r += P2T_WARPS) {
+    double m = 0.0;
+#pragma unroll
+    for (int a = 0; a < 10; ++a) m = fma(c_mom[r][a], T[a], m);
+    sm[r][lane] = fma(k1, m, k0 * c_mom0[r]);
+  }
+  for (int e = wid; e < 16; e += P2T_WARPS) {
+    // dT_theta/dlambda_l = sum_m tau_lm lambda_m: tau_ll = 3 T_l, tau_lm = 4 T_edge(l,m) - T_l
+    const int k = e >> 2, m = e & 3;
+    double s = 0.0;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const double g = sg[k < l ? pair_index(k, l, 4) : pair_index(l, k, 4)][lane];
+      double tau = 3.0 * (T[l] - T[0]);
+      if (l != m) {
+        const int lo = l < m ? l : m, hi = l < m ? m : l;   // edges 01, 02, 03, 12, 13, 23
+        tau = fma(4.0, sT[lo == 0 ? 3 + hi : lo + hi + 4][lane] - T[0], T[0] - T[l]);
+      }
+      s = fma(g, tau, s);
+    }
+    ssig[e][lane] = s;
+  }
+  __syncthreads();
+  const double rv = rho * vol, idt = steady ? 0.0 : 1.0 / A.dt;
+  const bool ok = sok[lane] != 0;
+  for (int pidx = wid; pidx < 55; pidx += P2T_WARPS) {
+    int i = 0, r = pidx;
     while (r >= 10 - i) {
       r -= 10 - i;
       ++i;
     }
     const int j = i + r;
-    double acc = 0.0;
-    for (int q = 0; q < NQ2; ++q) {
-      const double* gi = sg[wid][q][i];
-      const double* gj = sg[wid][q][j];
-      acc += sq[wid][q][0] * (gj[0] * gi[0] + gj[1] * gi[1] + gj[2] * gi[2]);
+    // edge ends (i, j >= 4)
+    const int ie = i - 4, je = j - 4;
+    const int ip = ie < 3 ? 0 : (ie < 5 ? 1 : 2), iq = ie < 3 ? ie + 1 : (ie == 3 ? 2 : 3);
+    const int jp = je < 3 ? 0 : (je < 5 ? 1 : 2), jq = je < 3 ? je + 1 : (je == 3 ? 2 : 3);
+    auto g = [&](int k, int l) { return sg[k < l ? pair_index(k, l, 4) : pair_index(l, k, 4)][lane]; };
+    auto m = [&](int k, int l) { return sm[k < l ? pair_index(k, l, 4) : pair_index(l, k, 4)][lane]; };
+    double cond;
+    if (j < 4) {          // vertex, vertex: int kappa (4 l_i - 1)(4 l_j - 1)
+      cond = g(i, j) * fma(16.0, m(i, j), fma(-4.0, sm[10 + i][lane] + sm[10 + j][lane], sm[14][lane]));
+    } else if (i < 4) {   // vertex, edge
+      cond = 4.0 * fma(fma(4.0, m(i, jq), -sm[10 + jq][lane]), g(i, jp),
+                       fma(4.0, m(i, jp), -sm[10 + jp][lane]) * g(i, jq));
+    } else {              // edge, edge
+      cond = 16.0 * fma(m(iq, jq), g(ip, jp), fma(m(iq, jp), g(ip, jq), fma(m(ip, jq), g(iq, jp), m(ip, jp) * g(iq, jq))));
     }
-    ssym[wid][e] = acc;
-  }
-  __syncwarp();
-  for (int e = lane; e < 110; e += 32) {
-    if (e < 100) {
-      const int i = e / 10, j = e % 10;
-      const int lo = i < j ? i : j, hi = i < j ? j : i;
-      double acc = ssym[wid][lo * 10 - lo * (lo - 1) / 2 + (hi - lo)];
-      for (int q = 0; q < NQ2; ++q) acc += sq[wid][q][1] * __ldg(&d_phic[q][j]) * stg[wid][q][i];
-      acc *= th;
-      if (!steady) {
-        double m = c0 * __ldg(&d_M2p2[i][j]) / A.dt;
-        for (int b2 = 0; b2 < 10; ++b2) m += sw[wid][b2] * __ldg(&d_T3p2[i][j][b2]);
-        acc += rho * vol * m;
-      }
-      scatter_J(A, sv[wid][i], sv[wid][j], acc);
-    } else {
-      const int i = e - 100;
-      double f = 0.0;
-      for (int q = 0; q < NQ2; ++q) f += sq[wid][q][0] * stg[wid][q][i];
-      if (!steady) {
-        double m = 0.0;
-        for (int b2 = 0; b2 < 10; ++b2) {
-          double cb = c0 * __ldg(&d_M2p2[b2][i]);
-          for (int a2 = 0; a2 < 10; ++a2) cb += c1 * st[wid][0][a2] * __ldg(&d_T3p2[a2][b2][i]);
-          m += st[wid][1][b2] * cb;
+    // non-symmetric part int phi_b grad T_theta . grad phi_a for (a, b) = (i, j) and (j, i)
+    auto nonsym = [&](int a, int p, int q, int b) {
+      double s = 0.0;
+      if (a < 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s = fma(ssig[4 * a + k][lane], c_gv[b][a][k], s);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          s = fma(ssig[4 * p + k][lane], c_ge[b][q][k], s);
+          s = fma(ssig[4 * q + k][lane], c_ge[b][p][k], s);
         }
-        f += rho * vol * m;
       }
-      if (!A.dmask[sv[wid][i]]) atomicAdd(&A.F[sv[wid][i]], f);
+      return s;
+    };
+    const double nij = nonsym(i, ip, iq, j);
+    double mass = 0.0, jm = 0.0;
+    if (!steady) {
+      // int T_theta phi_i phi_j and int dT/dt phi_i phi_j
+      double a1 = 0.0, a2 = 0.0;
+#pragma unroll
+      for (int a = 0; a < 10; ++a) {
+        a1 = fma(c_T3s[pidx][a], T[a], a1);
+        a2 = fma(c_T3s[pidx][a], D[a], a2);
+      }
+      mass = rv * fma(c1, a1, c0m * c_M2s[pidx]);
+      jm = fma(mass, idt, rv * c1 * th * a2);
     }
+    scond[pidx][lane] = cond;
+    smass[pidx][lane] = mass;
+    if (ok) scatter_J(A, sv[i][lane], sv[j][lane], fma(th, fma(k1, nij, cond), jm));
+    if (i != j) {
+      const double nji = nonsym(j, jp, jq, i);
+      if (ok) scatter_J(A, sv[j][lane], sv[i][lane], fma(th, fma(k1, nji, cond), jm));
+    }
+  }
+  __syncthreads();
+  for (int i = wid; i < 10; i += P2T_WARPS) {
+    double f = 0.0;
+#pragma unroll
+    for (int j = 0; j < 10; ++j) {
+      const int p = i < j ? pair_index(i, j, 10) : pair_index(j, i, 10);
+      f = fma(scond[p][lane], T[j] - T[0], f);
+      f = fma(smass[p][lane], D[j], f);
+    }
+    const int n = sv[i][lane];
+    if (ok && !A.dmask[n]) atomicAdd(&A.F[n], f);
   }
 }
 
@@ -572,7 +600,7 @@ void thermal_assemble(tam_thermal_s* th, const double* T, const double* T_old, d
     if (th->npc == 4)
       thermal_p1_kernel<<<grid_for(th->n_cells, 128), 128, 0, s>>>(a);
     else
-      thermal_p2_kernel<<<grid_for(th->n_cells, P2T_WARPS), P2T_WARPS * 32, 0, s>>>(a);
+      thermal_p2_kernel<<<grid_for(th->n_cells, P2T_CELLS), P2T_WARPS * 32, 0, s>>>(a);
     TAM_LAUNCH_CHECK();
   }
   if (th->n_faces > 0) {
