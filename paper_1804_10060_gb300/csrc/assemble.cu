@@ -352,160 +352,251 @@ __global__ void __launch_bounds__(128) assemble_p1_kernel(AsmArgs A) {
   }
 }
 
-// P2 quadrature.  Stiffness integrand is degree 2: 4-point rule with
-// barycentric points (A,B,B,B) and permutations, A = (5+3 sqrt5)/20,
-// B = (5-sqrt5)/20, equal weights 1/4.  Loads are degree 3 (thermal) and 4
-// (body): Keast's 11-point degree-4 rule (weights normalised to sum 1).
-__constant__ double c_q4[4][4] = {
-    {0.5854101966249685, 0.1381966011250105, 0.1381966011250105, 0.1381966011250105},
-    {0.1381966011250105, 0.5854101966249685, 0.1381966011250105, 0.1381966011250105},
-    {0.1381966011250105, 0.1381966011250105, 0.5854101966249685, 0.1381966011250105},
-    {0.1381966011250105, 0.1381966011250105, 0.1381966011250105, 0.5854101966249685}};
-__constant__ double c_k11[11][5] = {  // l0, l1, l2, l3, weight
-    {0.25, 0.25, 0.25, 0.25, -0.078933333333333333},
-    {0.7857142857142857, 0.0714285714285714, 0.0714285714285714, 0.0714285714285714, 0.045733333333333333},
-    {0.0714285714285714, 0.7857142857142857, 0.0714285714285714, 0.0714285714285714, 0.045733333333333333},
-    {0.0714285714285714, 0.0714285714285714, 0.7857142857142857, 0.0714285714285714, 0.045733333333333333},
-    {0.0714285714285714, 0.0714285714285714, 0.0714285714285714, 0.7857142857142857, 0.045733333333333333},
-    {0.3994035761667992, 0.3994035761667992, 0.1005964238332008, 0.1005964238332008, 0.149333333333333333},
-    {0.3994035761667992, 0.1005964238332008, 0.3994035761667992, 0.1005964238332008, 0.149333333333333333},
-    {0.3994035761667992, 0.1005964238332008, 0.1005964238332008, 0.3994035761667992, 0.149333333333333333},
-    {0.1005964238332008, 0.3994035761667992, 0.3994035761667992, 0.1005964238332008, 0.149333333333333333},
-    {0.1005964238332008, 0.3994035761667992, 0.1005964238332008, 0.3994035761667992, 0.149333333333333333},
-    {0.1005964238332008, 0.1005964238332008, 0.3994035761667992, 0.3994035761667992, 0.149333333333333333}};
+// P2 reference integrals / |K| (affine cells).  With grad phi_a =
+// (4 lambda_a - 1) G_a on vertices and 4 (lambda_q G_p + lambda_p G_q) on the
+// edge (p, q), a P2 stiffness block is a sum of at most four of the P1 blocks
+// B_kl = vol (lam G_k G_l^T + mu G_l G_k^T + mu (G_k . G_l) I):
+//   vertex a, vertex b:  0.6 B_aa, or -0.2 B_ab
+//   vertex a, edge pq:   c_q B_ap + c_p B_aq, c_k = int (4 l_a - 1) 4 l_k = 0.6 (k = a) or -0.2
+//   edge pq, edge rs:    d_qs B_pr + d_qr B_ps + d_ps B_qr + d_pr B_qs, d_kl = int 16 l_k l_l = 1.6 (k = l) or 0.8
+// The loads contract nodal values with int phi_a phi_b (body) and
+// int phi_c lambda_k (thermal).  All exact for the polynomial degrees involved.
 __constant__ int c_edge[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
 
-__device__ __forceinline__ double p2_phi(int a, const double* l) {
-  if (a < 4) return l[a] * (2.0 * l[a] - 1.0);
-  return 4.0 * l[c_edge[a - 4][0]] * l[c_edge[a - 4][1]];
+// int phi_a phi_b / |K| of two P2 functions
+__device__ __forceinline__ double p2_mass(int a, int b) {
+  const int lo = a < b ? a : b, hi = a < b ? b : a;
+  if (hi < 4) return lo == hi ? 6.0 / 420.0 : 1.0 / 420.0;
+  const int r = c_edge[hi - 4][0], s = c_edge[hi - 4][1];
+  if (lo < 4) return (lo == r || lo == s) ? -4.0 / 420.0 : -6.0 / 420.0;
+  if (lo == hi) return 32.0 / 420.0;
+  const int p = c_edge[lo - 4][0], q = c_edge[lo - 4][1];
+  return (p == r || p == s || q == r || q == s) ? 16.0 / 420.0 : 8.0 / 420.0;
 }
 
-__device__ __forceinline__ void p2_grad(int a, const double* l, const double g[4][3], double out[3]) {
-  if (a < 4) {
-    double s = 4.0 * l[a] - 1.0;
-    for (int d = 0; d < 3; ++d) out[d] = s * g[a][d];
-  } else {
-    int p = c_edge[a - 4][0], q = c_edge[a - 4][1];
-    for (int d = 0; d < 3; ++d) out[d] = 4.0 * (l[q] * g[p][d] + l[p] * g[q][d]);
+// int phi_c lambda_k / |K|
+__device__ __forceinline__ double p2_moment(int c, int k) {
+  if (c < 4) return c == k ? 0.0 : -1.0 / 60.0;
+  return (c_edge[c - 4][0] == k || c_edge[c - 4][1] == k) ? 4.0 / 60.0 : 2.0 / 60.0;
+}
+
+// Where the 3x3 block k (row na, column nb; local a, b of cell c) goes: its
+// slot in K's values, or -1 when it went elsewhere (the deterministic mode's
+// own slot, the load of a prescribed column) or nowhere.  fixed: nb is a
+// Dirichlet node.
+__device__ __forceinline__ int block_slot(const AsmArgs& A, int c, int a, int b, int na, int nb, bool fixed,
+                                          const double (&k)[9]) {
+  if (A.ck || fixed || A.loads_only) {
+    scatter_block(A, c, a, b, na, nb, k);
+    return -1;
   }
+  return bsearch_i32(A.col_idx, A.row_ptr[na], A.row_ptr[na + 1], nb);
 }
 
-constexpr int P2_WARPS = 4;
+// P2: 32 cells per block, one per lane; the block's warps share out the 55
+// node pairs a <= b.  The FP64 pipe (2 lanes per cycle and SM) and the atomic
+// scatter bound this kernel: the contraction of the ten P1 blocks takes about
+// 2,000 FP64 operations a cell where the 4-point (stiffness) and 11-point
+// (loads) quadrature took 13,000, every lane works (one entry for 32 cells at a time,
+// table indices warp-uniform, per-cell quantities in shared memory by
+// [quantity][cell]), and a warp's 32 blocks are scattered as one run of
+// 32 x 9 values, so that a request covers 9 neighbouring values of a block
+// (3 sectors) instead of one value of 32 blocks (32 sectors).  15.3 -> 1.4 ms
+// on 331,776 cells (the operations alone: 1.1 ms at the measured FP64 rate);
+// the whole assembly 18.0 -> 4.1 ms.
+constexpr int P2_WARPS = 8, P2_CELLS = 32;
 
-// P2: one warp per cell.  Lane 0 computes the geometry; the 4x10 gradient
-// table goes to shared memory; lanes then take the 100 (a,b) blocks.
+struct P2Tile {
+  double B[10][9][32];             // P1 blocks, k <= l, row-major
+  double G[4][3][32];              // gradients of the barycentric coordinates
+  double f[10][3][32];             // nodal body force
+  double mu[5][32];                // int (T_h - T_ref) lambda_k / |K|, then int (T_h - T_ref) / |K|
+  double vol[32];
+  double out[P2_WARPS][32][9];     // a warp's 32 blocks on their way out
+  int slot[P2_WARPS][32];
+  int v[10][32];
+  unsigned char dm[10][32], ok[32];
+};
+
 __global__ void __launch_bounds__(P2_WARPS * 32) assemble_p2_kernel(AsmArgs A) {
-  __shared__ double sg[P2_WARPS][4][10][3];  // basis gradients at the 4 stiffness points
-  __shared__ double sgeo[P2_WARPS][4][3];
-  __shared__ double svol[P2_WARPS];
-  __shared__ double sq[P2_WARPS][11][4];     // per load point: T_h - T_ref, f_h
-  __shared__ int sv[P2_WARPS][10];
+  extern __shared__ __align__(16) unsigned char p2_smem[];
+  P2Tile& S = *reinterpret_cast<P2Tile*>(p2_smem);
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c = blockIdx.x * P2_WARPS + wid;
-  if (c >= A.n_cells) return;
-  if (lane < 10) sv[wid][lane] = A.cells[10 * (size_t)c + lane];
-  __syncwarp();
-  int ok = 1;
-  if (lane == 0) {
-    double g[4][3], vol;
-    ok = tet_geometry(A.coords, sv[wid], g, vol) ? 1 : 0;
-    for (int k = 0; k < 4; ++k)
-      for (int d = 0; d < 3; ++d) sgeo[wid][k][d] = g[k][d];
-    svol[wid] = vol;
+  const long long c0 = (long long)blockIdx.x * P2_CELLS;
+  const int c = (int)min(c0 + lane, (long long)A.n_cells - 1);  // idle lanes repeat the last cell, unscattered
+  for (int t = threadIdx.x; t < 320; t += P2_WARPS * 32) {
+    const int cl = t / 10;
+    S.v[t - cl * 10][cl] = A.cells[min(c0 + cl, (long long)A.n_cells - 1) * 10 + (t - cl * 10)];
   }
-  ok = __shfl_sync(0xffffffffu, ok, 0);
-  if (!ok) {
-    if (lane == 0) atomicExch(A.bad_cell, 1);
-    return;
-  }
-  __syncwarp();
-  double g[4][3];
-  for (int k = 0; k < 4; ++k)
-    for (int d = 0; d < 3; ++d) g[k][d] = sgeo[wid][k][d];
-  const double vol = svol[wid];
-  for (int t = lane; t < 40; t += 32) {
-    int q = t / 10, a = t % 10;
-    double gr[3];
-    p2_grad(a, c_q4[q], g, gr);
-    for (int d = 0; d < 3; ++d) sg[wid][q][a][d] = gr[d];
-  }
+  __syncthreads();
   const int m = A.mat[c];
   double lam, mu;
   lame(A.props[3 * m], A.props[3 * m + 1], lam, mu);
   const double alpha = A.props[3 * m + 2];
-  // load values at the 11 load points, one lane each
-  const bool loads = A.T || A.body;
-  if (loads && lane < 11) {
-    const double* l = c_k11[lane];
-    double Th = 0.0, fh[3] = {0, 0, 0};
-    for (int ci = 0; ci < 10; ++ci) {
-      const double ph = p2_phi(ci, l);
-      const int nc = sv[wid][ci];
-      if (A.T) Th += ph * A.T[nc];
-      if (A.body)
-        for (int d = 0; d < 3; ++d) fh[d] += ph * A.body[3 * (size_t)nc + d];
-    }
-    sq[wid][lane][0] = A.T ? Th - A.T_ref : 0.0;
-    for (int d = 0; d < 3; ++d) sq[wid][lane][1 + d] = fh[d];
-  }
-  __syncwarp();
-  // stiffness, 4-point rule: K_ab = sum_q w (lam g_a g_b^T + mu g_b g_a^T + mu (g_a . g_b) I)
-  // for the 55 pairs a <= b, with the gradients pre-scaled by w lam and w mu;
-  // K_ba = K_ab^T is scattered for b > a (FP64 is GB300's scarce pipe)
-  const double wl = 0.25 * vol * lam, wm = 0.25 * vol * mu;
-  for (int pidx = lane; pidx < 55; pidx += 32) {
-    int a = 0, r = pidx;
-    while (r >= 10 - a) {
-      r -= 10 - a;
-      ++a;
-    }
-    const int b = a + r;
-    const int na = sv[wid][a], nb = sv[wid][b];
-    const bool ab = !A.dmask[na] && block_needed(A, nb);
-    const bool ba = b != a && !A.dmask[nb] && block_needed(A, na);
-    if (!ab && !ba) continue;
-    double k[9];
+  if (wid == 0) {
+    int v[4];
+    for (int a = 0; a < 4; ++a) v[a] = S.v[a][lane];
+    double g[4][3], vol;
+    const bool good = tet_geometry(A.coords, v, g, vol);
+    if (!good) atomicExch(A.bad_cell, 1);
+    S.ok[lane] = good && c0 + lane < A.n_cells;
+    if (good) {
+      S.vol[lane] = vol;
 #pragma unroll
-    for (int e = 0; e < 9; ++e) k[e] = 0.0;
+      for (int k = 0; k < 4; ++k)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const double* ga = sg[wid][q][a];
-      const double* gb = sg[wid][q][b];
-      const double gb0 = gb[0], gb1 = gb[1], gb2 = gb[2];
-      const double lga[3] = {wl * ga[0], wl * ga[1], wl * ga[2]};
-      const double mga[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
-      const double gbv[3] = {gb0, gb1, gb2};
-      const double mgg = mga[0] * gb0 + mga[1] * gb1 + mga[2] * gb2;
-#pragma unroll
-      for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-        for (int jj = 0; jj < 3; ++jj)
-          k[3 * ii + jj] += fma(lga[ii], gbv[jj], mga[jj] * gbv[ii]) + (ii == jj ? mgg : 0.0);
+        for (int d = 0; d < 3; ++d) S.G[k][d][lane] = g[k][d];
     }
-    if (ab) scatter_block(A, c, a, b, na, nb, k);
-    if (ba) {
-      const double kt[9] = {k[0], k[3], k[6], k[1], k[4], k[7], k[2], k[5], k[8]};
-      scatter_block(A, c, b, a, nb, na, kt);
-    }
-  }
-  // loads, Keast 11-point rule: lane 3a + d sums component d of node a over the points
-  if (loads && lane < 30) {
-    const int a = lane / 3, d = lane % 3, na = sv[wid][a];
-    if (!A.dmask[na]) {
-      const double kT = (3.0 * lam + 2.0 * mu) * alpha;
-      double f = 0.0;
-      for (int q = 0; q < 11; ++q) {
-        const double* l = c_k11[q];
-        const double wq = l[4] * vol;
-        double gr[3];
-        p2_grad(a, l, g, gr);
-        if (A.T) f += wq * kT * sq[wid][q][0] * gr[d];
-        if (A.body) f += wq * p2_phi(a, l) * sq[wid][q][1 + d];
+  } else if (wid == 1) {
+    double sum = 0.0, mk[4] = {0.0, 0.0, 0.0, 0.0};
+    if (A.T)
+#pragma unroll
+      for (int a = 0; a < 10; ++a) {
+        const double t = A.T[S.v[a][lane]] - A.T_ref;
+        sum = fma(a < 4 ? -0.05 : 0.2, t, sum);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mk[k] = fma(p2_moment(a, k), t, mk[k]);
       }
-      if (A.cf) A.cf[((size_t)c * 10 + a) * 3 + d] = f;
-      else atomicAdd(&A.rhs[3 * (size_t)na + d], f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) S.mu[k][lane] = mk[k];
+    S.mu[4][lane] = sum;
+  } else {
+    for (int a = wid - 2; a < 10; a += P2_WARPS - 2) {
+      const int n = S.v[a][lane];
+      S.dm[a][lane] = A.dmask[n];
+      if (A.body)
+        for (int d = 0; d < 3; ++d) S.f[a][d][lane] = A.body[3 * (size_t)n + d];
     }
   }
+  __syncthreads();
+  const double vol = S.vol[lane];
+  const bool ok = S.ok[lane] != 0;
+  // the loads alone need no stiffness unless a prescribed displacement is lifted
+  const bool stiffness = !A.loads_only || A.ud != nullptr;
+  if (stiffness) {
+    for (int p = wid; p < 10; p += P2_WARPS) {
+      const int k = p < 4 ? 0 : (p < 7 ? 1 : (p < 9 ? 2 : 3));
+      const int l = p - (k * 4 - k * (k - 1) / 2) + k;
+      double gk[3], gl[3], lg[3], mg[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        gk[d] = S.G[k][d][lane];
+        gl[d] = S.G[l][d][lane];
+        lg[d] = lam * vol * gk[d];
+        mg[d] = mu * vol * gk[d];
+      }
+      const double mgg = mg[0] * gl[0] + mg[1] * gl[1] + mg[2] * gl[2];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          S.B[p][3 * i + j][lane] = i == j ? fma(lg[i] + mg[i], gl[i], mgg) : fma(lg[i], gl[j], mg[j] * gl[i]);
+    }
+    __syncthreads();
+  }
+  if (stiffness)
+    for (int pidx = wid; pidx < 55; pidx += P2_WARPS) {
+      int a = 0, r = pidx;
+      while (r >= 10 - a) {
+        r -= 10 - a;
+        ++a;
+      }
+      const int b = a + r;
+      const int na = S.v[a][lane], nb = S.v[b][lane];
+      const bool da = S.dm[a][lane] != 0, db = S.dm[b][lane] != 0;
+      const bool ab = ok && !da && (!A.loads_only || (db && A.ud));
+      const bool ba = ok && b != a && !db && (!A.loads_only || (da && A.ud));
+      double k[9];
+#pragma unroll
+      for (int e = 0; e < 9; ++e) k[e] = 0.0;
+      auto add = [&](double w, int p, int q) {  // k += w B_pq
+        const int lo = p < q ? p : q, hi = p < q ? q : p;
+        const double(*B)[32] = S.B[lo * 4 - lo * (lo - 1) / 2 + (hi - lo)];
+        if (p <= q) {
+#pragma unroll
+          for (int e = 0; e < 9; ++e) k[e] = fma(w, B[e][lane], k[e]);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 9; ++e) k[e] = fma(w, B[(e % 3) * 3 + e / 3][lane], k[e]);
+        }
+      };
+      if (b < 4) {
+        add(a == b ? 0.6 : -0.2, a, b);
+      } else {
+        const int br = c_edge[b - 4][0], bs = c_edge[b - 4][1];
+        if (a < 4) {
+          add(a == bs ? 0.6 : -0.2, a, br);
+          add(a == br ? 0.6 : -0.2, a, bs);
+        } else {
+          const int ap = c_edge[a - 4][0], aq = c_edge[a - 4][1];
+          add(aq == bs ? 1.6 : 0.8, ap, br);
+          add(aq == br ? 1.6 : 0.8, ap, bs);
+          add(ap == bs ? 1.6 : 0.8, aq, br);
+          add(ap == br ? 1.6 : 0.8, aq, bs);
+        }
+      }
+      // out: the block to (a, b), then its transpose to (b, a)
+      double* out = S.out[wid][0];
+      int* slot = S.slot[wid];
+#pragma unroll 1
+      for (int side = 0; side < (a == b ? 1 : 2); ++side) {
+        int s = -1;
+        if (side == 0) {
+          if (ab) s = block_slot(A, c, a, b, na, nb, db, k);
+#pragma unroll
+          for (int e = 0; e < 9; ++e) out[lane * 9 + e] = k[e];
+        } else {
+          const double kt[9] = {k[0], k[3], k[6], k[1], k[4], k[7], k[2], k[5], k[8]};
+          if (ba) s = block_slot(A, c, b, a, nb, na, da, kt);
+#pragma unroll
+          for (int e = 0; e < 9; ++e) out[lane * 9 + e] = kt[e];
+        }
+        slot[lane] = s;
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+          const int idx = q * 32 + lane, cl = idx / 9;
+          if (slot[cl] >= 0) atomicAdd(A.vals + (size_t)slot[cl] * 9 + (idx - cl * 9), out[idx]);
+        }
+        __syncwarp();
+      }
+    }
+  // loads: f_a = kT vol int (T_h - T_ref) grad phi_a + vol int f_h phi_a
+  if (A.T || A.body) {
+    const double kT = (3.0 * lam + 2.0 * mu) * alpha * vol;
+    for (int a = wid; a < 10; a += P2_WARPS) {
+      if (!ok || S.dm[a][lane]) continue;
+      double f[3] = {0.0, 0.0, 0.0};
+      if (A.T) {
+        if (a < 4) {
+          const double w = kT * (4.0 * S.mu[a][lane] - S.mu[4][lane]);
+          for (int d = 0; d < 3; ++d) f[d] = w * S.G[a][d][lane];
+        } else {
+          const int p = c_edge[a - 4][0], q = c_edge[a - 4][1];
+          const double wp = 4.0 * kT * S.mu[q][lane], wq = 4.0 * kT * S.mu[p][lane];
+          for (int d = 0; d < 3; ++d) f[d] = fma(wp, S.G[p][d][lane], wq * S.G[q][d][lane]);
+        }
+      }
+      if (A.body) {
+        double s[3] = {0.0, 0.0, 0.0};
+        for (int b = 0; b < 10; ++b) {
+          const double w = p2_mass(a, b);
+#pragma unroll
+          for (int d = 0; d < 3; ++d) s[d] = fma(w, S.f[b][d][lane], s[d]);
+        }
+        for (int d = 0; d < 3; ++d) f[d] = fma(vol, s[d], f[d]);
+      }
+      for (int d = 0; d < 3; ++d) {
+        if (A.cf) A.cf[((size_t)c * 10 + a) * 3 + d] = f[d];
+        else atomicAdd(&A.rhs[3 * (size_t)S.v[a][lane] + d], f[d]);
+      }
+    }
+  }
+}
+
+void launch_p2(const AsmArgs& args, cudaStream_t s) {
+  TAM_CUDA(cudaFuncSetAttribute(assemble_p2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(P2Tile)));
+  assemble_p2_kernel<<<grid_for(args.n_cells, P2_CELLS), P2_WARPS * 32, sizeof(P2Tile), s>>>(args);
 }
 
 // ---------------------------------------------------------------------------
@@ -772,7 +863,7 @@ tam_matrix_s* assemble_elasticity(int n_nodes, const double* coords, int n_cells
       if (npc == 4)
         assemble_p1_kernel<<<grid_for(n_cells, 128), 128, 0, s>>>(args);
       else
-        assemble_p2_kernel<<<grid_for(n_cells, P2_WARPS), P2_WARPS * 32, 0, s>>>(args);
+        launch_p2(args, s);
       TAM_LAUNCH_CHECK();
     }
     if (det) gather_assembly(args, n_nodes, npc, cells, inc_ptr.p, inc.p, dmask, A.vals.p, rhs, T || body, s);
@@ -849,7 +940,7 @@ void assemble_loads(tam_matrix_s* K, const double* coords, int n_cells, int npc,
     if (npc == 4)
       assemble_p1_kernel<<<grid_for(n_cells, 128), 128, 0, s>>>(args);
     else
-      assemble_p2_kernel<<<grid_for(n_cells, P2_WARPS), P2_WARPS * 32, 0, s>>>(args);
+      launch_p2(args, s);
     TAM_LAUNCH_CHECK();
   }
   if (det) gather_assembly(args, n_nodes, npc, cells, inc_ptr.p, inc.p, K->dmask.p, nullptr, rhs, T || body, s);
