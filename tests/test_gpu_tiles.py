@@ -75,3 +75,33 @@ def test_elastic_p2_cell_tiles(n_cells, deterministic):
     assert sparse_rel(bsr_to_csr(*tam.tam_matrix_export_bsr(K), n_cols_blocks=n), Ko) <= 1e-12
     for f in (rhs, load):
         assert np.abs(f.cpu().numpy().ravel() - fo).max() <= 1e-12 * np.abs(fo).max()
+
+
+@pytest.mark.parametrize("n", [1, 31, 63, 65, 2 ** 17 + 1])
+@pytest.mark.parametrize("width,depth,offset", [(3, 1, 0), (33, 2, 0), (64, 3, 1), (96, 1, 0), (128, 3, 0), (128, 4, 1)])
+def test_network_row_and_column_tiles(n, width, depth, offset):
+    """FP32 forward pass and gradient at the edges of the 64- and 32-row tiles, of a piece of 2^17 rows, and for
+    every column tile (widths 3 to 128, rows that start off a 16-byte boundary when offset is 1), against the FP64
+    oracle: sums of at most 128 products in FP32 (forward 1e-5), and over the rows besides (gradient 1e-4)."""
+    tam = need_gpu()
+    net = tam.Mlp(8, width, depth, 3, seed=5)
+    shapes = omlp.layer_shapes(8, width, depth, 3)
+    rng = np.random.default_rng(n)
+    shift, scale = rng.standard_normal(8).astype(np.float32) * 0.1, (1.0 + rng.random(8)).astype(np.float32)
+    out_scale = np.array([0.5, 2.0, 1.5], np.float32)
+    net.set_normalization(shift, scale, out_scale)
+    theta = net.get_params().astype(np.float64)
+    flat = torch.from_numpy(rng.standard_normal(8 * n + offset).astype(np.float32)).cuda()
+    X = flat[offset:].view(n, 8)
+    Y = torch.from_numpy(rng.standard_normal((n, 3)).astype(np.float32)).cuda()
+    args = (shift.astype(np.float64), scale.astype(np.float64), out_scale.astype(np.float64))
+    ref, _ = omlp.forward(theta, shapes, X.cpu().numpy().astype(np.float64), *args)
+    got = net.forward(X).cpu().numpy()
+    assert np.abs(got - ref).max() <= 1e-5 * np.abs(ref).max() + 1e-6
+    if n < 2 ** 17:
+        loss_o, g_o = omlp.loss_and_grad(theta, shapes, X.cpu().numpy().astype(np.float64),
+                                         Y.cpu().numpy().astype(np.float64), *args)
+        for _ in range(2):  # the second call reuses the workspace
+            loss, g = net.loss_grad(X, Y)
+            assert abs(loss - loss_o) <= 1e-5 * loss_o
+            assert np.linalg.norm(g - g_o) <= 1e-4 * np.linalg.norm(g_o)
