@@ -534,120 +534,204 @@ __global__ void smooth_prolongator_kernel(const int* __restrict__ rp, const int*
 // ---------------------------------------------------------------------------
 // Coarsest level: dense Gauss-Jordan inverse (SPD, no pivoting)
 // ---------------------------------------------------------------------------
+// The coarsest operator in dense form, warp per block row (its values are one run), leading dimension ld.
 __global__ void bsr_to_dense_kernel(const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ v,
-                                    int n, int bs, double* __restrict__ D, int N) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+                                    int n, int bs, double* __restrict__ D, int ld) {
+  const int i = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;
-  for (int p = rp[i]; p < rp[i + 1]; ++p) {
-    int j = ci[p];
-    for (int r = 0; r < bs; ++r)
-      for (int c = 0; c < bs; ++c) D[(size_t)(i * bs + r) * N + j * bs + c] = v[(size_t)p * bs * bs + r * bs + c];
+  const int bb = bs * bs, p0 = rp[i], len = (rp[i + 1] - p0) * bb;
+  for (int e = lane; e < len; e += 32) {
+    const int p = e / bb, q = e - p * bb, r = q / bs;
+    D[(size_t)(i * bs + r) * ld + ci[p0 + p] * bs + (q - r * bs)] = v[(size_t)p0 * bb + e];
   }
 }
 
-__global__ void dense_inactive_kernel(double* __restrict__ D, int N, unsigned char* __restrict__ inactive) {
+// Rows without entries (dropped near-nullspace columns, and the padding rows
+// N .. ld): unit diagonal; flagged when they belong to the operator.
+__global__ void dense_inactive_kernel(double* __restrict__ D, int N, int ld, unsigned char* __restrict__ inactive) {
   int i = blockIdx.x;
   __shared__ int nz;
   if (threadIdx.x == 0) nz = 0;
   __syncthreads();
   for (int j = threadIdx.x; j < N; j += blockDim.x)
-    if (D[(size_t)i * N + j] != 0.0) nz = 1;
+    if (D[(size_t)i * ld + j] != 0.0) nz = 1;
   __syncthreads();
   if (threadIdx.x == 0) {
-    inactive[i] = nz ? 0 : 1;
-    if (!nz) D[(size_t)i * N + i] = 1.0;
+    if (i < N) inactive[i] = nz ? 0 : 1;
+    if (!nz) D[(size_t)i * ld + i] = 1.0;
   }
 }
 
 // In-place Gauss-Jordan inversion of an SPD matrix (no pivoting needed),
-// blocked by panels K = [k0, k0 + b) of GJB columns.  With A = [A_KK A_KJ;
-// A_IK A_IJ], eliminating K gives [A_KK^-1, A_KK^-1 A_KJ; -A_IK A_KK^-1,
-// A_IJ - A_IK A_KK^-1 A_KJ], the state the unblocked method reaches after b
-// pivots (D_kj /= p, D_ik = -D_ik / p, D_kk = 1 / p).  Per panel:
-//   1. block 0 inverts D_KK in shared memory by unblocked Gauss-Jordan (its
-//      pivots are the unblocked method's: positive for an SPD matrix);
-//   2. the new row panel D_KK^-1 D_KJ goes to rpan (GJB x N, a thread per
-//      element) and the column panel D_IK is saved (cpan, N x GJB);
-//   3. D_IJ -= cpan rpan, D_IK = -cpan D_KK^-1, and rpan is copied to D_KJ.
-// Three grid-wide barriers per panel instead of two per pivot (the barriers,
-// not the N^3 multiply-adds, dominated: 624 of them on a 312-DOF level).
-constexpr int GJB = 32;
+// blocked by panels K of GJB columns; ld a multiple of GJB (padded with a unit
+// diagonal).  With D = [D_KK D_KJ; D_IK D_IJ] and P = D_KK^-1, eliminating K
+// gives [P, P D_KJ; -D_IK P, D_IJ - D_IK P D_KJ], the state the unblocked
+// method reaches after GJB pivots.  Per panel:
+//   1. the row panel P D_KJ goes to rpan (GJB x ld), the column panel D_IK to
+//      cpan (ld x GJB);
+//   2. D_IJ -= cpan rpan, the new column and row panels; block 0 takes the
+//      next diagonal tile alone, updates it and inverts it (serial: GJB pivots
+//      of one division and one barrier each) while the other blocks update
+//      the rest, so the next panel starts with its P known.
+// Two grid-wide barriers per panel (three, and FP64 products with two global
+// loads each, before: the unit cube's 3,993-DOF solve, whose coarsest level
+// this inverts, 12.2 -> 5.0 ms in all).  Bound by the FP64 pipe (N^3 or, for SYM,
+// N^3 / 2 multiply-adds at 2 per cycle and SM) once N is large, by the GJB
+// dependent pivots (about 9 us a panel) and the barriers below N ~ 500.
+// SYM: a symmetric matrix; only tiles on or below the diagonal are kept.  An
+// eliminated (done) index and one that is not differ in sign: D_ij = -D_ji
+// when exactly one of i, j is done, D_ij = D_ji otherwise.
+constexpr int GJB = 32, GJ_COLS = 16, GJ_THREADS = 256;
 
-__global__ void __launch_bounds__(256) gj_coop_kernel(double* __restrict__ D, int N, double* __restrict__ cpan,
-                                                      double* __restrict__ rpan, int* __restrict__ bad) {
+// The SPD tile src (leading dimension ld) inverted by one block into P [GJB x
+// GJB] (global): thread (r, g) keeps the elements (r, 4 g .. 4 g + 3) in
+// registers; the owners of the next pivot's row, column and reciprocal publish
+// them before the one barrier of a pivot.
+__device__ void gj_invert_tile(const double* __restrict__ src, int ld, double* __restrict__ P, int* __restrict__ bad) {
+  __shared__ double srow[2][GJB], scol[2][GJB], sinv[2];
+  const int r = threadIdx.x >> 3, c0 = (threadIdx.x & 7) * 4;
+  double e[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) e[j] = src[(size_t)r * ld + c0 + j];
+  auto publish = [&](int k) {  // row k, column k and 1 / pivot for the step of pivot k
+    const int b = k & 1;
+    if (r == k)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) srow[b][c0 + j] = e[j];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (c0 + j == k) {
+        scol[b][r] = e[j];
+        if (r == k) {
+          if (!(e[j] > 0.0)) *bad = 1;
+          sinv[b] = 1.0 / e[j];
+        }
+      }
+  };
+  publish(0);
+  for (int k = 0; k < GJB; ++k) {
+    __syncthreads();
+    const int b = k & 1;
+    const double inv = sinv[b], ci = scol[b][r] * inv;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = c0 + j;
+      if (r == k) e[j] = c == k ? inv : e[j] * inv;
+      else if (c == k) e[j] = -ci;
+      else e[j] = fma(-ci, srow[b][c], e[j]);
+    }
+    if (k + 1 < GJB) publish(k + 1);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) P[r * GJB + c0 + j] = e[j];
+  __syncthreads();
+}
+
+template <bool SYM>
+__global__ void __launch_bounds__(GJ_THREADS)
+gj_coop_kernel(double* __restrict__ D, int ld, double* __restrict__ cpan, double* __restrict__ rpan,
+               double* __restrict__ P, int* __restrict__ bad) {
   cg::grid_group grid = cg::this_grid();
-  __shared__ double sd[GJB][GJB + 1];  // the diagonal block (step 1), then its inverse (steps 2-3)
-  __shared__ double ck[GJB];
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nth = gridDim.x * blockDim.x;
-  for (int k0 = 0; k0 < N; k0 += GJB) {
-    const int b = min(GJB, N - k0);
-    if (blockIdx.x == 0) {  // 1.
-      for (int e = threadIdx.x; e < b * b; e += blockDim.x) sd[e / b][e % b] = D[(size_t)(k0 + e / b) * N + k0 + e % b];
+  __shared__ double sp[GJB][GJB + 1];     // P of this panel
+  __shared__ double sa[GJB][GJB + 1];     // a tile's row factors
+  __shared__ double sb[GJB][GJ_COLS + 1]; // a half tile's column factors
+  const int t = ld / GJB;                 // tiles per side
+  const int r = threadIdx.x / GJ_COLS, c = threadIdx.x % GJ_COLS;  // elements (r, c) and (r + 16, c) of a half tile
+  const int first = gridDim.x > 1 ? 1 : 0;
+  if (blockIdx.x == 0) gj_invert_tile(D, ld, P, bad);
+  grid.sync();
+  for (int K = 0; K < t; ++K) {
+    const int k0 = K * GJB;
+    for (int e = threadIdx.x; e < GJB * GJB; e += GJ_THREADS) sp[e / GJB][e % GJB] = P[e];
+    __syncthreads();
+    // 1. the panels, 8 columns (rows) of a tile at a time
+    for (int item = blockIdx.x; item < t * 4; item += gridDim.x) {
+      const int J = item >> 2, q0 = J * GJB + (item & 3) * 8;
+      if (J == K) continue;
+      // D_KJ's 8 columns into sa[k][0..7], D_JK's 8 rows to cpan
+      {
+        const int k = threadIdx.x >> 3, q = threadIdx.x & 7;
+        const double row = (SYM && J > K) ? D[(size_t)(q0 + q) * ld + k0 + k] : D[(size_t)(k0 + k) * ld + q0 + q];
+        sa[k][q] = row;
+        cpan[(size_t)(q0 + q) * GJB + k] = SYM ? (J > K ? row : -row) : D[(size_t)(q0 + q) * ld + k0 + k];
+      }
       __syncthreads();
-      for (int k = 0; k < b; ++k) {
-        const double p = sd[k][k];
-        if (threadIdx.x == 0 && !(p > 0.0)) *bad = 1;
-        const double inv = 1.0 / p;
-        if (threadIdx.x < b) ck[threadIdx.x] = sd[threadIdx.x][k];
-        __syncthreads();
-        if (threadIdx.x < b && threadIdx.x != k) sd[k][threadIdx.x] *= inv;
-        __syncthreads();
-        for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-          const int i = e / b, j = e % b;
-          if (i == k) {
-            if (j == k) sd[k][k] = inv;
-            continue;
-          }
-          if (j == k) sd[i][k] = -ck[i] * inv;
-          else sd[i][j] -= ck[i] * sd[k][j];
+      {
+        const int i = threadIdx.x >> 3, q = threadIdx.x & 7;
+        double v = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < GJB; ++k) v = fma(sp[i][k], sa[k][q], v);
+        rpan[(size_t)i * ld + q0 + q] = v;
+      }
+      __syncthreads();
+    }
+    grid.sync();
+    // 2. half tiles (I, J): the rest, the new column panel (J = K) and row panel (I = K)
+    auto half_tile = [&](int I, int J, int h) {
+      const int i0 = I * GJB, j0 = J * GJB + h * GJ_COLS;
+      double* __restrict__ out = D + (size_t)(i0 + r) * ld + j0 + c;
+      if (I == K) {
+        out[0] = rpan[(size_t)r * ld + j0 + c];
+        out[(size_t)GJ_COLS * ld] = rpan[(size_t)(r + GJ_COLS) * ld + j0 + c];
+        return;
+      }
+      for (int e = threadIdx.x; e < GJB * GJB; e += GJ_THREADS) sa[e / GJB][e % GJB] = cpan[(size_t)i0 * GJB + e];
+      for (int e = threadIdx.x; e < GJB * GJ_COLS; e += GJ_THREADS) {
+        const int k = e / GJ_COLS, j = e % GJ_COLS;
+        sb[k][j] = J == K ? sp[k][h * GJ_COLS + j] : rpan[(size_t)k * ld + j0 + j];
+      }
+      __syncthreads();
+      double v0 = J == K ? 0.0 : out[0], v1 = J == K ? 0.0 : out[(size_t)GJ_COLS * ld];
+#pragma unroll 8
+      for (int k = 0; k < GJB; ++k) {
+        const double x = sb[k][c];
+        v0 = fma(-sa[r][k], x, v0);
+        v1 = fma(-sa[r + GJ_COLS][k], x, v1);
+      }
+      out[0] = v0;
+      out[(size_t)GJ_COLS * ld] = v1;
+      __syncthreads();
+    };
+    if ((int)blockIdx.x >= first) {
+      // items by row of tiles: SYM keeps J <= I
+      const int stride = gridDim.x - first;
+      int item = blockIdx.x - first;
+      for (int I = 0; I < t; ++I) {
+        const int cnt = 2 * (SYM ? I + 1 : t);
+        for (; item < cnt; item += stride) {
+          const int J = item >> 1;
+          if (J == K && I == K) continue;
+          if (first && I == K + 1 && J == K + 1) continue;  // block 0's
+          half_tile(I, J, item & 1);
+        }
+        item -= cnt;
+      }
+    }
+    if (blockIdx.x == 0) {
+      for (int e = threadIdx.x; e < GJB * GJB; e += GJ_THREADS)
+        D[(size_t)(k0 + e / GJB) * ld + k0 + e % GJB] = sp[e / GJB][e % GJB];
+      if (K + 1 < t) {
+        if (first) {
+          half_tile(K + 1, K + 1, 0);
+          half_tile(K + 1, K + 1, 1);
         }
         __syncthreads();
+        gj_invert_tile(D + (size_t)(k0 + GJB) * ld + k0 + GJB, ld, P, bad);
       }
-      for (int e = threadIdx.x; e < b * b; e += blockDim.x) D[(size_t)(k0 + e / b) * N + k0 + e % b] = sd[e / b][e % b];
-    }
-    grid.sync();
-    for (int e = threadIdx.x; e < b * b; e += blockDim.x) sd[e / b][e % b] = D[(size_t)(k0 + e / b) * N + k0 + e % b];
-    __syncthreads();
-    // 2. new row panel (a thread per element, columns outside K) and the
-    // saved column panel
-    for (int e = tid; e < b * (N - b); e += nth) {
-      const int r = e / (N - b), jj = e % (N - b), j = jj < k0 ? jj : jj + b;
-      double v = 0.0;
-      for (int t = 0; t < b; ++t) v = fma(sd[r][t], D[(size_t)(k0 + t) * N + j], v);
-      rpan[(size_t)r * N + j] = v;
-    }
-    for (int e = tid; e < (N - b) * b; e += nth) {
-      const int ii = e / b, c = e % b, i = ii < k0 ? ii : ii + b;
-      cpan[(size_t)i * GJB + c] = D[(size_t)i * N + k0 + c];
-    }
-    grid.sync();
-    // 3. the rest and the column panel (a thread per element of the rows outside K)
-    for (int e = tid; e < (N - b) * N; e += nth) {
-      const int ii = e / N, j = e % N, i = ii < k0 ? ii : ii + b;
-      const double* __restrict__ ci = cpan + (size_t)i * GJB;
-      double v = 0.0;
-      if (j >= k0 && j < k0 + b) {
-        for (int t = 0; t < b; ++t) v = fma(ci[t], sd[t][j - k0], v);
-        D[(size_t)i * N + j] = -v;
-      } else {
-        for (int t = 0; t < b; ++t) v = fma(ci[t], rpan[(size_t)t * N + j], v);
-        D[(size_t)i * N + j] -= v;
-      }
-    }
-    for (int e = tid; e < b * (N - b); e += nth) {
-      const int r = e / (N - b), jj = e % (N - b), j = jj < k0 ? jj : jj + b;
-      D[(size_t)(k0 + r) * N + j] = rpan[(size_t)r * N + j];
     }
     grid.sync();
   }
 }
 
-__global__ void dense_zero_inactive_kernel(double* __restrict__ D, int N, const unsigned char* __restrict__ inactive) {
+// The inverse out of the padded working matrix: rows and columns of inactive
+// unknowns zero; sym: tiles above the diagonal from below it.
+__global__ void dense_out_kernel(const double* __restrict__ W, int ld, int N, const unsigned char* __restrict__ inactive,
+                                 int sym, double* __restrict__ out) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   int i = blockIdx.y;
   if (j >= N) return;
-  if (inactive[i] || inactive[j]) D[(size_t)i * N + j] = 0.0;
+  const bool mirror = sym && j / GJB > i / GJB;
+  out[(size_t)i * N + j] = (inactive[i] || inactive[j]) ? 0.0 : (mirror ? W[(size_t)j * ld + i] : W[(size_t)i * ld + j]);
 }
 
 }  // namespace
@@ -869,39 +953,37 @@ static void tentative(Level& L, const double* B, double droptol, DBuf<double>& B
   (void)droptol;
 }
 
-static void coarse_inverse(tam_amg_s* H, const Level& L, cudaStream_t s) {
-  const int N = L.n_rows * L.bs;
+// sym: the operator is symmetric (K, and every Galerkin product).
+static void coarse_inverse(tam_amg_s* H, const Level& L, bool sym, cudaStream_t s) {
+  const int N = L.n_rows * L.bs, ld = (N + GJB - 1) / GJB * GJB;
   TAM_CHECK(N <= 12000, TAM_ERR_UNSUPPORTED, "amg_setup: coarsest level too large for the dense solve");
   H->n_coarse = N;
   H->coarse_inv = DBuf<double>((size_t)N * N, s);
-  H->coarse_inv.zero();
+  DBuf<double> W((size_t)ld * ld, s);
+  W.zero();
   const Bsr& A = *L.A;
-  bsr_to_dense_kernel<<<grid_for(L.n_rows, TPB), TPB, 0, s>>>(A.row_ptr.p, A.col_idx.p, A.vals.p, L.n_rows, L.bs,
-                                                              H->coarse_inv.p, N);
+  bsr_to_dense_kernel<<<grid_for((long long)L.n_rows * 32, TPB), TPB, 0, s>>>(A.row_ptr.p, A.col_idx.p, A.vals.p,
+                                                                              L.n_rows, L.bs, W.p, ld);
   TAM_LAUNCH_CHECK();
   DBuf<unsigned char> inactive(N, s);
-  dense_inactive_kernel<<<N, 128, 0, s>>>(H->coarse_inv.p, N, inactive.p);
+  dense_inactive_kernel<<<ld, 128, 0, s>>>(W.p, N, ld, inactive.p);
   TAM_LAUNCH_CHECK();
-  DBuf<double> colk((size_t)N * GJB, s), rowk((size_t)N * GJB, s);
+  DBuf<double> colk((size_t)ld * GJB, s), rowk((size_t)ld * GJB, s), pinv((size_t)GJB * GJB, s);
   DBuf<int> bad(1, s);
   bad.zero();
-  dim3 ug(grid_for(N, TPB), N);
   // all panels in one cooperative launch (grid-wide barriers between the
-  // three steps of a panel) instead of 3N / GJB kernel launches
-  int dev = 0, n_sm = 0, per_sm = 0;
-  TAM_CUDA(cudaGetDevice(&dev));
-  TAM_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  TAM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gj_coop_kernel, TPB, 0));
+  // steps of a panel), one block per SM
+  const void* kern = sym ? (const void*)gj_coop_kernel<true> : (const void*)gj_coop_kernel<false>;
+  int per_sm = 0;
+  TAM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GJ_THREADS, 0));
   TAM_CHECK(per_sm >= 1, TAM_ERR_INTERNAL, "amg_setup: Gauss-Jordan kernel cannot be resident");
-  double* dp = H->coarse_inv.p;
-  double* cp = colk.p;
-  double* rp = rowk.p;
+  double *wp = W.p, *cp = colk.p, *rp = rowk.p, *pp = pinv.p;
   int* bp = bad.p;
-  int n_arg = N;
-  void* args[] = {&dp, &n_arg, &cp, &rp, &bp};
-  TAM_CUDA(cudaLaunchCooperativeKernel((const void*)gj_coop_kernel, dim3(n_sm), dim3(TPB), args, 0, s));
+  int ld_arg = ld;
+  void* args[] = {&wp, &ld_arg, &cp, &rp, &pp, &bp};
+  TAM_CUDA(cudaLaunchCooperativeKernel(kern, dim3(sm_count()), dim3(GJ_THREADS), args, 0, s));
   TAM_LAUNCH_CHECK();
-  dense_zero_inactive_kernel<<<ug, TPB, 0, s>>>(H->coarse_inv.p, N, inactive.p);
+  dense_out_kernel<<<dim3(grid_for(N, TPB), N), TPB, 0, s>>>(W.p, ld, N, inactive.p, sym ? 1 : 0, H->coarse_inv.p);
   TAM_LAUNCH_CHECK();
   TAM_CHECK(read_back_int(bad.p, s) == 0, TAM_ERR_INTERNAL, "amg_setup: coarsest operator is not positive definite");
 }
@@ -1066,7 +1148,7 @@ tam_amg_s* amg_build(tam_matrix_s* K, const double* coords, const amg_params& pr
         T.mark(0, s);
         side.join(s);  // before the cooperative launch of the coarse inverse
         T.mark(7, s);
-        coarse_inverse(H, L, s);
+        coarse_inverse(H, L, lev > 0 || L.bs == 3, s);
         break;
       }
       DBuf<double> Bc;

@@ -105,3 +105,43 @@ def test_network_row_and_column_tiles(n, width, depth, offset):
             loss, g = net.loss_grad(X, Y)
             assert abs(loss - loss_o) <= 1e-5 * loss_o
             assert np.linalg.norm(g - g_o) <= 1e-4 * np.linalg.norm(g_o)
+
+
+@pytest.mark.parametrize("hexes", [(1, 1, 1), (3, 1, 3), (2, 2, 2), (3, 3, 3), (5, 5, 5), (8, 8, 7)])
+def test_dense_inverse_tiles(hexes):
+    """A K of at most 2,000 unknowns is its own coarsest level, so one V-cycle is K^-1 r: 24 unknowns (less than
+    a 32-wide panel), 96 and 192 (whole panels), 81, 648 and 1,944 (a ragged last one).  FP64 elimination of
+    matrices with condition numbers below 1e6: 1e-9."""
+    tam = need_gpu()
+    nx, ny, nz = hexes
+    coords, cells = meshgen.box_kuhn(nx, ny, nz)
+    n = coords.shape[0]
+    q = meshgen.Problem(name="dense", coords=coords, cells=cells, cell_material=np.zeros(len(cells), np.int32),
+                        mat_props=np.array([[1.0, 0.3, 1e-3]]), T=None, T_ref=0.0, body_force=None,
+                        dirichlet_mask=(coords[:, 0] == 0).astype(np.uint8), u_dirichlet=None)
+    d = tam.problem_to_device(q)
+    K, _ = tam.fem_assemble_elasticity(**d)
+    H = tam.amg_setup(K, d["coords"])
+    assert tam.amg_info(H)["n_levels"] == 1
+    r = np.random.default_rng(1).standard_normal((n, 3))
+    z = tam.amg_vcycle(H, torch.from_numpy(r).cuda()).cpu().numpy().ravel()
+    Ko, _ = fem.assemble_system(q)
+    ref = np.linalg.solve(Ko.toarray(), r.ravel())
+    assert np.linalg.norm(z - ref) <= 1e-9 * np.linalg.norm(ref)
+
+
+def test_dense_inverse_of_a_nonsymmetric_operator():
+    """A heat problem of 125 unknowns (its own coarsest level) whose Jacobian is not symmetric: with the inverse of
+    the whole matrix every Newton step's CG ends at once, and the solution is the oracle's."""
+    tam = need_gpu()
+    pb = meshgen.unit_cube_problem(4)
+    faces = meshgen.boundary_faces(pb.cells)
+    tp = meshgen.ThermalProblem(pb.coords, pb.cells, pb.cell_material, np.array([[1.0, 1.0, 5e-4, 0.05, 2e-3]]), faces,
+                                np.full(len(faces), -1.0), 300.0 + 300.0 * pb.coords[:, 2])
+    d = tam.thermal_to_device(tp)
+    th = tam.Thermal(d["coords"], d["cells"], d["cell_material"], tp.thermal_props, d["faces"])
+    T = torch.full((pb.n_nodes,), 400.0, dtype=torch.float64, device="cuda")
+    st = th.newton(T, beta=d["beta"], T_bc=d["T_bc"], rtol=1e-11, lin_rtol=1e-9, reuse=0)
+    assert st["linear"] <= 2 * st["newton"]
+    To = oth.newton(tp, np.full(pb.n_nodes, 400.0), rtol=1e-11)[0]
+    assert np.abs(T.cpu().numpy() - To).max() <= 1e-8 * np.abs(To).max()
