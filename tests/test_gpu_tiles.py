@@ -145,3 +145,36 @@ def test_dense_inverse_of_a_nonsymmetric_operator():
     assert st["linear"] <= 2 * st["newton"]
     To = oth.newton(tp, np.full(pb.n_nodes, 400.0), rtol=1e-11)[0]
     assert np.abs(T.cpu().numpy() - To).max() <= 1e-8 * np.abs(To).max()
+
+
+@pytest.mark.parametrize("hexes,degree", [((1, 1, 1), 1), ((3, 2, 2), 1), ((4, 3, 3), 2), ((44, 38, 38), 1), ((24, 20, 18), 2)])
+def test_vectors_off_a_16_byte_boundary(hexes, degree):
+    """x, b and y may start anywhere a float64 may: the same bits as from 16-byte aligned copies, for meshes that
+    take the lanes-per-row kernels and ones that take thread-per-row."""
+    tam = need_gpu()
+    pb = meshgen.slab_box_problem(*hexes, degree=degree)
+    d = tam.problem_to_device(pb)
+    before = tam.set_deterministic_assembly(True)
+    try:
+        K, rhs = tam.fem_assemble_elasticity(**d)
+        moved = torch.empty(d["cells"].numel() + 1, dtype=torch.int32, device="cuda")[1:].view(d["cells"].shape)
+        moved.copy_(d["cells"])
+        K2, rhs2 = tam.fem_assemble_elasticity(**dict(d, cells=moved))
+    finally:
+        tam.set_deterministic_assembly(before)
+    assert torch.equal(rhs, rhs2)
+    assert torch.equal(tam.tam_matrix_export_bsr(K)[2], tam.tam_matrix_export_bsr(K2)[2])
+    n = pb.n_nodes
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.randn((n, 3), dtype=torch.float64, device="cuda", generator=g)
+
+    def off(v):
+        w = torch.empty(v.numel() + 1, dtype=torch.float64, device="cuda")[1:].view(v.shape)
+        return w.copy_(v)
+
+    assert torch.equal(tam.tam_matrix_spmv(K, x), tam.tam_matrix_spmv(K, off(x), off(x)))
+    assert tam.tam_matrix_residual_norm(K, rhs, x) == tam.tam_matrix_residual_norm(K, off(rhs), off(x))
+    H = tam.amg_setup(K, d["coords"])
+    assert torch.equal(tam.amg_vcycle(H, x), tam.amg_vcycle(H, off(x), off(x)))
+    if tam.amg_info(H)["n_levels"] > 1:
+        assert torch.equal(tam.amg_smooth(H, rhs, x.clone(), 3), tam.amg_smooth(H, off(rhs), off(x), 3))
