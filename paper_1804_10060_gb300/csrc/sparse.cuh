@@ -1014,6 +1014,100 @@ void spop_apply(const SpOp& op, const double* x, Epi epi, cudaStream_t s) {
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
 
+// The FP32 vectors that SpMVs gather from (iterates, residuals, coarse
+// corrections) keep each node's bs entries in a record of f32_pitch(bs)
+// floats, so that a gather is one 16-byte (bs = 3) or 32-byte (bs = 6) request:
+// a warp's request costs the lines it touches, and a record of 3 or 6 packed
+// floats took 3 or 6 requests to the same lines.
+__host__ __device__ constexpr int f32_pitch(int bs) { return bs == 3 ? 4 : (bs == 6 ? 8 : bs); }
+
+// 32 bytes in one request (p 32-byte aligned)
+__device__ __forceinline__ void load_f32x8(const float* __restrict__ p, float (&v)[8]) {
+  asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+
+template <int BC>
+__device__ __forceinline__ void gather_f32(const float* __restrict__ x, int c, float (&v)[BC]) {
+  if constexpr (BC == 3) {
+    const float4 w = __ldg(reinterpret_cast<const float4*>(x) + c);
+    v[0] = w.x;
+    v[1] = w.y;
+    v[2] = w.z;
+  } else if constexpr (BC == 6) {
+    float w[8];
+    load_f32x8(x + (size_t)c * 8, w);
+#pragma unroll
+    for (int j = 0; j < 6; ++j) v[j] = w[j];
+  } else {
+#pragma unroll
+    for (int j = 0; j < BC; ++j) v[j] = __ldg(x + (size_t)c * BC + j);
+  }
+}
+
+// A node's BR entries of a record vector (whole records: the padding too)
+template <int BR>
+__device__ __forceinline__ void load_record(const float* __restrict__ x, int row, float (&v)[BR]) {
+  constexpr int P = f32_pitch(BR);
+  if constexpr (P % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < P / 4; ++q) {
+      const float4 w = reinterpret_cast<const float4*>(x)[(size_t)row * (P / 4) + q];
+      const float e[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (4 * q + j < BR) v[4 * q + j] = e[j];
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < BR; ++j) v[j] = x[(size_t)row * BR + j];
+  }
+}
+
+template <int BR>
+__device__ __forceinline__ void store_record(float* __restrict__ x, int row, const float (&v)[BR]) {
+  constexpr int P = f32_pitch(BR);
+  if constexpr (P % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < P / 4; ++q) {
+      float e[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) e[j] = 4 * q + j < BR ? v[4 * q + j < BR ? 4 * q + j : 0] : 0.f;
+      reinterpret_cast<float4*>(x)[(size_t)row * (P / 4) + q] = make_float4(e[0], e[1], e[2], e[3]);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < BR; ++j) x[(size_t)row * BR + j] = v[j];
+  }
+}
+
+// CNT consecutive values of a block in the widest loads their alignment
+// allows (blocks start at multiples of CNT values).
+template <int CNT, typename TV>
+__device__ __forceinline__ void block_load_low(const TV* __restrict__ p, TV (&out)[CNT]) {
+  if constexpr (std::is_same<TV, float>::value && CNT % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < CNT / 4; ++i) {
+      const float4 w = __ldg(reinterpret_cast<const float4*>(p) + i);
+      out[4 * i] = w.x;
+      out[4 * i + 1] = w.y;
+      out[4 * i + 2] = w.z;
+      out[4 * i + 3] = w.w;
+    }
+  } else if constexpr (std::is_same<TV, float>::value && CNT % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < CNT / 2; ++i) {
+      const float2 w = __ldg(reinterpret_cast<const float2*>(p) + i);
+      out[2 * i] = w.x;
+      out[2 * i + 1] = w.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < CNT; ++i) out[i] = p[i];
+  }
+}
+
 template <int BR, int BC, typename TV, class Epi>
 __global__ void __launch_bounds__(SPMV_THREADS)
 sell_spmv_f32_kernel(int n_slices, const int* __restrict__ slice_ptr, const int* __restrict__ cols,
@@ -1037,8 +1131,7 @@ sell_spmv_f32_kernel(int n_slices, const int* __restrict__ slice_ptr, const int*
       for (int e = 0; e < BR * BC; ++e) vv[e] = vp[e * 32];
       const int c = __ldg(cp);
       float xv[BC];
-#pragma unroll
-      for (int j = 0; j < BC; ++j) xv[j] = __ldg(x + (size_t)c * BC + j);
+      gather_f32<BC>(x, c, xv);
 #pragma unroll
       for (int r = 0; r < BR; ++r)
 #pragma unroll
@@ -1066,12 +1159,10 @@ bsr_vector_f32_kernel(int n_rows, const int* __restrict__ rp, const int* __restr
     for (int p = rp[row] + sub; p < pe; p += LPR) {
       const TV* __restrict__ vb = v + (size_t)p * BR * BC;
       TV vv[BR * BC];  // the block's values first, then the gather
-#pragma unroll
-      for (int e = 0; e < BR * BC; ++e) vv[e] = vb[e];
+      block_load_low<BR * BC>(vb, vv);
       const int c = ci[p];
       float xv[BC];
-#pragma unroll
-      for (int j = 0; j < BC; ++j) xv[j] = __ldg(x + (size_t)c * BC + j);
+      gather_f32<BC>(x, c, xv);
 #pragma unroll
       for (int r = 0; r < BR; ++r)
 #pragma unroll

@@ -13,6 +13,7 @@
 // move half or less of the bytes.  A preconditioner only has to be a fixed
 // SPD-like operator, so its rounding error costs at most a few iterations.
 #include <algorithm>
+#include <type_traits>
 
 #include "handles.cuh"
 
@@ -24,20 +25,27 @@ constexpr int TPB = 256;
 template <typename T>
 __device__ __forceinline__ float f32(T v) { return (float)v; }
 
-template <typename TB>
+// x: records of f32_pitch(BS) floats per node; the other vectors packed
+template <int BS, typename TB>
 __global__ void cheb_first_zero_f32_kernel(const TB* __restrict__ b, const float* __restrict__ dinv,
                                            const float* __restrict__ consts, float* __restrict__ d,
-                                           float* __restrict__ x, long long N, const int* __restrict__ stop) {
+                                           float* __restrict__ x, int n_rows, const int* __restrict__ stop) {
   if (stop && *stop) return;
   const float cr = consts[3];
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    float di = cr * dinv[i] * f32(b[i]);
-    d[i] = di;
-    x[i] = di;
+  for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n_rows; row += gridDim.x * blockDim.x) {
+    float v[BS];
+#pragma unroll
+    for (int r = 0; r < BS; ++r) {
+      const size_t i = (size_t)row * BS + r;
+      v[r] = cr * dinv[i] * f32(b[i]);
+      d[i] = v[r];
+    }
+    store_record<BS>(x, row, v);
   }
 }
 
-// One Chebyshev step fused into the FP32 SpMV of x.
+// One Chebyshev step fused into the FP32 SpMV of x (records; xn: records in
+// FP32, packed in FP64 -- the V-cycle's result on level 0).
 template <int BR, typename TB, typename TO>
 struct EpiChebF {
   const TB* b;
@@ -52,17 +60,26 @@ struct EpiChebF {
   __device__ void operator()(int row, const float (&acc)[BR], double*) const {
     if (row >= n_rows) return;
     const float cd = coef[0], cr = coef[1];
+    float v[BR];
+    load_record<BR>(x, row, v);
 #pragma unroll
     for (int r = 0; r < BR; ++r) {
       size_t i = (size_t)row * BR + r;
       float res = dinv[i] * (f32(b[i]) - acc[r]);
       float di = cd != 0.f ? cd * d[i] + cr * res : cr * res;
       d[i] = di;
-      xn[i] = (TO)(x[i] + di);
+      v[r] += di;
+    }
+    if constexpr (std::is_same<TO, float>::value) {
+      store_record<BR>(xn, row, v);
+    } else {
+#pragma unroll
+      for (int r = 0; r < BR; ++r) xn[(size_t)row * BR + r] = (TO)v[r];
     }
   }
 };
 
+// t = b - A x (t: records)
 template <int BR, typename TB>
 struct EpiResidualF {
   const TB* b;
@@ -71,15 +88,15 @@ struct EpiResidualF {
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
   __device__ void operator()(int row, const float (&acc)[BR], double*) const {
-    if (row < n_rows)
+    if (row >= n_rows) return;
+    float v[BR];
 #pragma unroll
-      for (int r = 0; r < BR; ++r) {
-        size_t i = (size_t)row * BR + r;
-        t[i] = f32(b[i]) - acc[r];
-      }
+    for (int r = 0; r < BR; ++r) v[r] = f32(b[(size_t)row * BR + r]) - acc[r];
+    store_record<BR>(t, row, v);
   }
 };
 
+// y = A x (y packed: the next level's right-hand side)
 template <int BR>
 struct EpiStoreF {
   float* y;
@@ -93,6 +110,7 @@ struct EpiStoreF {
   }
 };
 
+// y += A x (y: records)
 template <int BR>
 struct EpiAddF {
   float* y;
@@ -100,16 +118,20 @@ struct EpiAddF {
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
   __device__ void operator()(int row, const float (&acc)[BR], double*) const {
-    if (row < n_rows)
+    if (row >= n_rows) return;
+    float v[BR];
+    load_record<BR>(y, row, v);
 #pragma unroll
-      for (int r = 0; r < BR; ++r) y[(size_t)row * BR + r] += acc[r];
+    for (int r = 0; r < BR; ++r) v[r] += acc[r];
+    store_record<BR>(y, row, v);
   }
 };
 
-// coarsest level: FP64 dense inverse applied to an FP32 (or FP64) vector, FP64 dot products
+// coarsest level: FP64 dense inverse applied to an FP32 (or FP64) vector, FP64
+// dot products; y: records of bs entries in FP32, packed in FP64
 template <typename TI, typename TO>
 __global__ void dense_gemv_mixed_kernel(const double* __restrict__ A, const TI* __restrict__ b, TO* __restrict__ y,
-                                        int N, const int* __restrict__ stop) {
+                                        int N, int bs, const int* __restrict__ stop) {
   if (stop && *stop) return;
   int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= N) return;
@@ -117,7 +139,10 @@ __global__ void dense_gemv_mixed_kernel(const double* __restrict__ A, const TI* 
   double s = 0.0;
   for (int j = lane; j < N; j += 32) s = fma(a[j], (double)b[j], s);
   s = warp_sum(s);
-  if (lane == 0) y[row] = (TO)s;
+  if (lane == 0) {
+    const int i = row / bs;
+    y[std::is_same<TO, float>::value ? i * f32_pitch(bs) + (row - i * bs) : row] = (TO)s;
+  }
 }
 
 __global__ void to_f32_kernel(const double* __restrict__ in, float* __restrict__ out, long long n) {
@@ -167,17 +192,21 @@ void prolong_f(const Level& L, const float* xc, float* x, const int* stop, cudaS
 template <typename TB, typename TO>
 void vcycle_low(tam_amg_s* H, int l, const TB* b, TO* out, const int* stop, cudaStream_t s) {
   Level& L = H->levels[l];
-  const long long N = (long long)L.n_rows * L.bs;
   if (l == (int)H->levels.size() - 1) {
     dense_gemv_mixed_kernel<TB, TO><<<grid_for((long long)H->n_coarse * 32, TPB), TPB, 0, s>>>(
-        H->coarse_inv.p, b, out, H->n_coarse, stop);
+        H->coarse_inv.p, b, out, H->n_coarse, L.bs, stop);
     TAM_LAUNCH_CHECK();
     return;
   }
   const int deg = L.deg;
   float* xa = L.xa32.p;
   float* xb = L.xb32.p;
-  cheb_first_zero_f32_kernel<TB><<<vgrid(N), TPB, 0, s>>>(b, L.dinv32.p, L.consts32.p, L.d32.p, xa, N, stop);
+  if (L.bs == 3)
+    cheb_first_zero_f32_kernel<3, TB><<<vgrid(L.n_rows), TPB, 0, s>>>(b, L.dinv32.p, L.consts32.p, L.d32.p, xa,
+                                                                     L.n_rows, stop);
+  else
+    cheb_first_zero_f32_kernel<6, TB><<<vgrid(L.n_rows), TPB, 0, s>>>(b, L.dinv32.p, L.consts32.p, L.d32.p, xa,
+                                                                     L.n_rows, stop);
   TAM_LAUNCH_CHECK();
   for (int k = 1; k < deg; ++k) {
     cheb_step_f<TB, float>(L, b, xa, xb, k, stop, s);
@@ -217,13 +246,14 @@ void build_low_precision(tam_amg_s* H, cudaStream_t s) {
     L.consts32 = DBuf<float>(nc, s);
     to_f32_kernel<<<1, 32, 0, s>>>(L.consts.p, L.consts32.p, (long long)nc);
     TAM_LAUNCH_CHECK();
+    const size_t NP = (size_t)L.n_rows * f32_pitch(L.bs);  // vectors of records
     L.b32 = DBuf<float>(N, s);
-    L.y32 = DBuf<float>(N, s);
+    L.y32 = DBuf<float>(NP, s);
     if (coarsest) continue;
-    L.xa32 = DBuf<float>(N, s);
-    L.xb32 = DBuf<float>(N, s);
+    L.xa32 = DBuf<float>(NP, s);
+    L.xb32 = DBuf<float>(NP, s);
     L.d32 = DBuf<float>(N, s);
-    L.t32 = DBuf<float>(N, s);
+    L.t32 = DBuf<float>(NP, s);
     if (l == 0 && mode == 2) {
       convert_values_bf16(L.Aop, L.A16v, s);
       L.A16 = SpOpLow<__nv_bfloat16>{L.Aop, L.A16v.p};
