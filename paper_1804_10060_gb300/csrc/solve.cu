@@ -383,8 +383,8 @@ void spmv_outer_pq(tam_amg_s* H, cudaStream_t s) {
   GridReduce gr{H->partials.p, H->ticket.p};
   by_block(H->K->A.br, [&](auto B) {
     constexpr int BR = decltype(B)::value;
-    sell_spmv<BR, BR>(H->K->S, H->p.p, EpiPq<BR>{H->p.p, H->q.p, H->K->n_nodes, gr, H->sc.p}, s,
-                      H->levels[0].Aop.df, /*acc=*/true);
+    sell_spmv<BR, BR, true>(H->K->S, H->p.p, EpiPq<BR>{H->p.p, H->q.p, H->K->n_nodes, gr, H->sc.p}, s,
+                            H->levels[0].Aop.df);
   });
 }
 
@@ -457,7 +457,7 @@ cudaGraphExec_t build_loop_graph(const std::function<void(cudaStream_t)>& enqueu
 void spmv_K(tam_matrix_s* K, const double* x, double* y, cudaStream_t s) {
   by_block(K->A.br, [&](auto B) {
     constexpr int BR = decltype(B)::value;
-    sell_spmv<BR, BR>(K->S, x, EpiStore<BR>{y, K->n_nodes, nullptr}, s, K->df_ok, /*acc=*/true);
+    sell_spmv<BR, BR, true>(K->S, x, EpiStore<BR>{y, K->n_nodes, nullptr}, s, K->df_ok);
   });
 }
 
@@ -510,9 +510,8 @@ int pcg_solve(tam_amg_s* H, const double* b, double* x, double rtol, double atol
   x = H->xs.p;
   by_block(H->K->A.br, [&](auto B) {
     constexpr int BR = decltype(B)::value;
-    sell_spmv<BR, BR>(H->K->S, x, EpiInitResidual<BR>{b, H->r.p, H->K->n_nodes, gr, sc, H->hist.p}, s,
-                      H->levels[0].Aop.df,
-                      /*acc=*/true);
+    sell_spmv<BR, BR, true>(H->K->S, x, EpiInitResidual<BR>{b, H->r.p, H->K->n_nodes, gr, sc, H->hist.p}, s,
+                            H->levels[0].Aop.df);
   });
   precondition(H, H->r.p, H->z.p, &sc->stop, s);
   pcg_rz_kernel<<<vec_grid(N), TPB, 0, s>>>(H->r.p, H->z.p, H->p.p, N, gr, sc, 1);

@@ -286,66 +286,108 @@ __device__ __forceinline__ void by_alignment(const double* x, F&& f) {
 }
 
 
-template <int BR, int BC, class Epi, bool DF, bool ACC = false>
+// S: warps per slice.  With S = 2 the slice's slots alternate between two
+// warps, whose row sums meet in shared memory (each row: even slots, then odd
+// ones).  A row is a serial chain of its slots, and a mesh of a few thousand
+// slices (quadratic cells: 27 slots a row) leaves the chip with one or two
+// waves of long chains; see sell_split.
+template <int BR, int BC, class Epi, bool DF, bool ACC, int S>
 __global__ void __launch_bounds__(SPMV_THREADS)
 sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
+  static_assert(DF || S == 1, "sell_spmv_kernel: FP64 rows are not split");
+  constexpr int SLICES = SPMV_THREADS / 32 / S;  // per block
   __shared__ double sh[32];
+  [[maybe_unused]] __shared__ float2 part[S > 1 ? SLICES : 1][BR][32];
   if (epi.skip()) return;
-  const int pos = blockIdx.x * SPMV_THREADS + threadIdx.x;
-  const int slice = pos >> 5, lane = pos & 31;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, sub = wid % S;
+  const int slice = blockIdx.x * SLICES + wid / S, pos = slice * 32 + lane;
   double acc[BR];
 #pragma unroll
   for (int r = 0; r < BR; ++r) acc[r] = 0.0;
+  [[maybe_unused]] float2 run[BR];
+  if constexpr (DF)
+#pragma unroll
+    for (int r = 0; r < BR; ++r) run[r] = make_float2(0.f, 0.f);
   by_alignment(x, [&](auto al) {
     constexpr bool AL = decltype(al)::value;
-  if (slice < A.n_slices) {
-    const int k0 = A.slice_ptr[slice], k1 = A.slice_ptr[slice + 1];
+    if (slice >= A.n_slices) return;
+    const int k0 = A.slice_ptr[slice] + sub, k1 = A.slice_ptr[slice + 1];
     const int* __restrict__ cp = A.cols + (size_t)k0 * 32 + lane;
     if constexpr (DF) {
       const float2* __restrict__ vp = A.vals_df + (size_t)k0 * 32 * BR * BC + lane;
-      float2 ad[BR], run[BR];
-#pragma unroll
-      for (int r = 0; r < BR; ++r) ad[r] = run[r] = make_float2(0.f, 0.f);
-#pragma unroll 2
-      for (int k = k0; k < k1; ++k) {
-        float2 vv[BR * BC];  // the slot's values first, then the gather
-#pragma unroll
-        for (int e = 0; e < BR * BC; ++e) vv[e] = __ldg(vp + e * 32);
-        const int c = __ldg(cp);
-        double xg[BC];
-        gather_x<BC, AL>(x, c, xg);
+      // one slot's products into the rows' sums.  ACC: the slot's double-float
+      // partial sum (its BC products) is added into the row's running sum with
+      // the accurate double-word addition, so that the low part never carries
+      // more than one slot's rounding: a few 2^-48 of sum_j |A_ij x_j| per row
+      // whatever the row's length (the plain running double-float sum drifts
+      // to ~2^-45 on long P2 rows); FP32 work only (an FP64 sum every two
+      // slots cost 1.5 FP64 adds per row and slot pair on GB300's slow FP64
+      // pipe).
+      auto slot = [&](const float2 (&vv)[BR * BC], const double (&xg)[BC]) {
         float2 xv[BC];
 #pragma unroll
         for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
 #pragma unroll
-        for (int r = 0; r < BR; ++r)
+        for (int r = 0; r < BR; ++r) {
+          if constexpr (ACC) {
+            float2 ad = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int j = 0; j < BC; ++j) {
-            if constexpr (ACC) df_fma4(ad[r], vv[r * BC + j], xv[j]);
-            else df_fma(ad[r], vv[r * BC + j], xv[j]);
-          }
-        if constexpr (ACC) {
-          // ACC: each slot's double-float partial sum (its BC products) is
-          // added into the row's running sum with the accurate double-word
-          // addition, so that the low part never carries more than one
-          // slot's rounding: a few 2^-48 of sum_j |A_ij x_j| per row whatever
-          // the row's length (the plain running double-float sum drifts to
-          // ~2^-45 on long P2 rows); FP32 work only (an FP64 sum every two
-          // slots cost 1.5 FP64 adds per row and slot pair on GB300's slow
-          // FP64 pipe)
+            for (int j = 0; j < BC; ++j) df_fma4(ad, vv[r * BC + j], xv[j]);
+            df_add_accurate(run[r], ad);
+          } else {
 #pragma unroll
-          for (int r = 0; r < BR; ++r) {
-            df_add_accurate(run[r], ad[r]);
-            ad[r] = make_float2(0.f, 0.f);
+            for (int j = 0; j < BC; ++j) df_fma(run[r], vv[r * BC + j], xv[j]);
           }
         }
-        cp += 32;
-        vp += 32 * BR * BC;
-      }
+      };
+      // Columns ahead of their slots: a slot's gather goes out with its values
+      // instead of a memory round trip behind its column (level-0 Chebyshev
+      // step of the 3.26M-DOF box 206 -> 198 us, its accurate product 247 ->
+      // 230 us).
+      if constexpr (BR * BC > 1) {
+        int c0 = k0 < k1 ? __ldg(cp) : 0, c1 = k0 + S < k1 ? __ldg(cp + S * 32) : 0;
+#pragma unroll 2
+        for (int k = k0; k < k1; k += S) {
+          float2 vv[BR * BC];
 #pragma unroll
-      for (int r = 0; r < BR; ++r) {
-        if constexpr (ACC) acc[r] = df_to_double(run[r]);
-        else acc[r] += df_to_double(ad[r]);
+          for (int e = 0; e < BR * BC; ++e) vv[e] = __ldg(vp + e * 32);
+          double xg[BC];
+          gather_x<BC, AL>(x, c0, xg);
+          c0 = c1;
+          if (k + 2 * S < k1) c1 = __ldg(cp + 2 * S * 32);
+          slot(vv, xg);
+          cp += S * 32;
+          vp += S * 32 * BR * BC;
+        }
+      } else {
+        // scalar blocks: four slots a step, so that four gathers and four
+        // values are in flight per thread (thermal Chebyshev step of the
+        // 460k-unknown disc 79 -> 52 us)
+        constexpr int U = 4;
+        int cn[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) cn[u] = k0 + u * S < k1 ? __ldg(cp + u * S * 32) : 0;
+        for (int k = k0; k < k1; k += U * S) {
+          float2 vv[U][1];
+          double xg[U][1];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            vv[u][0] = make_float2(0.f, 0.f);
+            xg[u][0] = 0.0;
+            if (u == 0 || k + u * S < k1) {
+              vv[u][0] = __ldg(vp + u * S * 32);
+              gather_x<1, AL>(x, cn[u], xg[u]);
+            }
+          }
+          cp += U * S * 32;
+          vp += U * S * 32;
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (k + (U + u) * S < k1) cn[u] = __ldg(cp + u * S * 32);
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (u == 0 || k + u * S < k1) slot(vv[u], xg[u]);
+        }
       }
     } else {
       const double* __restrict__ vp = A.vals + (size_t)k0 * 32 * BR * BC + lane;
@@ -362,23 +404,42 @@ sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
         vp += 32 * BR * BC;
       }
     }
-  }
   });
-  epi(sell_row(A.perm, pos, A.n_rows), acc, sh);
+  if constexpr (S > 1) {
+    if (sub == 1)
+#pragma unroll
+      for (int r = 0; r < BR; ++r) part[wid / S][r][lane] = run[r];
+    __syncthreads();
+    if (sub == 0)
+#pragma unroll
+      for (int r = 0; r < BR; ++r) {
+        if constexpr (ACC) df_add_accurate(run[r], part[wid / S][r][lane]);
+        else df_add(run[r], part[wid / S][r][lane]);
+      }
+  }
+  if constexpr (DF)
+#pragma unroll
+    for (int r = 0; r < BR; ++r) acc[r] = df_to_double(run[r]);
+  epi(sub == 0 ? sell_row(A.perm, pos, A.n_rows) : A.n_rows, acc, sh);
 }
 
+// Warps per slice for the double-float and FP32 SELL kernels: two where one
+// would leave fewer than two and a half waves of the 64 warps an SM holds
+// (1.38M-DOF P2 disc, 14,388 slices: FP32 solve 95.0 -> 88.8 ms); the boxes of
+// 30,000 and more slices stay whole.
+inline int sell_split(int n_slices) { return n_slices < 160LL * sm_count() ? 2 : 1; }
+
 // df: use the split copy when the matrix has one (false: plain FP64).
-// acc: the accurate double-float accumulation (outer CG products with K and
+// ACC: the accurate double-float accumulation (outer CG products with K and
 // tam_matrix_spmv; the V-cycle's smoothing SpMVs keep the faster running sum).
-template <int BR, int BC, class Epi>
-void sell_spmv(const Sell& A, const double* x, Epi epi, cudaStream_t s, bool df = true, bool acc = false) {
-  unsigned grid = grid_for((long long)A.n_slices * 32, SPMV_THREADS);
-  if (df && A.vals_df.p && acc)
-    sell_spmv_kernel<BR, BC, Epi, true, true><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
-  else if (df && A.vals_df.p)
-    sell_spmv_kernel<BR, BC, Epi, true><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
-  else
-    sell_spmv_kernel<BR, BC, Epi, false><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
+template <int BR, int BC, bool ACC = false, class Epi>
+void sell_spmv(const Sell& A, const double* x, Epi epi, cudaStream_t s, bool df = true) {
+  const bool use = df && A.vals_df.p;
+  const int split = use ? sell_split(A.n_slices) : 1;
+  const unsigned grid = grid_for((long long)A.n_slices * 32 * split, SPMV_THREADS);
+  if (!use) sell_spmv_kernel<BR, BC, Epi, false, false, 1><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
+  else if (split == 2) sell_spmv_kernel<BR, BC, Epi, true, ACC, 2><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
+  else sell_spmv_kernel<BR, BC, Epi, true, ACC, 1><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
   TAM_LAUNCH_CHECK();
 }
 
@@ -1108,24 +1169,27 @@ __device__ __forceinline__ void block_load_low(const TV* __restrict__ p, TV (&ou
   }
 }
 
-template <int BR, int BC, typename TV, class Epi>
+// S: warps per slice, as in sell_spmv_kernel
+template <int BR, int BC, typename TV, class Epi, int S>
 __global__ void __launch_bounds__(SPMV_THREADS)
 sell_spmv_f32_kernel(int n_slices, const int* __restrict__ slice_ptr, const int* __restrict__ cols,
                      const TV* __restrict__ vals, const float* __restrict__ x, const int* __restrict__ perm,
                      int n_rows, Epi epi) {
+  constexpr int SLICES = SPMV_THREADS / 32 / S;  // per block
   __shared__ double sh[32];
+  [[maybe_unused]] __shared__ float part[S > 1 ? SLICES : 1][BR][32];
   if (epi.skip()) return;
-  const int pos = blockIdx.x * SPMV_THREADS + threadIdx.x;
-  const int slice = pos >> 5, lane = pos & 31;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, sub = wid % S;
+  const int slice = blockIdx.x * SLICES + wid / S, pos = slice * 32 + lane;
   float acc[BR];
 #pragma unroll
   for (int r = 0; r < BR; ++r) acc[r] = 0.f;
   if (slice < n_slices) {
-    const int k0 = slice_ptr[slice], k1 = slice_ptr[slice + 1];
+    const int k0 = slice_ptr[slice] + sub, k1 = slice_ptr[slice + 1];
     const int* __restrict__ cp = cols + (size_t)k0 * 32 + lane;
     const TV* __restrict__ vp = vals + (size_t)k0 * 32 * BR * BC + lane;
 #pragma unroll 4
-    for (int k = k0; k < k1; ++k) {
+    for (int k = k0; k < k1; k += S) {
       TV vv[BR * BC];  // the slot's values first, then the gather
 #pragma unroll
       for (int e = 0; e < BR * BC; ++e) vv[e] = vp[e * 32];
@@ -1136,11 +1200,20 @@ sell_spmv_f32_kernel(int n_slices, const int* __restrict__ slice_ptr, const int*
       for (int r = 0; r < BR; ++r)
 #pragma unroll
         for (int j = 0; j < BC; ++j) acc[r] = fmaf(to_f32(vv[r * BC + j]), xv[j], acc[r]);
-      cp += 32;
-      vp += 32 * BR * BC;
+      cp += S * 32;
+      vp += S * 32 * BR * BC;
     }
   }
-  epi(sell_row(perm, pos, n_rows), acc, sh);
+  if constexpr (S > 1) {
+    if (sub == 1)
+#pragma unroll
+      for (int r = 0; r < BR; ++r) part[wid / S][r][lane] = acc[r];
+    __syncthreads();
+    if (sub == 0)
+#pragma unroll
+      for (int r = 0; r < BR; ++r) acc[r] += part[wid / S][r][lane];
+  }
+  epi(sub == 0 ? sell_row(perm, pos, n_rows) : n_rows, acc, sh);
 }
 
 template <int BR, int BC, int LPR, typename TV, class Epi>
@@ -1189,8 +1262,14 @@ void spop_apply_f32(const SpOpLow<TV>& o, const float* x, Epi epi, cudaStream_t 
   const unsigned g = spop_grid(o.op);
   if (o.op.lpr == 0) {
     const Sell& S = *o.op.S;
-    sell_spmv_f32_kernel<BR, BC, TV, Epi><<<g, SPMV_THREADS, 0, s>>>(S.n_slices, S.slice_ptr.p, S.cols.p, o.vals, x,
-                                                                     S.perm.p, S.n_rows, epi);
+    const int split = sell_split(S.n_slices);
+    const unsigned grid = grid_for((long long)S.n_slices * 32 * split, SPMV_THREADS);
+    if (split == 2)
+      sell_spmv_f32_kernel<BR, BC, TV, Epi, 2><<<grid, SPMV_THREADS, 0, s>>>(S.n_slices, S.slice_ptr.p, S.cols.p, o.vals,
+                                                                             x, S.perm.p, S.n_rows, epi);
+    else
+      sell_spmv_f32_kernel<BR, BC, TV, Epi, 1><<<grid, SPMV_THREADS, 0, s>>>(S.n_slices, S.slice_ptr.p, S.cols.p, o.vals,
+                                                                             x, S.perm.p, S.n_rows, epi);
   } else {
     const Bsr& B = *o.op.B;
     switch (o.op.lpr) {
