@@ -22,7 +22,7 @@ namespace tam {
 namespace {
 
 constexpr int TPB = 256;
-constexpr int TMAX = 8;    // RHS per thread, compile-time register tile
+constexpr int TMAX = 8;    // most RHS per thread
 constexpr int MPMAX = 16;  // RHS per system
 constexpr int MT_MIN_THREADS = 64, MT_MAX_THREADS = 256;  // CTA sizes the autotuner tries
 enum { S_RHO = 0, S_ALPHA, S_BETA, S_RR, S_TOL2, S_BB, S_DONE, S_ITER, S_SCALE, S_COUNT };
@@ -33,41 +33,89 @@ __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((lon
 unsigned vgrid(long long n) { return stride_grid(n, TPB, 8); }
 
 // -------------------------------------------------------------------------
-// layout conversion
+// Vector kernels.  mp is 8 or 16, the vectors are [entry][mp], and a grid's
+// stride is a multiple of 16, so a thread keeps one right-hand side j for the
+// whole kernel: its scalars are read once, every access is coalesced, and it
+// carries one partial sum.
 // -------------------------------------------------------------------------
+__host__ __device__ __forceinline__ int rhs_shift(int mp) { return mp == 8 ? 3 : 4; }
+
 __global__ void interleave_kernel(const double* __restrict__ src, double* __restrict__ dst, int m, int mp, long long n3) {
+  const int sh = rhs_shift(mp);
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x) {
-    const long long i = e / mp;
-    const int j = (int)(e % mp);
-    dst[e] = j < m ? src[(size_t)j * n3 + i] : 0.0;
+    const int j = (int)(e & (mp - 1));
+    dst[e] = j < m ? src[(size_t)j * n3 + (e >> sh)] : 0.0;
   }
 }
 
 // back to one vector per RHS, undoing each RHS's power-of-two scaling
 __global__ void deinterleave_kernel(const double* __restrict__ src, double* __restrict__ dst, int m, int mp,
                                     long long n3, const double* __restrict__ sc) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * m; e += (long long)gridDim.x * blockDim.x) {
-    const int j = (int)(e / n3);
-    const long long i = e % n3;
-    dst[e] = src[i * mp + j] * pow2((int)sc[S_SCALE * mp + j]);
+  const int sh = rhs_shift(mp);
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x) {
+    const int j = (int)(e & (mp - 1));
+    if (j < m) dst[(size_t)j * n3 + (e >> sh)] = src[e] * pow2((int)sc[S_SCALE * mp + j]);
   }
 }
 
 // b and x of every RHS into the solve's scaling (b 2^-e_j, x 2^-e_j; see mstart_kernel)
 __global__ void mscale_in_kernel(double* __restrict__ b, double* __restrict__ x, long long n3, int mp,
                                  const double* __restrict__ sc) {
+  const double f = pow2(-(int)sc[S_SCALE * mp + (int)(threadIdx.x & (mp - 1))]);
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x) {
-    const double f = pow2(-(int)sc[S_SCALE * mp + (int)(e % mp)]);
     b[e] *= f;
     x[e] *= f;
   }
 }
 
-// -------------------------------------------------------------------------
-// per-RHS reductions: every thread holds up to MPMAX partial sums
-// -------------------------------------------------------------------------
-__device__ bool reduce_rhs(GridReduce gr, double (&v)[MPMAX], double (&tot)[MPMAX], double* sh) {
-  return grid_reduce<MPMAX>(gr, v, tot, sh);
+// Grid-wide sums of the blocks' partial sums of nv quantities (part[k] in
+// shared memory, k < nv), in block order: true in the last block to finish,
+// with the totals in tot[k].  The ticket is reset for the next launch.
+__device__ __forceinline__ bool grid_totals(GridReduce gr, const double* part, int nv, double* tot) {
+  __shared__ bool s_last;
+  if (threadIdx.x < nv) {
+    gr.partials[(size_t)blockIdx.x * nv + threadIdx.x] = part[threadIdx.x];
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(gr.ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  // nv divides 32: lane l sums quantity l % nv over every 32 / nv-th block of its warp's share
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, k = lane & (nv - 1);
+  __shared__ double sh[8][16];
+  double acc = 0.0;
+  for (unsigned b = (threadIdx.x) / nv; b < gridDim.x; b += blockDim.x / nv)
+    acc += ((volatile double*)gr.partials)[(size_t)b * nv + k];
+  for (int o = 16; o >= nv; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane < nv) sh[wid][lane] = acc;
+  __syncthreads();
+  if (threadIdx.x < nv) {
+    double t = 0.0;
+    for (int w = 0; w < nw; ++w) t += sh[w][threadIdx.x];
+    tot[threadIdx.x] = t;
+  }
+  if (threadIdx.x == 0) *gr.ticket = 0u;
+  __syncthreads();
+  return true;
+}
+
+// Per-RHS sum of every thread's v (the RHS of thread t: t % mp), see grid_totals
+__device__ __forceinline__ bool reduce_rhs(GridReduce gr, double v, int mp, double* tot) {
+  __shared__ double sh[TPB / 32][MPMAX];
+  __shared__ double part[MPMAX];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int o = 16; o >= mp; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane < mp) sh[wid][lane] = v;
+  __syncthreads();
+  if (threadIdx.x < mp) {
+    double t = 0.0;
+    for (int w = 0; w < TPB / 32; ++w) t += sh[w][threadIdx.x];
+    part[threadIdx.x] = t;
+  }
+  __syncthreads();
+  return grid_totals(gr, part, mp, tot);
 }
 
 // Per RHS: ||b||^2, and the power of two e_j the solve divides b_j and x_j by
@@ -77,19 +125,11 @@ __device__ bool reduce_rhs(GridReduce gr, double (&v)[MPMAX], double (&tot)[MPMA
 __global__ void mstart_kernel(const double* __restrict__ b, long long n3, int m, int mp, double rtol, double atol,
                               int max_iter, int half_exp, GridReduce gr, double* __restrict__ sc,
                               int* __restrict__ flags) {
-  __shared__ double sh[32];
-  double acc[MPMAX];
-#pragma unroll
-  for (int j = 0; j < MPMAX; ++j) acc[j] = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x)
-#pragma unroll
-    for (int j = 0; j < MPMAX; ++j)
-      if (j < mp) {
-        const double v = b[i * mp + j];
-        acc[j] += v * v;
-      }
-  double tot[MPMAX];
-  if (reduce_rhs(gr, acc, tot, sh) && threadIdx.x == 0) {
+  __shared__ double tot[MPMAX];
+  double acc = 0.0;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x)
+    acc += b[e] * b[e];
+  if (reduce_rhs(gr, acc, mp, tot) && threadIdx.x == 0) {
     for (int j = 0; j < mp; ++j) {
       int e = 0;
       if (tot[j] > 0.0 && isfinite(tot[j])) {
@@ -123,24 +163,19 @@ __global__ void mcheck_kernel(const double* __restrict__ sc, int mp, int* __rest
 __global__ void mupdate_kernel(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
                                const double* __restrict__ q, long long n3, int mp, GridReduce gr,
                                double* __restrict__ sc, int* __restrict__ flags) {
-  __shared__ double sh[32];
+  __shared__ double tot[MPMAX];
   if (flags[0]) return;
-  double acc[MPMAX];
-#pragma unroll
-  for (int j = 0; j < MPMAX; ++j) acc[j] = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x)
-#pragma unroll
-    for (int j = 0; j < MPMAX; ++j)
-      if (j < mp && sc[S_DONE * mp + j] == 0.0) {
-        const double a = sc[S_ALPHA * mp + j];
-        const long long k = i * mp + j;
-        x[k] += a * p[k];
-        const double rk = r[k] - a * q[k];
-        r[k] = rk;
-        acc[j] += rk * rk;
-      }
-  double tot[MPMAX];
-  if (reduce_rhs(gr, acc, tot, sh) && threadIdx.x == 0) {
+  const int jt = (int)(threadIdx.x & (mp - 1));
+  const double a = sc[S_ALPHA * mp + jt];
+  double acc = 0.0;
+  if (sc[S_DONE * mp + jt] == 0.0)
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x) {
+      x[e] += a * p[e];
+      const double rk = r[e] - a * q[e];
+      r[e] = rk;
+      acc += rk * rk;
+    }
+  if (reduce_rhs(gr, acc, mp, tot) && threadIdx.x == 0) {
     bool all = true;
     for (int j = 0; j < mp; ++j) {
       if (sc[S_DONE * mp + j] == 0.0) {
@@ -159,21 +194,15 @@ __global__ void mupdate_kernel(double* __restrict__ x, double* __restrict__ r, c
 __global__ void mrz_kernel(const double* __restrict__ r, const double* __restrict__ z, double* __restrict__ p,
                            long long n3, int mp, int first, GridReduce gr, double* __restrict__ sc,
                            int* __restrict__ flags) {
-  __shared__ double sh[32];
+  __shared__ double tot[MPMAX];
   if (flags[0]) return;
-  double acc[MPMAX];
-#pragma unroll
-  for (int j = 0; j < MPMAX; ++j) acc[j] = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x)
-#pragma unroll
-    for (int j = 0; j < MPMAX; ++j)
-      if (j < mp) {
-        const long long k = i * mp + j;
-        acc[j] += r[k] * z[k];
-        if (first) p[k] = z[k];
-      }
-  double tot[MPMAX];
-  if (reduce_rhs(gr, acc, tot, sh) && threadIdx.x == 0) {
+  double acc = 0.0;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x) {
+    const double zk = z[e];
+    acc += r[e] * zk;
+    if (first) p[e] = zk;
+  }
+  if (reduce_rhs(gr, acc, mp, tot) && threadIdx.x == 0) {
     for (int j = 0; j < mp; ++j) {
       if (sc[S_DONE * mp + j] != 0.0) continue;
       const double rz = tot[j];
@@ -189,39 +218,141 @@ __global__ void mrz_kernel(const double* __restrict__ r, const double* __restric
 __global__ void mdir_kernel(const double* __restrict__ z, double* __restrict__ p, long long n3, int mp,
                             const double* __restrict__ sc, const int* __restrict__ flags) {
   if (flags[0]) return;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x) {
-    const int j = (int)(e % mp);
-    if (sc[S_DONE * mp + j] == 0.0) p[e] = z[e] + sc[S_BETA * mp + j] * p[e];
+  const int j = (int)(threadIdx.x & (mp - 1));
+  if (sc[S_DONE * mp + j] != 0.0) return;
+  const double beta = sc[S_BETA * mp + j];
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n3 * mp; e += (long long)gridDim.x * blockDim.x)
+    p[e] = z[e] + beta * p[e];
+}
+
+// TM consecutive right-hand sides in the widest requests (TM * sizeof(T)-aligned)
+template <int TM, typename T>
+__device__ __forceinline__ void load_rhs(const T* __restrict__ p, T (&v)[TM]) {
+  if constexpr (std::is_same<T, float>::value && TM == 8) {
+    load_f32x8(p, v);
+  } else if constexpr (std::is_same<T, float>::value && TM == 4) {
+    const float4 w = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = w.x;
+    v[1] = w.y;
+    v[2] = w.z;
+    v[3] = w.w;
+  } else if constexpr (std::is_same<T, float>::value && TM == 2) {
+    const float2 w = __ldg(reinterpret_cast<const float2*>(p));
+    v[0] = w.x;
+    v[1] = w.y;
+  } else if constexpr (std::is_same<T, double>::value && TM % 2 == 0) {
+#pragma unroll
+    for (int k = 0; k < TM / 2; ++k) {
+      const double2 w = __ldg(reinterpret_cast<const double2*>(p) + k);
+      v[2 * k] = w.x;
+      v[2 * k + 1] = w.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < TM; ++k) v[k] = __ldg(p + k);
   }
 }
 
+// the same through plain loads (a vector this kernel also writes)
+template <int TM, typename T>
+__device__ __forceinline__ void read_rhs(const T* p, T (&v)[TM]) {
+  constexpr int W = 16 / sizeof(T);
+  if constexpr (TM % W == 0) {
+    using V = typename std::conditional<std::is_same<T, float>::value, float4, double2>::type;
+#pragma unroll
+    for (int k = 0; k < TM / W; ++k) {
+      const V w = reinterpret_cast<const V*>(p)[k];
+      if constexpr (W == 4) {
+        v[4 * k] = w.x;
+        v[4 * k + 1] = w.y;
+        v[4 * k + 2] = w.z;
+        v[4 * k + 3] = w.w;
+      } else {
+        v[2 * k] = w.x;
+        v[2 * k + 1] = w.y;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < TM; ++k) v[k] = p[k];
+  }
+}
+
+template <int TM, typename T>
+__device__ __forceinline__ void write_rhs(T* p, const T (&v)[TM]) {
+  constexpr int W = 16 / sizeof(T);
+  if constexpr (TM % W == 0) {
+#pragma unroll
+    for (int k = 0; k < TM / W; ++k) {
+      if constexpr (W == 4) reinterpret_cast<float4*>(p)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+      else reinterpret_cast<double2*>(p)[k] = make_double2(v[2 * k], v[2 * k + 1]);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < TM; ++k) p[k] = v[k];
+  }
+}
+
+// Block-wide sums of TM quantities, then grid_totals.  A warp folds the
+// quantities into its lanes (half of them leave at each of the first steps):
+// TM - 1 + log2(32 / TM) FP64 additions instead of 5 TM.
+template <int TM>
+__device__ __forceinline__ bool reduce_tile(GridReduce gr, double (&v)[TM], double* tot) {
+  __shared__ double sh[MT_MAX_THREADS / 32][TM];
+  __shared__ double part[TM];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int o = 16, at = 0;  // at: the quantity this lane holds
+#pragma unroll
+  for (int h = TM / 2; h > 0; h >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double mine = up ? v[k + h] : v[k], other = up ? v[k] : v[k + h];
+      v[k] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+    }
+    at += up ? h : 0;
+    o >>= 1;
+  }
+  double s = v[0];
+  for (; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((lane & (32 / TM - 1)) == 0) sh[wid][at] = s;
+  __syncthreads();
+  if (threadIdx.x < TM) {
+    double t = 0.0;
+    for (int w = 0; w < nw; ++w) t += sh[w][threadIdx.x];
+    part[threadIdx.x] = t;
+  }
+  __syncthreads();
+  return grid_totals(gr, part, TM, tot);
+}
+
 // -------------------------------------------------------------------------
-// SpMM with K (SELL-32, thread per row, RHS chunk per blockIdx.y)
+// SpMM with K (SELL-32, thread per row and TM right-hand sides, the chunk of
+// right-hand sides per blockIdx.y)
 // -------------------------------------------------------------------------
-// DF: double-float products on K's split values (each value feeds tm
+// DF: double-float products on K's split values (each value feeds TM
 // right-hand sides, so the FP64 version is far past GB300's FP64 rate).
-template <class Epi, bool DF>
+template <class Epi, bool DF, int TM>
 __global__ void __launch_bounds__(MT_MAX_THREADS)
-kspmm_kernel(SellView A, const double* __restrict__ x, int mp, int tm, Epi epi) {
-  __shared__ double sh[32];
+kspmm_kernel(SellView A, const double* __restrict__ x, int mp, Epi epi) {
   if (epi.skip()) return;
   const int pos = blockIdx.x * blockDim.x + threadIdx.x;
   const int slice = pos >> 5, lane = pos & 31;
   const int row = sell_row(A.perm, pos, A.n_rows);
-  const int j0 = blockIdx.y * tm;
-  double acc[3][TMAX];
+  const int j0 = blockIdx.y * TM;
+  double acc[3][TM];
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
-    for (int k = 0; k < TMAX; ++k) acc[r][k] = 0.0;
-  if constexpr (DF) {
-    if (slice < A.n_slices) {
-      float2 ad[3][TMAX];
+    for (int k = 0; k < TM; ++k) acc[r][k] = 0.0;
+  if (slice < A.n_slices) {
+    const int k0 = A.slice_ptr[slice], k1 = A.slice_ptr[slice + 1];
+    if constexpr (DF) {
+      float2 ad[3][TM];
 #pragma unroll
       for (int r = 0; r < 3; ++r)
 #pragma unroll
-        for (int k = 0; k < TMAX; ++k) ad[r][k] = make_float2(0.f, 0.f);
-      const int k0 = A.slice_ptr[slice], k1 = A.slice_ptr[slice + 1];
+        for (int k = 0; k < TM; ++k) ad[r][k] = make_float2(0.f, 0.f);
       for (int s = k0; s < k1; ++s) {
         const int c = __ldg(A.cols + (size_t)s * 32 + lane);
         const float2* __restrict__ vp = A.vals_df + (size_t)s * 32 * 9 + lane;
@@ -230,46 +361,40 @@ kspmm_kernel(SellView A, const double* __restrict__ x, int mp, int tm, Epi epi) 
         for (int e = 0; e < 9; ++e) v[e] = __ldg(vp + e * 32);
 #pragma unroll
         for (int jc = 0; jc < 3; ++jc) {
-          const double* xr = x + ((size_t)c * 3 + jc) * mp + j0;
+          double xr[TM];
+          load_rhs<TM>(x + ((size_t)c * 3 + jc) * mp + j0, xr);
 #pragma unroll
-          for (int k = 0; k < TMAX; ++k)
-            if (k < tm) {
-              const float2 xv = split_bits(__ldg(xr + k));
+          for (int k = 0; k < TM; ++k) {
+            const float2 xv = split_bits(xr[k]);
 #pragma unroll
-              for (int r = 0; r < 3; ++r) df_fma(ad[r][k], v[r * 3 + jc], xv);
-            }
+            for (int r = 0; r < 3; ++r) df_fma(ad[r][k], v[r * 3 + jc], xv);
+          }
         }
       }
 #pragma unroll
       for (int r = 0; r < 3; ++r)
 #pragma unroll
-        for (int k = 0; k < TMAX; ++k) acc[r][k] = df_to_double(ad[r][k]);
-    }
-    epi(row, j0, tm, acc, sh);
-    return;
-  }
-  if (slice < A.n_slices) {
-    const int k0 = A.slice_ptr[slice], k1 = A.slice_ptr[slice + 1];
-    for (int s = k0; s < k1; ++s) {
-      const int c = __ldg(A.cols + (size_t)s * 32 + lane);
-      const double* __restrict__ vp = A.vals + (size_t)s * 32 * 9 + lane;
-      double v[9];
+        for (int k = 0; k < TM; ++k) acc[r][k] = df_to_double(ad[r][k]);
+    } else {
+      for (int s = k0; s < k1; ++s) {
+        const int c = __ldg(A.cols + (size_t)s * 32 + lane);
+        const double* __restrict__ vp = A.vals + (size_t)s * 32 * 9 + lane;
+        double v[9];
 #pragma unroll
-      for (int e = 0; e < 9; ++e) v[e] = __ldg(vp + e * 32);
+        for (int e = 0; e < 9; ++e) v[e] = __ldg(vp + e * 32);
 #pragma unroll
-      for (int jc = 0; jc < 3; ++jc) {
-        const double* xr = x + ((size_t)c * 3 + jc) * mp + j0;
+        for (int jc = 0; jc < 3; ++jc) {
+          double xr[TM];
+          load_rhs<TM>(x + ((size_t)c * 3 + jc) * mp + j0, xr);
 #pragma unroll
-        for (int k = 0; k < TMAX; ++k)
-          if (k < tm) {
-            const double xv = __ldg(xr + k);
+          for (int k = 0; k < TM; ++k)
 #pragma unroll
-            for (int r = 0; r < 3; ++r) acc[r][k] = fma(v[r * 3 + jc], xv, acc[r][k]);
-          }
+            for (int r = 0; r < 3; ++r) acc[r][k] = fma(v[r * 3 + jc], xr[k], acc[r][k]);
+        }
       }
     }
   }
-  epi(row, j0, tm, acc, sh);
+  epi(row, j0, acc);
 }
 
 // q = K p, per-RHS p.q -> alpha
@@ -281,24 +406,25 @@ struct EpiPqM {
   double* sc;
   int* flags;
   __device__ bool skip() const { return flags[0]; }
-  __device__ void operator()(int row, int j0, int tm, const double (&acc)[3][TMAX], double* sh) const {
-    double s[TMAX];
+  template <int TM>
+  __device__ void operator()(int row, int j0, const double (&acc)[3][TM]) const {
+    __shared__ double tot[TM];
+    double s[TM];
 #pragma unroll
-    for (int k = 0; k < TMAX; ++k) s[k] = 0.0;
+    for (int k = 0; k < TM; ++k) s[k] = 0.0;
     if (row < n_rows)
 #pragma unroll
-      for (int r = 0; r < 3; ++r)
+      for (int r = 0; r < 3; ++r) {
+        const size_t i = ((size_t)row * 3 + r) * mp + j0;
+        double pv[TM];
+        load_rhs<TM>(p + i, pv);
+        write_rhs<TM>(q + i, acc[r]);
 #pragma unroll
-        for (int k = 0; k < TMAX; ++k)
-          if (k < tm) {
-            const size_t i = ((size_t)row * 3 + r) * mp + j0 + k;
-            q[i] = acc[r][k];
-            s[k] += p[i] * acc[r][k];
-          }
-    GridReduce g{gr.partials + (size_t)blockIdx.y * gridDim.x * TMAX, gr.ticket + blockIdx.y};
-    double tot[TMAX];
-    if (grid_reduce<TMAX>(g, s, tot, sh) && threadIdx.x == 0) {
-      for (int k = 0; k < tm; ++k) {
+        for (int k = 0; k < TM; ++k) s[k] += pv[k] * acc[r][k];
+      }
+    GridReduce g{gr.partials + (size_t)blockIdx.y * gridDim.x * TM, gr.ticket + blockIdx.y};
+    if (reduce_tile<TM>(g, s, tot) && threadIdx.x == 0) {
+      for (int k = 0; k < TM; ++k) {
         const int j = j0 + k;
         if (sc[S_DONE * mp + j] != 0.0) { sc[S_ALPHA * mp + j] = 0.0; continue; }
         const double pq = tot[k];
@@ -320,25 +446,28 @@ struct EpiResInitM {
   double* out;  // if non-null: store ||b - Kx||^2 here instead (final residual)
   int* flags;
   __device__ bool skip() const { return false; }
-  __device__ void operator()(int row, int j0, int tm, const double (&acc)[3][TMAX], double* sh) const {
-    double s[TMAX];
+  template <int TM>
+  __device__ void operator()(int row, int j0, const double (&acc)[3][TM]) const {
+    __shared__ double tot[TM];
+    double s[TM];
 #pragma unroll
-    for (int k = 0; k < TMAX; ++k) s[k] = 0.0;
+    for (int k = 0; k < TM; ++k) s[k] = 0.0;
     if (row < n_rows)
 #pragma unroll
-      for (int rr = 0; rr < 3; ++rr)
+      for (int rr = 0; rr < 3; ++rr) {
+        const size_t i = ((size_t)row * 3 + rr) * mp + j0;
+        double v[TM];
+        load_rhs<TM>(b + i, v);
 #pragma unroll
-        for (int k = 0; k < TMAX; ++k)
-          if (k < tm) {
-            const size_t i = ((size_t)row * 3 + rr) * mp + j0 + k;
-            const double v = b[i] - acc[rr][k];
-            if (r) r[i] = v;
-            s[k] += v * v;
-          }
-    GridReduce g{gr.partials + (size_t)blockIdx.y * gridDim.x * TMAX, gr.ticket + blockIdx.y};
-    double tot[TMAX];
-    if (grid_reduce<TMAX>(g, s, tot, sh) && threadIdx.x == 0) {
-      for (int k = 0; k < tm; ++k) {
+        for (int k = 0; k < TM; ++k) {
+          v[k] -= acc[rr][k];
+          s[k] += v[k] * v[k];
+        }
+        if (r) write_rhs<TM>(r + i, v);
+      }
+    GridReduce g{gr.partials + (size_t)blockIdx.y * gridDim.x * TM, gr.ticket + blockIdx.y};
+    if (reduce_tile<TM>(g, s, tot) && threadIdx.x == 0) {
+      for (int k = 0; k < TM; ++k) {
         const int j = j0 + k;
         if (out) { out[j] = tot[k]; continue; }
         sc[S_RR * mp + j] = tot[k];
@@ -353,45 +482,56 @@ struct EpiStoreKM {
   double* y;
   int n_rows, mp;
   __device__ bool skip() const { return false; }
-  __device__ void operator()(int row, int j0, int tm, const double (&acc)[3][TMAX], double*) const {
+  template <int TM>
+  __device__ void operator()(int row, int j0, const double (&acc)[3][TM]) const {
     if (row < n_rows)
 #pragma unroll
-      for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int k = 0; k < TMAX; ++k)
-          if (k < tm) y[((size_t)row * 3 + r) * mp + j0 + k] = acc[r][k];
+      for (int r = 0; r < 3; ++r) write_rhs<TM>(y + ((size_t)row * 3 + r) * mp + j0, acc[r]);
   }
 };
+
+// f(std::integral_constant<int, TM>()) for the tile's right-hand sides per thread
+template <class F>
+void by_tile(int tm, F&& f) {
+  switch (tm) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
+    default: throw Error(TAM_ERR_INTERNAL, "batch: right-hand sides per thread must be 1, 2, 4 or 8");
+  }
+}
 
 // df: the double-float kernel on K's split values (the hierarchy's level-0
 // choice, amg_params.spmv_fp64); false: plain FP64.
 template <class Epi>
 void kspmm(const Sell& S, const double* x, int mp, const MTile& t, Epi epi, cudaStream_t s, bool df) {
   dim3 g(grid_for((long long)S.n_slices * 32, t.threads), mp / t.tm);
-  if (df && S.vals_df.p)
-    kspmm_kernel<Epi, true><<<g, t.threads, 0, s>>>(view(S), x, mp, t.tm, epi);
-  else
-    kspmm_kernel<Epi, false><<<g, t.threads, 0, s>>>(view(S), x, mp, t.tm, epi);
+  by_tile(t.tm, [&](auto tm) {
+    constexpr int TM = decltype(tm)::value;
+    if (df && S.vals_df.p) kspmm_kernel<Epi, true, TM><<<g, t.threads, 0, s>>>(view(S), x, mp, epi);
+    else kspmm_kernel<Epi, false, TM><<<g, t.threads, 0, s>>>(view(S), x, mp, epi);
+  });
   TAM_LAUNCH_CHECK();
 }
 
 // -------------------------------------------------------------------------
 // FP32 multi-vector SpMM for the V-cycle (SELL or lanes-per-row layouts)
 // -------------------------------------------------------------------------
-template <int BR, int BC, typename TV, class Epi>
+template <int BR, int BC, typename TV, class Epi, int TM>
 __global__ void __launch_bounds__(MT_MAX_THREADS)
 msell_kernel(int n_slices, const int* __restrict__ slice_ptr, const int* __restrict__ cols, const TV* __restrict__ vals,
-             const float* __restrict__ x, int mp, int tm, const int* __restrict__ perm, Epi epi) {
+             const float* __restrict__ x, int mp, const int* __restrict__ perm, Epi epi) {
   if (epi.skip()) return;
   const int pos = blockIdx.x * blockDim.x + threadIdx.x;
   const int slice = pos >> 5, lane = pos & 31;
   const int row = sell_row(perm, pos, epi.n_rows);
-  const int j0 = blockIdx.y * tm;
-  float acc[BR][TMAX];
+  const int j0 = blockIdx.y * TM;
+  float acc[BR][TM];
 #pragma unroll
   for (int r = 0; r < BR; ++r)
 #pragma unroll
-    for (int k = 0; k < TMAX; ++k) acc[r][k] = 0.f;
+    for (int k = 0; k < TM; ++k) acc[r][k] = 0.f;
   if (slice < n_slices) {
     const int k0 = slice_ptr[slice], k1 = slice_ptr[slice + 1];
     for (int s = k0; s < k1; ++s) {
@@ -402,55 +542,49 @@ msell_kernel(int n_slices, const int* __restrict__ slice_ptr, const int* __restr
       const int c = __ldg(cols + (size_t)s * 32 + lane);
 #pragma unroll
       for (int jc = 0; jc < BC; ++jc) {
-        const float* xr = x + ((size_t)c * BC + jc) * mp + j0;
-        float xv[TMAX];
-#pragma unroll
-        for (int k = 0; k < TMAX; ++k) xv[k] = k < tm ? __ldg(xr + k) : 0.f;
+        float xv[TM];
+        load_rhs<TM>(x + ((size_t)c * BC + jc) * mp + j0, xv);
 #pragma unroll
         for (int r = 0; r < BR; ++r) {
           const float a = to_f32(vv[r * BC + jc]);
 #pragma unroll
-          for (int k = 0; k < TMAX; ++k) acc[r][k] = fmaf(a, xv[k], acc[r][k]);
+          for (int k = 0; k < TM; ++k) acc[r][k] = fmaf(a, xv[k], acc[r][k]);
         }
       }
     }
   }
-  if (row < epi.n_rows) epi(row, j0, tm, acc);
+  if (row < epi.n_rows) epi(row, j0, acc);
 }
 
-template <int BR, int BC, typename TV, class Epi>
+template <int BR, int BC, typename TV, class Epi, int TM>
 __global__ void __launch_bounds__(MT_MAX_THREADS)
 mvec_kernel(int n_rows, const int* __restrict__ rp, const int* __restrict__ ci, const TV* __restrict__ v,
-            const float* __restrict__ x, int mp, int tm, int lpr_log2, Epi epi) {
+            const float* __restrict__ x, int mp, int lpr_log2, Epi epi) {
   if (epi.skip()) return;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int lpr = 1 << lpr_log2;
   const int row = t >> lpr_log2, sub = t & (lpr - 1);
-  const int j0 = blockIdx.y * tm;
-  float acc[BR][TMAX];
+  const int j0 = blockIdx.y * TM;
+  float acc[BR][TM];
 #pragma unroll
   for (int r = 0; r < BR; ++r)
 #pragma unroll
-    for (int k = 0; k < TMAX; ++k) acc[r][k] = 0.f;
+    for (int k = 0; k < TM; ++k) acc[r][k] = 0.f;
   if (row < n_rows) {
     const int pe = rp[row + 1];
     for (int p = rp[row] + sub; p < pe; p += lpr) {
-      const TV* __restrict__ vb = v + (size_t)p * BR * BC;
       TV vv[BR * BC];  // the block's values first, then the gathers
-#pragma unroll
-      for (int e = 0; e < BR * BC; ++e) vv[e] = vb[e];
+      block_load_low<BR * BC>(v + (size_t)p * BR * BC, vv);
       const int c = ci[p];
 #pragma unroll
       for (int jc = 0; jc < BC; ++jc) {
-        const float* xr = x + ((size_t)c * BC + jc) * mp + j0;
-        float xv[TMAX];
-#pragma unroll
-        for (int k = 0; k < TMAX; ++k) xv[k] = k < tm ? __ldg(xr + k) : 0.f;
+        float xv[TM];
+        load_rhs<TM>(x + ((size_t)c * BC + jc) * mp + j0, xv);
 #pragma unroll
         for (int r = 0; r < BR; ++r) {
           const float a = to_f32(vv[r * BC + jc]);
 #pragma unroll
-          for (int k = 0; k < TMAX; ++k) acc[r][k] = fmaf(a, xv[k], acc[r][k]);
+          for (int k = 0; k < TM; ++k) acc[r][k] = fmaf(a, xv[k], acc[r][k]);
         }
       }
     }
@@ -459,8 +593,8 @@ mvec_kernel(int n_rows, const int* __restrict__ rp, const int* __restrict__ ci, 
 #pragma unroll
     for (int r = 0; r < BR; ++r)
 #pragma unroll
-      for (int k = 0; k < TMAX; ++k) acc[r][k] += __shfl_xor_sync(0xffffffffu, acc[r][k], o);
-  if (sub == 0 && row < n_rows) epi(row, j0, tm, acc);
+      for (int k = 0; k < TM; ++k) acc[r][k] += __shfl_xor_sync(0xffffffffu, acc[r][k], o);
+  if (sub == 0 && row < n_rows) epi(row, j0, acc);
 }
 
 template <int BR, typename TB, typename TO>
@@ -474,20 +608,28 @@ struct EpiChebMF {
   int n_rows, mp;
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
-  __device__ void operator()(int row, int j0, int tm, const float (&acc)[BR][TMAX]) const {
+  template <int TM>
+  __device__ void operator()(int row, int j0, const float (&acc)[BR][TM]) const {
     const float cd = coef[0], cr = coef[1];
 #pragma unroll
     for (int r = 0; r < BR; ++r) {
       const float dr = dinv[(size_t)row * BR + r];
+      const size_t i = ((size_t)row * BR + r) * mp + j0;
+      TB bv[TM];
+      load_rhs<TM>(b + i, bv);
+      float xv[TM], dv[TM];
+      load_rhs<TM>(x + i, xv);
+      read_rhs<TM>(d + i, dv);
+      TO ov[TM];
 #pragma unroll
-      for (int k = 0; k < TMAX; ++k)
-        if (k < tm) {
-          const size_t i = ((size_t)row * BR + r) * mp + j0 + k;
-          const float res = dr * ((float)b[i] - acc[r][k]);
-          const float di = cd != 0.f ? cd * d[i] + cr * res : cr * res;
-          d[i] = di;
-          xn[i] = (TO)(x[i] + di);
-        }
+      for (int k = 0; k < TM; ++k) {
+        const float res = dr * ((float)bv[k] - acc[r][k]);
+        const float di = cd != 0.f ? cd * dv[k] + cr * res : cr * res;
+        dv[k] = di;
+        ov[k] = (TO)(xv[k] + di);
+      }
+      write_rhs<TM>(d + i, dv);
+      write_rhs<TM>(xn + i, ov);
     }
   }
 };
@@ -499,15 +641,18 @@ struct EpiResMF {
   int n_rows, mp;
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
-  __device__ void operator()(int row, int j0, int tm, const float (&acc)[BR][TMAX]) const {
+  template <int TM>
+  __device__ void operator()(int row, int j0, const float (&acc)[BR][TM]) const {
 #pragma unroll
-    for (int r = 0; r < BR; ++r)
+    for (int r = 0; r < BR; ++r) {
+      const size_t i = ((size_t)row * BR + r) * mp + j0;
+      TB bv[TM];
+      load_rhs<TM>(b + i, bv);
+      float v[TM];
 #pragma unroll
-      for (int k = 0; k < TMAX; ++k)
-        if (k < tm) {
-          const size_t i = ((size_t)row * BR + r) * mp + j0 + k;
-          t[i] = (float)b[i] - acc[r][k];
-        }
+      for (int k = 0; k < TM; ++k) v[k] = (float)bv[k] - acc[r][k];
+      write_rhs<TM>(t + i, v);
+    }
   }
 };
 
@@ -517,15 +662,17 @@ struct EpiPutMF {
   int n_rows, mp;
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
-  __device__ void operator()(int row, int j0, int tm, const float (&acc)[BR][TMAX]) const {
+  template <int TM>
+  __device__ void operator()(int row, int j0, const float (&acc)[BR][TM]) const {
 #pragma unroll
-    for (int r = 0; r < BR; ++r)
+    for (int r = 0; r < BR; ++r) {
+      const size_t i = ((size_t)row * BR + r) * mp + j0;
+      float v[TM];
+      if constexpr (ADD) read_rhs<TM>(y + i, v);
 #pragma unroll
-      for (int k = 0; k < TMAX; ++k)
-        if (k < tm) {
-          const size_t i = ((size_t)row * BR + r) * mp + j0 + k;
-          y[i] = ADD ? y[i] + acc[r][k] : acc[r][k];
-        }
+      for (int k = 0; k < TM; ++k) v[k] = ADD ? v[k] + acc[r][k] : acc[r][k];
+      write_rhs<TM>(y + i, v);
+    }
   }
 };
 
@@ -535,16 +682,20 @@ void mspmm(const SpOpLow<TV>& o, const float* x, int mp, const MTile& t, Epi epi
   if (op.lpr == 0) {
     const Sell& S = *op.S;
     dim3 g(grid_for((long long)S.n_slices * 32, t.threads), mp / t.tm);
-    msell_kernel<BR, BC, TV, Epi><<<g, t.threads, 0, s>>>(S.n_slices, S.slice_ptr.p, S.cols.p, o.vals, x, mp, t.tm,
-                                                          S.perm.p, epi);
+    by_tile(t.tm, [&](auto tm) {
+      msell_kernel<BR, BC, TV, Epi, decltype(tm)::value><<<g, t.threads, 0, s>>>(S.n_slices, S.slice_ptr.p, S.cols.p,
+                                                                                 o.vals, x, mp, S.perm.p, epi);
+    });
   } else {
     const Bsr& B = *op.B;
     const int lpr = t.lpr ? t.lpr : op.lpr;
     int lg = 0;
     while ((1 << lg) < lpr) ++lg;
     dim3 g(grid_for((long long)B.n_rows << lg, t.threads), mp / t.tm);
-    mvec_kernel<BR, BC, TV, Epi><<<g, t.threads, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, mp, t.tm, lg,
-                                                         epi);
+    by_tile(t.tm, [&](auto tm) {
+      mvec_kernel<BR, BC, TV, Epi, decltype(tm)::value><<<g, t.threads, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p,
+                                                                                o.vals, x, mp, lg, epi);
+    });
   }
   TAM_LAUNCH_CHECK();
 }
@@ -555,24 +706,50 @@ __global__ void mfirst_kernel(const TB* __restrict__ b, const float* __restrict_
                               const int* __restrict__ stop) {
   if (stop && *stop) return;
   const float cr = consts[3];
+  const int sh = rhs_shift(mp);
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < N * mp; e += (long long)gridDim.x * blockDim.x) {
-    const float di = cr * dinv[e / mp] * (float)b[e];
+    const float di = cr * dinv[e >> sh] * (float)b[e];
     d[e] = di;
     x[e] = di;
   }
 }
 
+// Y = A^-1 B for 8 right-hand sides a warp: warp per row, the lanes over its
+// columns (a thread per output walked N columns alone, one dependent FP64
+// multiply-add after the other).
 template <typename TI, typename TO>
 __global__ void mcoarse_kernel(const double* __restrict__ A, const TI* __restrict__ b, TO* __restrict__ y, int N, int mp,
                                const int* __restrict__ stop) {
   if (stop && *stop) return;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)N * mp) return;
-  const int i = (int)(t / mp), k = (int)(t % mp);
-  const double* a = A + (size_t)i * N;
-  double s = 0.0;
-  for (int j = 0; j < N; ++j) s = fma(a[j], (double)b[(size_t)j * mp + k], s);
-  y[t] = (TO)s;
+  const int i = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (i >= N) return;
+  const int j0 = blockIdx.y * 8;
+  const double* __restrict__ a = A + (size_t)i * N;
+  double s[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) s[k] = 0.0;
+  for (int j = lane; j < N; j += 32) {
+    const double aj = a[j];
+    TI bv[8];
+    load_rhs<8>(b + (size_t)j * mp + j0, bv);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] = fma(aj, (double)bv[k], s[k]);
+  }
+  // fold the 8 sums into the lanes: lane group (lane >> 2) ends with one of them
+  int at = 0;
+#pragma unroll
+  for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double mine = up ? s[k + h] : s[k], other = up ? s[k] : s[k + h];
+      s[k] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+    }
+    at += up ? h : 0;
+  }
+  s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+  s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+  if ((lane & 3) == 0) y[(size_t)i * mp + j0 + at] = (TO)s[0];
 }
 
 // A x on a level with its FP32 / BF16 values
@@ -621,8 +798,8 @@ void mvcycle(tam_amg_s* H, int l, const TB* b, TO* out, const int* stop, cudaStr
   Level& L = H->levels[l];
   MultiLevel& ML = MS.lv[l];
   if (l == (int)H->levels.size() - 1) {
-    mcoarse_kernel<TB, TO><<<grid_for((long long)H->n_coarse * mp, TPB), TPB, 0, s>>>(H->coarse_inv.p, b, out,
-                                                                                      H->n_coarse, mp, stop);
+    mcoarse_kernel<TB, TO><<<dim3(grid_for((long long)H->n_coarse * 32, TPB), mp / 8), TPB, 0, s>>>(
+        H->coarse_inv.p, b, out, H->n_coarse, mp, stop);
     TAM_LAUNCH_CHECK();
     return;
   }
@@ -783,10 +960,10 @@ void enqueue_multi_iteration(tam_amg_s* H, cudaStream_t s) {
   GridReduce gk{MS.partials.p, MS.tickets.p};
   kspmm(H->K->S, MS.p.p, mp, MS.tK, EpiPqM{MS.p.p, MS.q.p, H->K->n_nodes, mp, gk, MS.sc.p, flags}, s, H->levels[0].Aop.df);
   GridReduce ge{MS.partials.p, MS.tickets.p + MPMAX};
-  mupdate_kernel<<<vgrid(n3), TPB, 0, s>>>(MS.x.p, MS.r.p, MS.p.p, MS.q.p, n3, mp, ge, MS.sc.p, flags);
+  mupdate_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(MS.x.p, MS.r.p, MS.p.p, MS.q.p, n3, mp, ge, MS.sc.p, flags);
   TAM_LAUNCH_CHECK();
   mvcycle<double, double>(H, 0, MS.r.p, MS.z.p, flags, s);
-  mrz_kernel<<<vgrid(n3), TPB, 0, s>>>(MS.r.p, MS.z.p, MS.p.p, n3, mp, 0, ge, MS.sc.p, flags);
+  mrz_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(MS.r.p, MS.z.p, MS.p.p, n3, mp, 0, ge, MS.sc.p, flags);
   TAM_LAUNCH_CHECK();
   mdir_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(MS.z.p, MS.p.p, n3, mp, MS.sc.p, flags);
   TAM_LAUNCH_CHECK();
@@ -803,7 +980,7 @@ void start_multi(tam_amg_s* H, int m, const double* B, const double* X, double r
   interleave_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(X, MS.x.p, m, mp, n3);
   TAM_LAUNCH_CHECK();
   GridReduce ge{MS.partials.p, MS.tickets.p + MPMAX};
-  mstart_kernel<<<vgrid(n3), TPB, 0, s>>>(MS.b.p, n3, m, mp, rtol, atol, max_iter, H->K->vmax_exp / 2, ge, MS.sc.p,
+  mstart_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(MS.b.p, n3, m, mp, rtol, atol, max_iter, H->K->vmax_exp / 2, ge, MS.sc.p,
                                           MS.flags.p);
   TAM_LAUNCH_CHECK();
   mscale_in_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(MS.b.p, MS.x.p, n3, mp, MS.sc.p);
@@ -814,7 +991,7 @@ void start_multi(tam_amg_s* H, int m, const double* B, const double* X, double r
   mcheck_kernel<<<1, 32, 0, s>>>(MS.sc.p, mp, MS.flags.p);
   TAM_LAUNCH_CHECK();
   mvcycle<double, double>(H, 0, MS.r.p, MS.z.p, MS.flags.p, s);
-  mrz_kernel<<<vgrid(n3), TPB, 0, s>>>(MS.r.p, MS.z.p, MS.p.p, n3, mp, 1, ge, MS.sc.p, MS.flags.p);
+  mrz_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(MS.r.p, MS.z.p, MS.p.p, n3, mp, 1, ge, MS.sc.p, MS.flags.p);
   TAM_LAUNCH_CHECK();
 }
 
@@ -827,7 +1004,7 @@ int finish_multi(tam_amg_s* H, int m, const double* B, double* X, int* iters, do
   // the reported true residual is always a plain FP64 product
   kspmm(H->K->S, MS.x.p, mp, MS.tK, EpiResInitM{MS.b.p, nullptr, H->K->n_nodes, mp, gk, MS.sc.p, rn.p, MS.flags.p},
         s, false);
-  deinterleave_kernel<<<vgrid(n3 * m), TPB, 0, s>>>(MS.x.p, X, m, mp, n3, MS.sc.p);
+  deinterleave_kernel<<<vgrid(n3 * mp), TPB, 0, s>>>(MS.x.p, X, m, mp, n3, MS.sc.p);
   TAM_LAUNCH_CHECK();
   std::vector<double> sc(S_COUNT * (size_t)mp), r2(mp);
   int flags[4];
