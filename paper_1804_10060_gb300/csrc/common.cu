@@ -205,8 +205,49 @@ __global__ void scan_apply(const T* in, T* out, long long n, const T* __restrict
   }
 }
 
+// Short arrays: one block scans tile after tile (the next tile's items are
+// read before this one is scanned), one launch instead of three.
+template <typename T>
+__global__ void __launch_bounds__(SCAN_THREADS) scan_small(const T* in, T* out, int n) {
+  __shared__ T sh[32];
+  T carry = 0;
+  T v[SCAN_ITEMS];
+  auto fetch = [&](int base) {
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = base + k < n ? in[base + k] : T(0);
+  };
+  fetch(threadIdx.x * SCAN_ITEMS);
+  for (int t0 = 0; t0 < n; t0 += SCAN_TILE) {
+    const int base = t0 + threadIdx.x * SCAN_ITEMS;
+    T w[SCAN_ITEMS], s = 0;
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+      w[k] = v[k];
+      s += v[k];
+    }
+    fetch(base + SCAN_TILE);  // this tile's writes stay below the next tile (in and out may alias)
+    T tot;
+    T run = carry + block_exclusive_scan<T>(s, sh, &tot);
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+      if (base + k < n) out[base + k] = run;
+      run += w[k];
+    }
+    carry += tot;
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
+// at this length one block's ten tiles take about what three launches do
+constexpr long long SCAN_SMALL = 10 * SCAN_TILE;
+
 template <typename T>
 void exclusive_scan_impl(const T* in, T* out, long long n, cudaStream_t s) {
+  if (n <= SCAN_SMALL) {
+    scan_small<T><<<1, SCAN_THREADS, 0, s>>>(in, out, (int)n);
+    TAM_LAUNCH_CHECK();
+    return;
+  }
   long long tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   if (tiles < 1) tiles = 1;
   DBuf<T> sums((size_t)tiles, s);

@@ -379,12 +379,22 @@ void by_block(int br, F&& f) {
   else f(std::integral_constant<int, 3>());
 }
 
+// K x with an FP64 epilogue, as the CG's products run: accurate double-float
+// over SELL where level 0 multiplies in double-float; plain FP64 otherwise, in
+// level 0's own layout -- a K too small to fill the GPU with a thread per row
+// takes several lanes per row there (unit cube of 1,331 rows: 33 -> 9 us).
+template <int BR, class Epi>
+void spmv_outer(tam_amg_s* H, const double* x, Epi epi, cudaStream_t s) {
+  const SpOp& op = H->levels[0].Aop;
+  if (!op.df && op.lpr != 0) spop_apply<BR, BR>(op, x, epi, s);
+  else sell_spmv<BR, BR, true>(H->K->S, x, epi, s, op.df);
+}
+
 void spmv_outer_pq(tam_amg_s* H, cudaStream_t s) {
   GridReduce gr{H->partials.p, H->ticket.p};
   by_block(H->K->A.br, [&](auto B) {
     constexpr int BR = decltype(B)::value;
-    sell_spmv<BR, BR, true>(H->K->S, H->p.p, EpiPq<BR>{H->p.p, H->q.p, H->K->n_nodes, gr, H->sc.p}, s,
-                            H->levels[0].Aop.df);
+    spmv_outer<BR>(H, H->p.p, EpiPq<BR>{H->p.p, H->q.p, H->K->n_nodes, gr, H->sc.p}, s);
   });
 }
 
@@ -510,8 +520,7 @@ int pcg_solve(tam_amg_s* H, const double* b, double* x, double rtol, double atol
   x = H->xs.p;
   by_block(H->K->A.br, [&](auto B) {
     constexpr int BR = decltype(B)::value;
-    sell_spmv<BR, BR, true>(H->K->S, x, EpiInitResidual<BR>{b, H->r.p, H->K->n_nodes, gr, sc, H->hist.p}, s,
-                            H->levels[0].Aop.df);
+    spmv_outer<BR>(H, x, EpiInitResidual<BR>{b, H->r.p, H->K->n_nodes, gr, sc, H->hist.p}, s);
   });
   precondition(H, H->r.p, H->z.p, &sc->stop, s);
   pcg_rz_kernel<<<vec_grid(N), TPB, 0, s>>>(H->r.p, H->z.p, H->p.p, N, gr, sc, 1);

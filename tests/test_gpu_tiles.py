@@ -205,3 +205,17 @@ def test_batch_right_hand_side_tiles(n_rhs):
             y = torch.zeros_like(b)
             tam.amg_pcg_solve(H, b, y, rtol=1e-10)
             assert float((x - y).norm()) <= 1e-5 * float(y.norm())
+
+
+@pytest.mark.parametrize("n", [0, 1, 4095, 4096, 4097, 40960, 40961, 70001])
+def test_scan_lengths(n):
+    """Meshes of n isolated nodes beside one cell: the pattern's scans at one tile, several tiles of one block and
+    the three-launch path must give every row one block (the cell's four nodes: 4)."""
+    tam = need_gpu()
+    coords = np.concatenate([np.array([[0.0, 0, 0], [1, 0, 0], [0, 1, 0], [0, 0, 1]]), np.full((n, 3), 5.0)])
+    q = meshgen.Problem(name="scan", coords=coords, cells=np.array([[0, 1, 2, 3]], np.int32),
+                        cell_material=np.zeros(1, np.int32), mat_props=np.array([[1.0, 0.3, 1e-3]]), T=None, T_ref=0.0,
+                        body_force=None, dirichlet_mask=np.zeros(n + 4, np.uint8), u_dirichlet=None)
+    K, _ = tam.fem_assemble_elasticity(**tam.problem_to_device(q))
+    rp = tam.tam_matrix_export_bsr(K)[0].cpu().numpy()
+    assert np.array_equal(np.diff(rp), np.r_[np.full(4, 4), np.ones(n, int)])
