@@ -46,12 +46,15 @@ __global__ void __launch_bounds__(256) sell_sort_window_kernel(const int* __rest
 }
 
 // One thread per (slice, lane).  Pads a row with zero blocks pointing at the
-// row's last real column (keeps the padded x reads local).
+// row's last real column (keeps the padded x reads local).  range (may be
+// null): the operator's exponent range of the same pass, see
+// ExponentRange -- [0] the largest biased FP64 exponent over the
+// rows with more than one block, [1] whether an inf or NaN was met.
 __global__ void sell_fill_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col_idx,
                                  const double* __restrict__ vals, int n_rows, int n_slices, int bb,
                                  const int* __restrict__ slice_ptr, const int* __restrict__ perm,
                                  int* __restrict__ scols, double* __restrict__ svals, float2* __restrict__ svals_df,
-                                 bool with_pattern) {
+                                 bool with_pattern, int* __restrict__ range) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   int s = t >> 5, lane = t & 31;
   if (s >= n_slices) return;
@@ -63,6 +66,7 @@ __global__ void sell_fill_kernel(const int* __restrict__ row_ptr, const int* __r
   }
   int k0 = slice_ptr[s], K = slice_ptr[s + 1] - k0;
   int lastc = len > 0 ? col_idx[rp + len - 1] : 0;
+  int emax = 0, bad = 0;
   for (int k = 0; k < K; ++k) {
     size_t slot = (size_t)(k0 + k);
     if (with_pattern) scols[slot * 32 + lane] = k < len ? col_idx[rp + k] : lastc;
@@ -70,13 +74,32 @@ __global__ void sell_fill_kernel(const int* __restrict__ row_ptr, const int* __r
       const double x = k < len ? vals[((size_t)rp + k) * bb + e] : 0.0;
       svals[(slot * bb + e) * 32 + lane] = x;
       if (svals_df) svals_df[(slot * bb + e) * 32 + lane] = split_bits(x);  // the split copy in the same pass
+      const int ex = (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff);
+      if (ex == 0x7ff) bad = 1;
+      else emax = max(emax, ex);
+    }
+  }
+  if (range) {  // whole warps are here (n_slices x 32 threads)
+    if (len <= 1) emax = 0;
+    emax = __reduce_max_sync(0xffffffffu, emax);
+    bad = __reduce_or_sync(0xffffffffu, bad);
+    if (lane == 0) {
+      if (emax) atomicMax(range, emax);
+      if (bad) atomicOr(range + 1, 1);
     }
   }
 }
 
 }  // namespace
 
-void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df) {
+static void read_range(const DBuf<int>& out, ExponentRange* range, cudaStream_t s) {
+  int e = 0, bad = 0;
+  read_back_int2(out.p, out.p + 1, &e, &bad, s);
+  range->max_exp = e ? e - 1023 : 0;
+  range->finite = bad == 0;
+}
+
+void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df, ExponentRange* range) {
   TAM_CHECK(A.n_cols > 0, TAM_ERR_INTERNAL, "SELL of a matrix without columns");
   S.n_rows = A.n_rows;
   S.br = A.br;
@@ -102,59 +125,29 @@ void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df) {
   S.cols = DBuf<int>((size_t)S.n_slots * 32, s);
   S.vals = DBuf<double>((size_t)S.n_slots * 32 * A.block_elems(), s);
   if (df) S.vals_df = DBuf<float2>((size_t)std::max(1LL, S.n_slots * 32 * (long long)A.block_elems()), s);
+  DBuf<int> out;
+  if (range) {
+    out = DBuf<int>(2, s);
+    out.zero();
+  }
   sell_fill_kernel<<<grid_for((long long)S.n_slices * 32, 256), 256, 0, s>>>(
       A.row_ptr.p, A.col_idx.p, A.vals.p, A.n_rows, S.n_slices, (int)A.block_elems(),
-      S.slice_ptr.p, S.perm.p, S.cols.p, S.vals.p, df ? S.vals_df.p : nullptr, true);
+      S.slice_ptr.p, S.perm.p, S.cols.p, S.vals.p, df ? S.vals_df.p : nullptr, true, out.p);
   TAM_LAUNCH_CHECK();
+  if (range) read_range(out, range, s);
 }
 
-void sell_refresh_values(const Bsr& A, Sell& S, cudaStream_t s) {
+void sell_refresh_values(const Bsr& A, Sell& S, cudaStream_t s, ExponentRange* range) {
+  DBuf<int> out;
+  if (range) {
+    out = DBuf<int>(2, s);
+    out.zero();
+  }
   sell_fill_kernel<<<grid_for((long long)S.n_slices * 32, 256), 256, 0, s>>>(
       A.row_ptr.p, A.col_idx.p, A.vals.p, A.n_rows, S.n_slices, (int)A.block_elems(),
-      S.slice_ptr.p, S.perm.p, S.cols.p, S.vals.p, S.vals_df.p, false);
+      S.slice_ptr.p, S.perm.p, S.cols.p, S.vals.p, S.vals_df.p, false, out.p);
   TAM_LAUNCH_CHECK();
-}
-
-namespace {
-// Largest biased FP64 exponent (out[0]; 0: none) of the entries of a
-// block-CSR matrix and an inf/NaN flag (out[1]), leaving out rows that hold only their diagonal block (Dirichlet and cell-less nodes:
-// identity rows whose 1.0 says nothing about the operator's scale); inf/NaN
-// are flagged in every row.
-__global__ void row_exponent_range_kernel(const int* __restrict__ rp, const double* __restrict__ v, int n_rows,
-                                          int bb, int* __restrict__ out) {
-  int emax = 0, bad = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_rows; i += gridDim.x * blockDim.x) {
-    const int p0 = rp[i], p1 = rp[i + 1];
-    const bool scale_row = p1 - p0 > 1;
-    for (long long k = (long long)p0 * bb; k < (long long)p1 * bb; ++k) {
-      const int e = (int)(((unsigned long long)__double_as_longlong(v[k]) >> 52) & 0x7ff);
-      if (e == 0x7ff) bad = 1;
-      else if (scale_row) emax = max(emax, e);
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (emax) atomicMax(out, emax);
-    if (bad) atomicOr(out + 1, 1);
-  }
-}
-}  // namespace
-
-void operator_exponent_range(const Bsr& A, int* max_exp, bool* finite, cudaStream_t s) {
-  DBuf<int> out(2, s);
-  out.zero();
-  if (A.n_rows > 0) {
-    row_exponent_range_kernel<<<stride_grid(A.n_rows, 256, 8), 256, 0, s>>>(A.row_ptr.p, A.vals.p, A.n_rows,
-                                                                           (int)A.block_elems(), out.p);
-    TAM_LAUNCH_CHECK();
-  }
-  int e = 0, bad = 0;
-  read_back_int2(out.p, out.p + 1, &e, &bad, s);
-  *max_exp = e ? e - 1023 : 0;
-  *finite = bad == 0;
+  if (range) read_range(out, range, s);
 }
 
 namespace {

@@ -146,12 +146,14 @@ __device__ __forceinline__ void df_add_accurate(float2& a, float2 b) {
 // to FP64 outside it).
 constexpr int kDfExpLimit = 90;
 
-struct Bsr;
-// Binary exponent of A's largest |entry| (floor(log2 max |A_ij|); 0 when there
-// is none) into *max_exp, over the block rows that hold more than their
-// diagonal block (identity rows of Dirichlet and cell-less nodes do not set
-// the scale), and whether every entry is finite.  Synchronising.
-void operator_exponent_range(const Bsr& A, int* max_exp, bool* finite, cudaStream_t s);
+// Binary exponent of an operator's largest |entry| (floor(log2 max |A_ij|); 0
+// when there is none), over the block rows that hold more than their diagonal
+// block (identity rows of Dirichlet and cell-less nodes do not set the scale),
+// and whether every entry is finite.  Found while the SELL copy is written.
+struct ExponentRange {
+  int max_exp = 0;
+  bool finite = true;
+};
 
 struct Bsr {
   int n_rows = 0, n_cols = 0, br = 0, bc = 0;
@@ -199,10 +201,11 @@ void build_df_values(Sell& S, cudaStream_t s);
 void build_df_values(Bsr& B, cudaStream_t s);
 
 // Builds the SELL-32 copy of a Bsr (pattern + values).
-void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df = false);  // df: the split copy too
+// df: the split copy too; range: the values' exponent range (then synchronising)
+void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df = false, ExponentRange* range = nullptr);
 // Refreshes only the values of an existing SELL copy built from A (and its
 // split copy, when it has one).
-void sell_refresh_values(const Bsr& A, Sell& S, cudaStream_t s);
+void sell_refresh_values(const Bsr& A, Sell& S, cudaStream_t s, ExponentRange* range = nullptr);
 
 // Transpose (block transpose included): R = A^T.  Rows of R sorted by column.
 void bsr_transpose(const Bsr& A, Bsr& R, cudaStream_t s);

@@ -615,8 +615,10 @@ void thermal_assemble(tam_thermal_s* th, const double* T, const double* T_old, d
   TAM_LAUNCH_CHECK();
   TAM_CHECK(read_back_int(bad.p, s) == 0, TAM_ERR_DEGENERATE_CELL, "thermal: a cell has non-positive volume");
   // the SpMV copy and the exponent range of the new values
-  sell_refresh_values(A, th->J->S, s);
-  operator_exponent_range(A, &th->J->vmax_exp, &th->J->finite, s);
+  ExponentRange range;
+  sell_refresh_values(A, th->J->S, s, &range);
+  th->J->vmax_exp = range.max_exp;
+  th->J->finite = range.finite;
   th->J->df_ok = th->J->finite && std::abs(th->J->vmax_exp) <= kDfExpLimit && th->J->S.vals_df.p;
 }
 
