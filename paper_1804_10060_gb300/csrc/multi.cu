@@ -355,10 +355,8 @@ kspmm_kernel(SellView A, const double* __restrict__ x, int mp, Epi epi) {
         for (int k = 0; k < TM; ++k) ad[r][k] = make_float2(0.f, 0.f);
       for (int s = k0; s < k1; ++s) {
         const int c = __ldg(A.cols + (size_t)s * 32 + lane);
-        const float2* __restrict__ vp = A.vals_df + (size_t)s * 32 * 9 + lane;
         float2 v[9];
-#pragma unroll
-        for (int e = 0; e < 9; ++e) v[e] = __ldg(vp + e * 32);
+        slot_load<9, 32>(A.vals_df + (size_t)s * 32 * 9, lane, v);
 #pragma unroll
         for (int jc = 0; jc < 3; ++jc) {
           double xr[TM];
@@ -535,10 +533,8 @@ msell_kernel(int n_slices, const int* __restrict__ slice_ptr, const int* __restr
   if (slice < n_slices) {
     const int k0 = slice_ptr[slice], k1 = slice_ptr[slice + 1];
     for (int s = k0; s < k1; ++s) {
-      const TV* __restrict__ vp = vals + (size_t)s * 32 * BR * BC + lane;
       TV vv[BR * BC];  // the slot's values first, then the gathers
-#pragma unroll
-      for (int e = 0; e < BR * BC; ++e) vv[e] = vp[e * 32];
+      slot_load<BR * BC, 32>(vals + (size_t)s * 32 * BR * BC, lane, vv);
       const int c = __ldg(cols + (size_t)s * 32 + lane);
 #pragma unroll
       for (int jc = 0; jc < BC; ++jc) {

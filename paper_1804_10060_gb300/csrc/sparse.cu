@@ -73,7 +73,7 @@ __global__ void sell_fill_kernel(const int* __restrict__ row_ptr, const int* __r
     for (int e = 0; e < bb; ++e) {
       const double x = k < len ? vals[((size_t)rp + k) * bb + e] : 0.0;
       svals[(slot * bb + e) * 32 + lane] = x;
-      if (svals_df) svals_df[(slot * bb + e) * 32 + lane] = split_bits(x);  // the split copy in the same pass
+      if (svals_df) svals_df[slot * bb * 32 + pack_pos(2, 32, bb, e, lane)] = split_bits(x);  // the split copy in the same pass
       const int ex = (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff);
       if (ex == 0x7ff) bad = 1;
       else emax = max(emax, ex);
@@ -197,7 +197,7 @@ __global__ void lpr_fill_kernel(const int* __restrict__ rp, const int* __restric
     const int idx = s0 + (e & (lpr - 1));
     const double x = idx < e0 ? v[(size_t)idx * bb + (e >> sh)] : 0.0;
     vals[w * n + e] = x;
-    if (vals_df) vals_df[w * n + e] = split_bits(x);
+    if (vals_df) vals_df[w * n + pack_pos(2, lpr, bb, e >> sh, e & (lpr - 1))] = split_bits(x);
   }
 }
 }  // namespace
@@ -225,10 +225,6 @@ void build_lpr_store(const Bsr& A, int lpr, bool df, LprStore& L, cudaStream_t s
       A.row_ptr.p, A.col_idx.p, A.vals.p, lpr, (int)A.block_elems(), L.grp_ptr.p, grow.p, L.n_groups, L.cols.p,
       L.vals.p, df ? L.vals_df.p : nullptr);
   TAM_LAUNCH_CHECK();
-}
-
-void build_df_values(Sell& S, cudaStream_t s) {
-  split_into(S.vals.p, S.n_slots * 32 * (long long)S.br * S.bc, S.vals_df, s);
 }
 
 void build_df_values(Bsr& B, cudaStream_t s) {
@@ -1176,36 +1172,36 @@ bool bsr_spgemm_tentative(const Bsr& X, const Bsr& Pt, const int* agg, Bsr& C, c
 // Reduced-precision value copies
 // ---------------------------------------------------------------------------
 namespace {
+__device__ __forceinline__ void round_to(double v, float& out) { out = __double2float_rn(v); }
+__device__ __forceinline__ void round_to(double v, __nv_bfloat16& out) { out = __double2bfloat16(v); }
+
 template <typename T>
-__global__ void convert_kernel(const double* __restrict__ in, T* __restrict__ out, long long n);
-template <>
-__global__ void convert_kernel<float>(const double* __restrict__ in, float* __restrict__ out, long long n) {
+__global__ void convert_kernel(const double* __restrict__ in, T* __restrict__ out, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    out[i] = __double2float_rn(in[i]);
+    round_to(in[i], out[i]);
 }
-template <>
-__global__ void convert_kernel<__nv_bfloat16>(const double* __restrict__ in, __nv_bfloat16* __restrict__ out,
-                                              long long n) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    out[i] = __double2bfloat16(in[i]);
+
+// SELL values (element-major slots) into packed slots
+template <typename T>
+__global__ void convert_slots_kernel(const double* __restrict__ in, T* __restrict__ out, long long n, int bb) {
+  const int slot = 32 * bb;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long s0 = i / slot * slot;
+    const int r = (int)(i - s0);
+    round_to(in[i], out[s0 + pack_pos(pack_of(sizeof(T)), 32, bb, r >> 5, r & 31)]);
+  }
 }
 
 template <typename T>
 void convert_values(const SpOp& op, DBuf<T>& out, cudaStream_t s) {
-  const double* src;
-  long long n;
-  if (op.lpr == 0) {
-    src = op.S->vals.p;
-    n = op.S->n_slots * 32 * (long long)op.S->br * op.S->bc;
-  } else {
-    src = op.B->vals.p;
-    n = op.B->nnzb * (long long)op.B->block_elems();
-  }
+  const bool sell = op.lpr == 0;
+  const int bb = sell ? op.S->br * op.S->bc : (int)op.B->block_elems();
+  const long long n = (sell ? op.S->n_slots * 32 : op.B->nnzb) * (long long)bb;
   out = DBuf<T>((size_t)std::max(1LL, n), s);
-  if (n > 0) {
-    convert_kernel<T><<<stride_grid(n, 256, 16), 256, 0, s>>>(src, out.p, n);
-    TAM_LAUNCH_CHECK();
-  }
+  if (n <= 0) return;
+  if (sell) convert_slots_kernel<T><<<stride_grid(n, 256, 16), 256, 0, s>>>(op.S->vals.p, out.p, n, bb);
+  else convert_kernel<T><<<stride_grid(n, 256, 16), 256, 0, s>>>(op.B->vals.p, out.p, n);
+  TAM_LAUNCH_CHECK();
 }
 }  // namespace
 

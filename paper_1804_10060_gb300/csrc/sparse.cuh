@@ -170,13 +170,53 @@ struct Sell {
   DBuf<int> slice_ptr;    // [n_slices + 1]
   DBuf<int> cols;         // [n_slots * 32]
   DBuf<double> vals;      // [n_slots * 32 * br * bc]
-  DBuf<float2> vals_df;   // optional split copy of vals
+  DBuf<float2> vals_df;   // optional split copy of vals, packed (pack_pos)
   // optional row order (SELL-C-sigma): slot position p holds row perm[p]; rows
   // are sorted by length within windows of 256 so that a slice's rows have
   // similar lengths (P2 meshes interleave long vertex rows with short edge
   // rows: 40% padding unsorted, 8% sorted).  Empty: position p holds row p.
   DBuf<int> perm;
 };
+
+// The split and reduced-precision copies of the slot layouts (SELL: 32 blocks a
+// slot, LprStore: lpr blocks a group) keep a block's elements in packs of W
+// for one request (16 bytes: W = 2 float2, 4 float, 8 BF16): pack q of block j
+// at [(q * width + j) * W], the elements left over after the whole packs one by
+// one behind them.  Element by element a 3 x 3 slot took nine requests, and the
+// FP32 kernels stalled on the load queue rather than on memory.
+__host__ __device__ constexpr int pack_of(size_t value_bytes) { return (int)(16 / value_bytes); }
+__host__ __device__ constexpr int pack_pos(int W, int width, int bb, int e, int j) {
+  return e < bb / W * W ? (e / W * width + j) * W + e % W : e * width + j;
+}
+
+// Block j of a slot (or group) of `width` packed blocks.
+template <int BB, int WIDTH, typename V>
+__device__ __forceinline__ void slot_load(const V* __restrict__ slot, int j, V (&out)[BB]) {
+  constexpr int W = pack_of(sizeof(V)), Q = BB / W;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(slot) + q * WIDTH + j);
+    if constexpr (sizeof(V) == 8) {
+      out[2 * q] = make_float2(v.x, v.y);
+      out[2 * q + 1] = make_float2(v.z, v.w);
+    } else if constexpr (sizeof(V) == 4) {
+      out[4 * q] = v.x;
+      out[4 * q + 1] = v.y;
+      out[4 * q + 2] = v.z;
+      out[4 * q + 3] = v.w;
+    } else {
+      const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&w[i]);
+        out[8 * q + 2 * i] = b.x;
+        out[8 * q + 2 * i + 1] = b.y;
+      }
+    }
+  }
+#pragma unroll
+  for (int e = Q * W; e < BB; ++e) out[e] = __ldg(slot + e * WIDTH + j);
+}
 
 struct SellView {
   int n_rows, n_slices;
@@ -197,7 +237,6 @@ __device__ __forceinline__ int sell_row(const int* __restrict__ perm, int pos, i
 }
 
 // (Re)builds the split copy vals_df from vals (integer operations only).
-void build_df_values(Sell& S, cudaStream_t s);
 void build_df_values(Bsr& B, cudaStream_t s);
 
 // Builds the SELL-32 copy of a Bsr (pattern + values).
@@ -317,7 +356,7 @@ sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
     const int k0 = A.slice_ptr[slice] + sub, k1 = A.slice_ptr[slice + 1];
     const int* __restrict__ cp = A.cols + (size_t)k0 * 32 + lane;
     if constexpr (DF) {
-      const float2* __restrict__ vp = A.vals_df + (size_t)k0 * 32 * BR * BC + lane;
+      const float2* __restrict__ vp = A.vals_df + (size_t)k0 * 32 * BR * BC;
       // one slot's products into the rows' sums.  ACC: the slot's double-float
       // partial sum (its BC products) is added into the row's running sum with
       // the accurate double-word addition, so that the low part never carries
@@ -352,8 +391,7 @@ sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
 #pragma unroll 2
         for (int k = k0; k < k1; k += S) {
           float2 vv[BR * BC];
-#pragma unroll
-          for (int e = 0; e < BR * BC; ++e) vv[e] = __ldg(vp + e * 32);
+          slot_load<BR * BC, 32>(vp, lane, vv);
           double xg[BC];
           gather_x<BC, AL>(x, c0, xg);
           c0 = c1;
@@ -378,7 +416,7 @@ sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
             vv[u][0] = make_float2(0.f, 0.f);
             xg[u][0] = 0.0;
             if (u == 0 || k + u * S < k1) {
-              vv[u][0] = __ldg(vp + u * S * 32);
+              vv[u][0] = __ldg(vp + u * S * 32 + lane);
               gather_x<1, AL>(x, cn[u], xg[u]);
             }
           }
@@ -561,7 +599,7 @@ struct LprStore {
   DBuf<int> grp_ptr;     // [n_rows + 1], in groups
   DBuf<int> cols;        // [n_groups * lpr]
   DBuf<double> vals;     // [n_groups * lpr * br * bc]
-  DBuf<float2> vals_df;  // optional split copy
+  DBuf<float2> vals_df;  // optional split copy, packed (pack_pos)
 };
 
 // Builds L from A for lanes-per-row width lpr (and the split copy when df).
@@ -608,10 +646,8 @@ lpr_spmv_kernel(LprView A, const double* __restrict__ x, Epi epi) {
         gather_x<BC, AL && BC != 3>(x, c, xg);
       }
       for (int g = g0; g < g1; ++g) {
-        const float2* __restrict__ vb = A.v_df + (size_t)g * BB * LPR + sub;
         float2 vv[BB];
-#pragma unroll
-        for (int e = 0; e < BB; ++e) vv[e] = __ldg(vb + e * LPR);
+        slot_load<BB, LPR>(A.v_df + (size_t)g * BB * LPR, sub, vv);
         float2 xv[BC];
 #pragma unroll
         for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
@@ -693,10 +729,8 @@ lpr_rows_kernel(LprView A, const double* __restrict__ x, Epi epi) {
     if (row < A.n_rows) {
       const int g1 = A.gp[row + 1];
       for (int g = A.gp[row] + sub / ROWS_LPR; g < g1; g += GS) {
-        const float2* __restrict__ vb = A.v_df + (size_t)g * BB * ROWS_LPR + ln;
         float2 vv[BB];
-#pragma unroll
-        for (int e = 0; e < BB; ++e) vv[e] = __ldg(vb + e * ROWS_LPR);
+        slot_load<BB, ROWS_LPR>(A.v_df + (size_t)g * BB * ROWS_LPR, ln, vv);
         const int c = __ldg(A.cols + (size_t)g * ROWS_LPR + ln);
         double xg[BC];
         gather_x<BC, AL>(x, c, xg);
@@ -1190,12 +1224,11 @@ sell_spmv_f32_kernel(int n_slices, const int* __restrict__ slice_ptr, const int*
   if (slice < n_slices) {
     const int k0 = slice_ptr[slice] + sub, k1 = slice_ptr[slice + 1];
     const int* __restrict__ cp = cols + (size_t)k0 * 32 + lane;
-    const TV* __restrict__ vp = vals + (size_t)k0 * 32 * BR * BC + lane;
+    const TV* __restrict__ vp = vals + (size_t)k0 * 32 * BR * BC;
 #pragma unroll 4
     for (int k = k0; k < k1; k += S) {
       TV vv[BR * BC];  // the slot's values first, then the gather
-#pragma unroll
-      for (int e = 0; e < BR * BC; ++e) vv[e] = vp[e * 32];
+      slot_load<BR * BC, 32>(vp, lane, vv);
       const int c = __ldg(cp);
       float xv[BC];
       gather_f32<BC>(x, c, xv);
@@ -1286,7 +1319,7 @@ void spop_apply_f32(const SpOpLow<TV>& o, const float* x, Epi epi, cudaStream_t 
   TAM_LAUNCH_CHECK();
 }
 
-// Values of `op` (whichever layout it uses) as a reduced-precision copy.
+// Values of `op` (whichever layout it uses; SELL slots packed, see pack_pos) as a reduced-precision copy.
 void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s);
 void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s);
 
