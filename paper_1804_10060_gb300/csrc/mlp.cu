@@ -45,6 +45,16 @@ namespace {
 constexpr int ROWS = 64;   // rows of the activation tile per block
 constexpr int THREADS = 256;
 
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf's): the FP32
+// kernels below are bound by instruction issue, and the packed form halves
+// their multiply-adds' share of it.
+__device__ __forceinline__ void fma2(float2& acc, float2 a, float2 b) {
+  unsigned long long& c = reinterpret_cast<unsigned long long&>(acc);
+  asm("fma.rn.f32x2 %0, %1, %2, %0;"
+      : "+l"(c)
+      : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)));
+}
+
 // out[n x N] = epi(A[n x K] W + bias) with W [K x N] row-major (or W^T when
 // TRANS: W stored [N x K]).  MODE: 0 linear, 1 tanh, 2 output (* out_scale),
 // 3 backward through tanh: out = (A W^T) * (1 - H^2) with H = `aux`.
@@ -56,9 +66,9 @@ constexpr int THREADS = 256;
 // steps of k cost TM + TN 16-byte shared loads for 4 TM TN multiply-adds (the
 // kernel before, one row by 8 outputs a thread with scalar loads and a bounds
 // test per product, spent nine loads on eight products).  Threads: NG column
-// groups x 256 / NG row groups; a thread's rows are its group's number plus
-// multiples of the group count, which keeps a warp's row reads on different
-// banks.  Two blocks fit an SM and hide each other's loads.  Each output sums
+// groups x 256 / NG row groups, a warp 8 x 4 of them, so that its weight reads
+// are 128 bytes; a thread's rows are its group's number plus multiples of the
+// group count, which keeps a warp's row reads on different banks.  Two blocks fit an SM and hide each other's loads.  Each output sums
 // its products in increasing k.  The 8-128-128-128-3 network on 468,864 rows:
 // 8.74 -> 1.14 ms (28 TFLOP/s of 76.8).
 template <int MODE, bool TRANS, bool STD, int TM, int TN, int NG>
@@ -76,9 +86,15 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
   if (TRANS) {
     for (int e = threadIdx.x; e < Kp * Np; e += THREADS) Ws[e] = 0.f;
     __syncthreads();
-    for (int e = threadIdx.x; e < K * N; e += THREADS) {
-      const int j = e / K, k = e - j * K;
-      Ws[k * Np + j] = W[e];
+    // a warp transposes 8 rows x 4 groups of 4 columns: 8 lines per read, 4
+    // lanes per bank and write
+    const int kq = (K + 3) >> 2, jb = (N + 7) >> 3, kb = (kq + 3) >> 2;
+    for (int t = threadIdx.x >> 5; t < jb * kb; t += THREADS / 32) {
+      const int j = (t % jb) * 8 + (threadIdx.x & 7), k = ((t / jb) * 4 + ((threadIdx.x & 31) >> 3)) * 4;
+      if (j < N)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (k + q < K) Ws[(k + q) * Np + j] = W[(size_t)j * K + k + q];
     }
   } else {
     for (int e = threadIdx.x; e < Kp * Np; e += THREADS) {
@@ -86,7 +102,10 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
       Ws[e] = (k < K && j < N) ? W[(size_t)k * N + j] : 0.f;
     }
   }
-  const int cg = threadIdx.x % NG, rg = threadIdx.x / NG;
+  // a warp: CW column groups (128 bytes of a weight row) x 32 / CW row groups
+  constexpr int CW = NG < 8 ? NG : 8, NW = NG / CW;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int cg = lane % CW + CW * (wid % NW), rg = lane / CW + (32 / CW) * (wid / NW);
   for (long long r0 = (long long)blockIdx.x * ROWS; r0 < n; r0 += (long long)gridDim.x * ROWS) {
     __syncthreads();
     if (a_vec) {
@@ -115,11 +134,12 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
       }
     }
     __syncthreads();
-    float acc[TM][TN];
+    constexpr int TP = (TN + 1) / 2;  // output pairs (TN = 1: the second half idle)
+    float2 acc[TM][TP];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+      for (int j = 0; j < TP; ++j) acc[i][j] = make_float2(0.f, 0.f);
     for (int k = 0; k < Kp; k += 4) {
       float av[TM][4];
 #pragma unroll
@@ -133,23 +153,25 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
         const float* wr = Ws + (k + kk) * Np;
-        float w[TN];
         if constexpr (TN == 1) {
-          w[0] = wr[cg];
+          const float w = wr[cg];
+#pragma unroll
+          for (int i = 0; i < TM; ++i) acc[i][0].x = fmaf(av[i][kk], w, acc[i][0].x);
         } else {
+          float2 w[TP];
 #pragma unroll
           for (int h = 0; h < TN / 4; ++h) {
             const float4 v = *reinterpret_cast<const float4*>(wr + h * 4 * NG + cg * 4);
-            w[4 * h] = v.x;
-            w[4 * h + 1] = v.y;
-            w[4 * h + 2] = v.z;
-            w[4 * h + 3] = v.w;
+            w[2 * h] = make_float2(v.x, v.y);
+            w[2 * h + 1] = make_float2(v.z, v.w);
+          }
+#pragma unroll
+          for (int i = 0; i < TM; ++i) {
+            const float2 a = make_float2(av[i][kk], av[i][kk]);
+#pragma unroll
+            for (int j = 0; j < TP; ++j) fma2(acc[i][j], a, w[j]);
           }
         }
-#pragma unroll
-        for (int i = 0; i < TM; ++i)
-#pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(av[i][kk], w[j], acc[i][j]);
       }
     }
 #pragma unroll
@@ -166,7 +188,8 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
           const int c = c0 + q;
           z[q] = 0.f;
           if (c >= N) continue;
-          z[q] = acc[i][h * 4 + q] + (bias ? bias[c] : 0.f);
+          const float2 p = acc[i][(h * 4 + q) / 2];
+          z[q] = ((q & 1) ? p.y : p.x) + (bias ? bias[c] : 0.f);
           if (MODE == 1) z[q] = tanhf(z[q]);
           else if (MODE == 2) z[q] *= out_scale[c];
           else if (MODE == 3) {
@@ -202,14 +225,18 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
   constexpr int Kp = 16 * TK, Np = 16 * TN;  // 16 x 16 threads
   __shared__ __align__(16) float Hs[WG_ROWS][Kp];
   __shared__ __align__(16) float Ds[WG_ROWS][Np];
-  const int kg = threadIdx.x >> 4, ng = threadIdx.x & 15;
-  float acc[TK][TN], accb[TN];
+  // a warp: 4 x 8 threads, so that its reads of a row are 64 and 128 bytes
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int kg = (lane >> 3) + 4 * (wid >> 1), ng = (lane & 7) + 8 * (wid & 1);
+  constexpr int TP = (TN + 1) / 2;  // pairs of outputs (TN = 1: the second half idle)
+  float2 acc[TK][TP];
+  float accb[TN];
 #pragma unroll
-  for (int j = 0; j < TN; ++j) {
-    accb[j] = 0.f;
+  for (int j = 0; j < TN; ++j) accb[j] = 0.f;
 #pragma unroll
-    for (int i = 0; i < TK; ++i) acc[i][j] = 0.f;
-  }
+  for (int j = 0; j < TP; ++j)
+#pragma unroll
+    for (int i = 0; i < TK; ++i) acc[i][j] = make_float2(0.f, 0.f);
   // rows of src [n x M] from r0 into dst [WG_ROWS][Mp], zero-padded
   auto fill = [&](const float* __restrict__ src, int M, int Mp, float* dst, bool vec, bool std_, long long r0) {
     if (vec) {
@@ -266,11 +293,18 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
       float h[TK], d[TN];
       take(Hs[r], kg, h);
       take(Ds[r], ng, d);
+      if (kg == 0)
 #pragma unroll
-      for (int j = 0; j < TN; ++j) {
-        if (kg == 0) accb[j] += d[j];
+        for (int j = 0; j < TN; ++j) accb[j] += d[j];
 #pragma unroll
-        for (int i = 0; i < TK; ++i) acc[i][j] = fmaf(h[i], d[j], acc[i][j]);
+      for (int i = 0; i < TK; ++i) {
+        if constexpr (TN == 1) {
+          acc[i][0].x = fmaf(h[i], d[0], acc[i][0].x);
+        } else {
+          const float2 hh = make_float2(h[i], h[i]);
+#pragma unroll
+          for (int j = 0; j < TP; ++j) fma2(acc[i][j], hh, make_float2(d[2 * j], d[2 * j + 1]));
+        }
       }
     }
   }
@@ -281,7 +315,7 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
       const int c = TN == 1 ? ng : (j / 4) * 64 + 4 * ng + (j & 3);
-      if (k < K && c < N) o[(size_t)k * N + c] = acc[i][j];
+      if (k < K && c < N) o[(size_t)k * N + c] = (j & 1) ? acc[i][j / 2].y : acc[i][j / 2].x;
       if (kg == 0 && i == 0 && c < N) o[(size_t)K * N + c] = accb[j];
     }
   }
