@@ -311,6 +311,10 @@ __global__ void mis_round1_kernel(const int* __restrict__ rp, const int* __restr
                                   const int* __restrict__ prev_und) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n || (prev_und && *prev_und == 0)) return;
+  // once a root is in the closed neighbourhood that is all round 2 asks (any
+  // root's tuple sends an undecided node out): later rounds skip the node --
+  // after the first few, nearly all of them
+  if (prev_und && (m1[i] >> 62) == 2ull) return;
   unsigned long long m = tup[i];
   for (int p = rp[i]; p < rp[i + 1]; ++p)
     if (strong[p]) {
