@@ -925,13 +925,17 @@ blockrow_spmv_kernel(BsrView A, const double* __restrict__ x, Epi epi) {
 }
 
 // Warps per row for blockrow_spmv_kernel: enough warps for two waves of 32
-// resident warps per SM, while each warp keeps at least four steps.
+// resident warps per SM.  A warp keeps at least four steps where its rows come
+// near that (the sums of its row's warps cost a barrier), one where the rows
+// alone leave most of the chip idle (level 1 of a 56k-DOF box: 700 rows of 8
+// steps, 12.3 us with a warp each, 8.5 with four).
 inline int blockrow_wpr(int n_rows, long long nnzb, int br) {
   if (n_rows <= 0) return 1;
   const long long want = 2LL * sm_count() * 32;
   const double steps = (double)nnzb / n_rows / (32 / br);
   int w = 1;
-  while (w < 8 && (long long)n_rows * w < want && steps / (2 * w) >= 4.0) w <<= 1;
+  while (w < 8 && (long long)n_rows * w < want && steps / (2 * w) >= ((long long)n_rows * w < want / 4 ? 1.0 : 4.0))
+    w <<= 1;
   return w;
 }
 
@@ -999,6 +1003,10 @@ inline int choose_lpr(const Bsr& A) {
   const int per_lane = A.n_rows < 65536 ? 8 : 16;
   while (l < 32 && per_lane * l < avg) l <<= 1;
   if (A.n_rows < 8192) l = std::max(l, 16);  // few rows: spread them over more lanes
+  // more rows, but still less than half the chip's threads: two blocks a lane
+  // (level 0 of a 56k-DOF box, 18,785 rows of 14, 2 -> 4 lanes: with the rule of
+  // blockrow_wpr its V-cycle took 178 -> 146 us)
+  while (A.n_rows < 65536 && l < 8 && 2LL * A.n_rows * l <= spmv_fill_threads() && avg / (2 * l) >= 1.75) l <<= 1;
   // rows enough to fill the GPU at 8 lanes each: the coalesced 8-lane
   // interleaved store beats 16-32 lanes over the block-CSR arrays
   if (l > 8 && (long long)A.n_rows * 8 >= spmv_fill_threads()) l = 8;
