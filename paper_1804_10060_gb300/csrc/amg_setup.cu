@@ -789,7 +789,9 @@ static void lanczos_lambda(tam_amg_s* H, Level& L, int level, cudaStream_t s, Gr
   DBuf<int> mdone(2, s);
   ab.zero();
   TAM_CUDA(cudaMemsetAsync(mdone.p, 0, 2 * sizeof(int), s));
-  const unsigned g = std::min<unsigned>(grid_for(N, TPB), (unsigned)H->max_grid);
+  // several entries a thread: with one each, the FP64 block sums of 12,700
+  // blocks took longer than the vectors (3.26M entries: 73 us a pass)
+  const unsigned g = stride_grid(N, TPB, 8);
   lanczos_init_kernel<<<g, TPB, 0, s>>>(L.dinv.p, N, level, sv.p, v.p, gr, nrm.p);
   TAM_LAUNCH_CHECK();
   lanczos_normalize_kernel<<<g, TPB, 0, s>>>(N, v.p, sv.p, u.p, vp.p, nrm.p);
@@ -1149,10 +1151,10 @@ tam_amg_s* amg_build(tam_matrix_s* K, const double* coords, const amg_params& pr
       if (last || L.n_agg == 0 || L.n_agg >= L.n_rows) {
         L.n_agg = 0;
         L.agg.reset();
-        T.mark(0, s);
-        side.join(s);  // before the cooperative launch of the coarse inverse
         T.mark(7, s);
-        coarse_inverse(H, L, lev > 0 || L.bs == 3, s);
+        coarse_inverse(H, L, lev > 0 || L.bs == 3, s);  // beside this level's Lanczos estimate
+        T.mark(0, s);
+        side.join(s);
         break;
       }
       DBuf<double> Bc;

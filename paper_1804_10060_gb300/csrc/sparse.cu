@@ -556,10 +556,20 @@ spgemm_numeric_os_kernel(const int* __restrict__ xrp, const int* __restrict__ xc
 #pragma unroll
   for (int e = 0; e < M * N; ++e) acc[e] = Ar::zero();
   const int pe = xrp[i + 1];
-  for (int p = xrp[i]; p < pe; ++p) {
-    const int j = xci[p];
-    int lo = yrp[j], hi = yrp[j + 1];
+  // the next X entry's column and Y row are requested while this one's are
+  // used: two dependent round trips an entry instead of four
+  int p = xrp[i];
+  int jn = p < pe ? xci[p] : 0;
+  int lo_n = p < pe ? yrp[jn] : 0, hi_n = p < pe ? yrp[jn + 1] : 0;
+  jn = p + 1 < pe ? xci[p + 1] : 0;
+  for (; p < pe; ++p) {
+    int lo = lo_n, hi = hi_n;
     const int end = hi;
+    if (p + 1 < pe) {
+      lo_n = yrp[jn];
+      hi_n = yrp[jn + 1];
+    }
+    if (p + 2 < pe) jn = xci[p + 2];
     if (hi - lo <= 8) {
       // short Y rows (prolongators): all candidates loaded at once, one
       // memory round trip instead of a chain of dependent probes
@@ -673,9 +683,18 @@ spgemm_numeric_rs_kernel(const int* __restrict__ xrp, const int* __restrict__ xc
     for (int i = lane; i < wn * MN; i += 32) acc[i] = Ar::zero();
     __syncwarp();
     const int clo = wcols[0], chi = wcols[wn - 1];
-    for (int p = xs + p0; p < xe; p += pstep) {
-      const int j = xci[p];
-      int qs = yrp[j], qe = yrp[j + 1];
+    // the next X entry's column and Y row ahead, as above
+    int p = xs + p0;
+    int jn = p < xe ? xci[p] : 0;
+    int qs_n = p < xe ? yrp[jn] : 0, qe_n = p < xe ? yrp[jn + 1] : 0;
+    jn = p + pstep < xe ? xci[p + pstep] : 0;
+    for (; p < xe; p += pstep) {
+      int qs = qs_n, qe = qe_n;
+      if (p + pstep < xe) {
+        qs_n = yrp[jn];
+        qe_n = yrp[jn + 1];
+      }
+      if (p + 2 * pstep < xe) jn = xci[p + 2 * pstep];
       if (upper || wn < ce - cs) {
         // restrict Y's row to the window's column range: the warp reads the
         // (short, sorted) row 32 columns at a time and ballots, one memory
