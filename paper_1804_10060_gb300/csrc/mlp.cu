@@ -42,7 +42,8 @@ struct tam_mlp_s {
 namespace tam {
 namespace {
 
-constexpr int ROWS = 64;   // rows of the activation tile per block
+constexpr int ROWS = 128;  // rows of the activation tile per block
+constexpr int DENSE_THREADS = 512;
 constexpr int THREADS = 256;
 
 // Two FP32 multiply-adds in one instruction (each rounded as fmaf's): the FP32
@@ -60,36 +61,65 @@ __device__ __forceinline__ void fma2(float2& acc, float2 a, float2 b) {
 // 3 backward through tanh: out = (A W^T) * (1 - H^2) with H = `aux`.
 // STD: standardise A on load with (a - shift) * scale.
 //
-// Bound by the FP32 pipe: a 64-row tile of the activations and the whole
+// Bound by the FP32 pipe: a 128-row tile of the activations and the whole
 // weight matrix (zero-padded to Kp x Np) sit in shared memory, and each of the
-// 256 threads keeps a TM x TN tile of outputs in registers, so that four
+// 512 threads keeps a TM x TN tile of outputs in registers, so that four
 // steps of k cost TM + TN 16-byte shared loads for 4 TM TN multiply-adds (the
 // kernel before, one row by 8 outputs a thread with scalar loads and a bounds
 // test per product, spent nine loads on eight products).  Threads: NG column
-// groups x 256 / NG row groups, a warp 8 x 4 of them, so that its weight reads
+// groups x 512 / NG row groups, a warp 8 x 4 of them, so that its weight reads
 // are 128 bytes; a thread's rows are its group's number plus multiples of the
-// group count, which keeps a warp's row reads on different banks.  Two blocks fit an SM and hide each other's loads.  Each output sums
-// its products in increasing k.  The 8-128-128-128-3 network on 468,864 rows:
-// 8.74 -> 1.14 ms (28 TFLOP/s of 76.8).
+// group count, which keeps a warp's row reads on different banks.  The next
+// tile is copied while this one is multiplied, one barrier a tile (two blocks
+// of 256 threads an SM, each loading and then multiplying 64 rows: 1.09 ms).
+// Each output sums its products in increasing k.  The 8-128-128-128-3 network
+// on 468,864 rows: 8.74 -> 1.03 ms (31 TFLOP/s of 76.8).
 template <int MODE, bool TRANS, bool STD, int TM, int TN, int NG>
-__global__ void __launch_bounds__(THREADS, 2)
+__global__ void __launch_bounds__(DENSE_THREADS, 1)
 dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float* __restrict__ W,
              const float* __restrict__ bias, const float* __restrict__ shift, const float* __restrict__ scale,
              const float* __restrict__ out_scale, const float* __restrict__ aux, float* __restrict__ out, bool a_vec,
              bool o_vec) {
-  constexpr int RG = THREADS / NG, Np = NG * TN;
+  constexpr int RG = DENSE_THREADS / NG, Np = NG * TN;
   static_assert(RG * TM == ROWS && (TN == 1 || TN == 4 || TN == 8), "dense_kernel: tile");
   extern __shared__ __align__(16) float sm[];
   const int Kp = (K + 3) & ~3, lda = Kp + 4;
   float* Ws = sm;                     // [Kp][Np]
-  float* As = sm + (size_t)Kp * Np;   // [ROWS][lda]
+  float* As = sm + (size_t)Kp * Np;   // two buffers of [ROWS][lda]
+  // the tile of rows r0 .. into buffer b (asynchronously where it is copied as it is)
+  auto fetch = [&](long long r0, int b) {
+    float* dst = As + (size_t)b * ROWS * lda;
+    if (a_vec && !STD) {
+      const int q = K >> 2;  // K = Kp: whole 16-byte groups
+      for (int e = threadIdx.x; e < ROWS * q; e += DENSE_THREADS) {
+        const int r = e / q, k = (e - r * q) * 4;
+        const bool in = r0 + r < n;
+        const unsigned to = (unsigned)__cvta_generic_to_shared(dst + r * lda + k);
+        const float* from = A + (in ? (r0 + r) * K + k : 0);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(in ? 16 : 0));
+      }
+    } else {
+      for (int e = threadIdx.x; e < ROWS * Kp; e += DENSE_THREADS) {
+        const int r = e / Kp, k = e - r * Kp;
+        float a = 0.f;
+        if (r0 + r < n && k < K) {
+          a = A[(r0 + r) * K + k];
+          if (STD) a = (a - shift[k]) * scale[k];
+        }
+        dst[r * lda + k] = a;
+      }
+    }
+  };
+  long long r0 = (long long)blockIdx.x * ROWS;
+  const long long stride = (long long)gridDim.x * ROWS;
+  if (r0 < n) fetch(r0, 0);
   if (TRANS) {
-    for (int e = threadIdx.x; e < Kp * Np; e += THREADS) Ws[e] = 0.f;
+    for (int e = threadIdx.x; e < Kp * Np; e += DENSE_THREADS) Ws[e] = 0.f;
     __syncthreads();
     // a warp transposes 8 rows x 4 groups of 4 columns: 8 lines per read, 4
     // lanes per bank and write
     const int kq = (K + 3) >> 2, jb = (N + 7) >> 3, kb = (kq + 3) >> 2;
-    for (int t = threadIdx.x >> 5; t < jb * kb; t += THREADS / 32) {
+    for (int t = threadIdx.x >> 5; t < jb * kb; t += DENSE_THREADS / 32) {
       const int j = (t % jb) * 8 + (threadIdx.x & 7), k = ((t / jb) * 4 + ((threadIdx.x & 31) >> 3)) * 4;
       if (j < N)
 #pragma unroll
@@ -97,7 +127,7 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
           if (k + q < K) Ws[(k + q) * Np + j] = W[(size_t)j * K + k + q];
     }
   } else {
-    for (int e = threadIdx.x; e < Kp * Np; e += THREADS) {
+    for (int e = threadIdx.x; e < Kp * Np; e += DENSE_THREADS) {
       const int k = e / Np, j = e - k * Np;
       Ws[e] = (k < K && j < N) ? W[(size_t)k * N + j] : 0.f;
     }
@@ -106,34 +136,11 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
   constexpr int CW = NG < 8 ? NG : 8, NW = NG / CW;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int cg = lane % CW + CW * (wid % NW), rg = lane / CW + (32 / CW) * (wid / NW);
-  for (long long r0 = (long long)blockIdx.x * ROWS; r0 < n; r0 += (long long)gridDim.x * ROWS) {
-    __syncthreads();
-    if (a_vec) {
-      const int q = K >> 2;  // K = Kp: whole 16-byte groups
-      for (int e = threadIdx.x; e < ROWS * q; e += THREADS) {
-        const int r = e / q, k = (e - r * q) * 4;
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r0 + r < n) a = *reinterpret_cast<const float4*>(A + (r0 + r) * K + k);
-        if (STD) {
-          a.x = (a.x - shift[k]) * scale[k];
-          a.y = (a.y - shift[k + 1]) * scale[k + 1];
-          a.z = (a.z - shift[k + 2]) * scale[k + 2];
-          a.w = (a.w - shift[k + 3]) * scale[k + 3];
-        }
-        *reinterpret_cast<float4*>(As + r * lda + k) = a;
-      }
-    } else {
-      for (int e = threadIdx.x; e < ROWS * Kp; e += THREADS) {
-        const int r = e / Kp, k = e - r * Kp;
-        float a = 0.f;
-        if (r0 + r < n && k < K) {
-          a = A[(r0 + r) * K + k];
-          if (STD) a = (a - shift[k]) * scale[k];
-        }
-        As[r * lda + k] = a;
-      }
-    }
-    __syncthreads();
+  for (int b = 0; r0 < n; r0 += stride, b ^= 1) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();  // this tile is in place, and the other buffer's readers are done
+    if (r0 + stride < n) fetch(r0 + stride, b ^ 1);
+    const float* Ab = As + (size_t)b * ROWS * lda;
     constexpr int TP = (TN + 1) / 2;  // output pairs (TN = 1: the second half idle)
     float2 acc[TM][TP];
 #pragma unroll
@@ -144,7 +151,7 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
       float av[TM][4];
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
-        const float4 a = *reinterpret_cast<const float4*>(As + (rg + i * RG) * lda + k);
+        const float4 a = *reinterpret_cast<const float4*>(Ab + (rg + i * RG) * lda + k);
         av[i][0] = a.x;
         av[i][1] = a.y;
         av[i][2] = a.z;
@@ -644,11 +651,12 @@ template <int MODE, bool TRANS, bool STD, int TM, int TN, int NG>
 void dense_launch(const float* A, long long n, int K, int N, const float* W, const float* bias, const tam_mlp_s* M,
                   const float* aux, float* out, cudaStream_t s) {
   const int Kp = (K + 3) & ~3;
-  const size_t smem = sizeof(float) * ((size_t)Kp * NG * TN + (size_t)ROWS * (Kp + 4));
+  const size_t smem = sizeof(float) * ((size_t)Kp * NG * TN + 2 * (size_t)ROWS * (Kp + 4));
   auto kern = dense_kernel<MODE, TRANS, STD, TM, TN, NG>;
   TAM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<row_grid(n, ROWS), THREADS, smem, s>>>(A, n, K, N, W, bias, M->shift.p, M->scale.p, M->out_scale.p, aux, out,
-                                                K % 4 == 0 && aligned16(A), N % 4 == 0 && aligned16(out));
+  const unsigned grid = (unsigned)std::min<long long>((n + ROWS - 1) / ROWS, sm_count());
+  kern<<<grid, DENSE_THREADS, smem, s>>>(A, n, K, N, W, bias, M->shift.p, M->scale.p, M->out_scale.p, aux, out,
+                                         K % 4 == 0 && aligned16(A), N % 4 == 0 && aligned16(out));
   TAM_LAUNCH_CHECK();
 }
 
