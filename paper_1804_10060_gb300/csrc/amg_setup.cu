@@ -579,7 +579,7 @@ __global__ void dense_inactive_kernel(double* __restrict__ D, int N, int ld, uns
 //      the rest, so the next panel starts with its P known.
 // Two grid-wide barriers per panel (three, and FP64 products with two global
 // loads each, before: the unit cube's 3,993-DOF solve, whose coarsest level
-// this inverts, 12.2 -> 5.0 ms in all).  Bound by the FP64 pipe (N^3 or, for SYM,
+// this inverts, 12.2 -> 4.4 ms in all).  Bound by the FP64 pipe (N^3 or, for SYM,
 // N^3 / 2 multiply-adds at 2 per cycle and SM) once N is large, by the GJB
 // dependent pivots (about 9 us a panel) and the barriers below N ~ 500.
 // SYM: a symmetric matrix; only tiles on or below the diagonal are kept.  An
@@ -670,55 +670,98 @@ gj_coop_kernel(double* __restrict__ D, int ld, double* __restrict__ cpan, double
       __syncthreads();
     }
     grid.sync();
-    // 2. half tiles (I, J): the rest, the new column panel (J = K) and row panel (I = K)
-    auto half_tile = [&](int I, int J, int h) {
+    // 2. half tiles (I, J): the rest, the new column panel (J = K) and row panel
+    // (I = K).  A tile's factors and values are requested while the tile
+    // before it is multiplied (an L2 round trip of 1 us beside 4 us of FP64).
+    double fa[4], fb[2], v0 = 0.0, v1 = 0.0;  // a half tile on its way in
+    auto request = [&](int I, int J, int h) {
       const int i0 = I * GJB, j0 = J * GJB + h * GJ_COLS;
-      double* __restrict__ out = D + (size_t)(i0 + r) * ld + j0 + c;
-      if (I == K) {
-        out[0] = rpan[(size_t)r * ld + j0 + c];
-        out[(size_t)GJ_COLS * ld] = rpan[(size_t)(r + GJ_COLS) * ld + j0 + c];
-        return;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) fa[q] = cpan[(size_t)i0 * GJB + threadIdx.x + q * GJ_THREADS];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int e = threadIdx.x + q * GJ_THREADS, k = e / GJ_COLS, j = e % GJ_COLS;
+        fb[q] = J == K ? sp[k][h * GJ_COLS + j] : rpan[(size_t)k * ld + j0 + j];
       }
-      for (int e = threadIdx.x; e < GJB * GJB; e += GJ_THREADS) sa[e / GJB][e % GJB] = cpan[(size_t)i0 * GJB + e];
-      for (int e = threadIdx.x; e < GJB * GJ_COLS; e += GJ_THREADS) {
-        const int k = e / GJ_COLS, j = e % GJ_COLS;
-        sb[k][j] = J == K ? sp[k][h * GJ_COLS + j] : rpan[(size_t)k * ld + j0 + j];
+      const double* __restrict__ from = D + (size_t)(i0 + r) * ld + j0 + c;
+      v0 = J == K ? 0.0 : from[0];
+      v1 = J == K ? 0.0 : from[(size_t)GJ_COLS * ld];
+    };
+    auto place = [&]() {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int e = threadIdx.x + q * GJ_THREADS;
+        sa[e / GJB][e % GJB] = fa[q];
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int e = threadIdx.x + q * GJ_THREADS;
+        sb[e / GJ_COLS][e % GJ_COLS] = fb[q];
       }
       __syncthreads();
-      double v0 = J == K ? 0.0 : out[0], v1 = J == K ? 0.0 : out[(size_t)GJ_COLS * ld];
+    };
+    auto multiply = [&](int I, int J, int h, double w0, double w1) {
 #pragma unroll 8
       for (int k = 0; k < GJB; ++k) {
         const double x = sb[k][c];
-        v0 = fma(-sa[r][k], x, v0);
-        v1 = fma(-sa[r + GJ_COLS][k], x, v1);
+        w0 = fma(-sa[r][k], x, w0);
+        w1 = fma(-sa[r + GJ_COLS][k], x, w1);
       }
-      out[0] = v0;
-      out[(size_t)GJ_COLS * ld] = v1;
+      double* __restrict__ out = D + (size_t)(I * GJB + r) * ld + J * GJB + h * GJ_COLS + c;
+      out[0] = w0;
+      out[(size_t)GJ_COLS * ld] = w1;
       __syncthreads();
     };
     if ((int)blockIdx.x >= first) {
       // items by row of tiles: SYM keeps J <= I
       const int stride = gridDim.x - first;
-      int item = blockIdx.x - first;
-      for (int I = 0; I < t; ++I) {
-        const int cnt = 2 * (SYM ? I + 1 : t);
-        for (; item < cnt; item += stride) {
-          const int J = item >> 1;
-          if (J == K && I == K) continue;
-          if (first && I == K + 1 && J == K + 1) continue;  // block 0's
-          half_tile(I, J, item & 1);
+      int I = 0, item = blockIdx.x - first;
+      // the block's next half tile to multiply (row panel copies done on the way); false at the end
+      auto next = [&](int& ti, int& tj, int& th) {
+        for (; I < t; ++I) {
+          const int cnt = 2 * (SYM ? I + 1 : t);
+          while (item < cnt) {
+            const int J = item >> 1, h = item & 1;
+            item += stride;
+            if (J == K && I == K) continue;
+            if (first && I == K + 1 && J == K + 1) continue;  // block 0's
+            if (I == K) {
+              const int j = J * GJB + h * GJ_COLS + c;
+              D[(size_t)(k0 + r) * ld + j] = rpan[(size_t)r * ld + j];
+              D[(size_t)(k0 + r + GJ_COLS) * ld + j] = rpan[(size_t)(r + GJ_COLS) * ld + j];
+              continue;
+            }
+            ti = I;
+            tj = J;
+            th = h;
+            return true;
+          }
+          item -= cnt;
         }
-        item -= cnt;
+        return false;
+      };
+      int ti = 0, tj = 0, th = 0;
+      bool have = next(ti, tj, th);
+      if (have) request(ti, tj, th);
+      while (have) {
+        place();
+        const int ci = ti, cj = tj, ch = th;
+        const double w0 = v0, w1 = v1;
+        have = next(ti, tj, th);
+        if (have) request(ti, tj, th);
+        multiply(ci, cj, ch, w0, w1);
       }
     }
     if (blockIdx.x == 0) {
       for (int e = threadIdx.x; e < GJB * GJB; e += GJ_THREADS)
         D[(size_t)(k0 + e / GJB) * ld + k0 + e % GJB] = sp[e / GJB][e % GJB];
       if (K + 1 < t) {
-        if (first) {
-          half_tile(K + 1, K + 1, 0);
-          half_tile(K + 1, K + 1, 1);
-        }
+        if (first)
+          for (int h = 0; h < 2; ++h) {
+            request(K + 1, K + 1, h);
+            place();
+            multiply(K + 1, K + 1, h, v0, v1);
+          }
         __syncthreads();
         gj_invert_tile(D + (size_t)(k0 + GJB) * ld + k0 + GJB, ld, P, bad);
       }
@@ -978,7 +1021,9 @@ static void coarse_inverse(tam_amg_s* H, const Level& L, bool sym, cudaStream_t 
   DBuf<int> bad(1, s);
   bad.zero();
   // all panels in one cooperative launch (grid-wide barriers between the
-  // steps of a panel), one block per SM
+  // steps of a panel), one block per SM (two: 2.08 ms against 1.80 on the unit
+  // cube's coarsest level, the barriers cost more than the overlap gains; 1.57
+  // with the next half tile requested ahead)
   const void* kern = sym ? (const void*)gj_coop_kernel<true> : (const void*)gj_coop_kernel<false>;
   int per_sm = 0;
   TAM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GJ_THREADS, 0));
