@@ -129,14 +129,17 @@ struct EpiLanczos {
   __device__ bool skip() const { return *done; }
   __device__ void operator()(int row, const double (&acc)[BR], double* sh) const {
     double dot[1] = {0.0};
-    if (row < n_rows)
+    if (row < n_rows) {
+      double wr[BR];  // all loads ahead of the stores
 #pragma unroll
       for (int r = 0; r < BR; ++r) {
-        size_t i = (size_t)row * BR + r;
-        double wi = s[i] * acc[r];
-        w[i] = wi;
-        dot[0] += wi * v[i];
+        const size_t i = (size_t)row * BR + r;
+        wr[r] = s[i] * acc[r];
+        dot[0] += wr[r] * v[i];
       }
+#pragma unroll
+      for (int r = 0; r < BR; ++r) w[(size_t)row * BR + r] = wr[r];
+    }
     double tot[1];
     if (grid_reduce<1>(gr, dot, tot, sh) && threadIdx.x == 0) *alpha_out = tot[0];
   }

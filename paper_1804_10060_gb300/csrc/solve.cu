@@ -55,13 +55,28 @@ struct EpiCheb {
   __device__ void operator()(int row, const double (&acc)[BR], double*) const {
     if (row >= n_rows) return;
     const double cd = coef[0], cr = coef[1];
+    const size_t i0 = (size_t)row * BR;
+    // the row's operands first: behind the stores of d and xn (which may alias
+    // them, as far as the compiler can tell) each load would wait for the last
+    double v[BR], dv[BR], xv[BR];
 #pragma unroll
     for (int r = 0; r < BR; ++r) {
-      size_t i = (size_t)row * BR + r;
-      double res = dinv[i] * (b[i] - acc[r]);
-      double di = cd != 0.0 ? cd * d[i] + cr * res : cr * res;
-      d[i] = di;
-      xn[i] = x[i] + di;
+      v[r] = dinv[i0 + r] * (b[i0 + r] - acc[r]);
+      xv[r] = x[i0 + r];
+    }
+    if (cd != 0.0) {
+#pragma unroll
+      for (int r = 0; r < BR; ++r) dv[r] = d[i0 + r];
+#pragma unroll
+      for (int r = 0; r < BR; ++r) dv[r] = cd * dv[r] + cr * v[r];
+    } else {
+#pragma unroll
+      for (int r = 0; r < BR; ++r) dv[r] = cr * v[r];
+    }
+#pragma unroll
+    for (int r = 0; r < BR; ++r) {
+      d[i0 + r] = dv[r];
+      xn[i0 + r] = xv[r] + dv[r];
     }
   }
 };
@@ -143,14 +158,16 @@ struct EpiInitResidual {
   __device__ bool skip() const { return false; }
   __device__ void operator()(int row, const double (&acc)[BR], double* sh) const {
     double s[1] = {0.0};
-    if (row < n_rows)
+    if (row < n_rows) {
+      double v[BR];
 #pragma unroll
       for (int k = 0; k < BR; ++k) {
-        size_t i = (size_t)row * BR + k;
-        double v = b[i] - acc[k];
-        r[i] = v;
-        s[0] += v * v;
+        v[k] = b[(size_t)row * BR + k] - acc[k];
+        s[0] += v[k] * v[k];
       }
+#pragma unroll
+      for (int k = 0; k < BR; ++k) r[(size_t)row * BR + k] = v[k];
+    }
     double tot[1];
     if (grid_reduce<1>(gr, s, tot, sh) && threadIdx.x == 0) {
       sc->rr = tot[0];
@@ -195,11 +212,10 @@ struct EpiPq {
     double s[1] = {0.0};
     if (row < n_rows)
 #pragma unroll
-      for (int k = 0; k < BR; ++k) {
-        size_t i = (size_t)row * BR + k;
-        q[i] = acc[k];
-        s[0] += p[i] * acc[k];
-      }
+      for (int k = 0; k < BR; ++k) s[0] += p[(size_t)row * BR + k] * acc[k];
+    if (row < n_rows)
+#pragma unroll
+      for (int k = 0; k < BR; ++k) q[(size_t)row * BR + k] = acc[k];
     double tot[1];
     if (grid_reduce<1>(gr, s, tot, sh) && threadIdx.x == 0) {
       const double pq = tot[0];

@@ -1358,9 +1358,12 @@ struct EpiAdd {
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
   __device__ void operator()(int row, const double (&acc)[BR], double*) const {
-    if (row < n_rows)
+    if (row >= n_rows) return;
+    double v[BR];  // all loads ahead of the stores
 #pragma unroll
-      for (int r = 0; r < BR; ++r) y[(size_t)row * BR + r] += acc[r];
+    for (int r = 0; r < BR; ++r) v[r] = y[(size_t)row * BR + r];
+#pragma unroll
+    for (int r = 0; r < BR; ++r) y[(size_t)row * BR + r] = v[r] + acc[r];
   }
 };
 
@@ -1373,12 +1376,12 @@ struct EpiResidual {
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
   __device__ void operator()(int row, const double (&acc)[BR], double*) const {
-    if (row < n_rows)
+    if (row >= n_rows) return;
+    double v[BR];  // all loads ahead of the stores
 #pragma unroll
-      for (int r = 0; r < BR; ++r) {
-        size_t i = (size_t)row * BR + r;
-        t[i] = b[i] - acc[r];
-      }
+    for (int r = 0; r < BR; ++r) v[r] = b[(size_t)row * BR + r];
+#pragma unroll
+    for (int r = 0; r < BR; ++r) t[(size_t)row * BR + r] = v[r] - acc[r];
   }
 };
 
