@@ -66,6 +66,12 @@ struct Level {
   DBuf<__nv_bfloat16> A16v;
   SpOpLow<float> A32, P32, R32;
   SpOpLow<__nv_bfloat16> A16;
+  // the batched solve's operators: the same copies, or block-CSR-ordered ones
+  // of its own where the solve's follow a lanes-per-row store
+  DBuf<float> A32mv, P32mv, R32mv;
+  DBuf<__nv_bfloat16> A16mv;
+  SpOpLow<float> A32m, P32m, R32m;
+  SpOpLow<__nv_bfloat16> A16m;
 };
 
 // Multi-right-hand-side solve state (block of independent CGs sharing every
@@ -171,6 +177,8 @@ void vcycle_apply(tam_amg_s* H, const double* r, double* z, const int* stop, cud
 // level 0 and FP64 dense coarsest solve), and its set-up after amg_build.
 void vcycle_apply_low(tam_amg_s* H, const double* r, double* z, const int* stop, cudaStream_t s);
 void build_low_precision(tam_amg_s* H, cudaStream_t s);
+// The batched solve's operators, after build_low_precision.
+void build_batch_operators(tam_amg_s* H, cudaStream_t s);
 // x <- degree Chebyshev-Jacobi steps on K x = b from x over [lo, hi] * lambda_max(D^-1 K)
 void smooth_fine(tam_amg_s* H, const double* b, double* x, int degree, double lo, double hi, cudaStream_t s);
 

@@ -751,8 +751,8 @@ __global__ void mcoarse_kernel(const double* __restrict__ A, const TI* __restric
 // A x on a level with its FP32 / BF16 values
 template <int BS, class Epi>
 void level_mspmm(const Level& L, const float* x, int mp, const MTile& t, Epi epi, cudaStream_t s) {
-  if (L.A16.vals) mspmm<BS, BS, __nv_bfloat16>(L.A16, x, mp, t, epi, s);
-  else mspmm<BS, BS, float>(L.A32, x, mp, t, epi, s);
+  if (L.A16m.vals) mspmm<BS, BS, __nv_bfloat16>(L.A16m, x, mp, t, epi, s);
+  else mspmm<BS, BS, float>(L.A32m, x, mp, t, epi, s);
 }
 
 template <typename TB, typename TO>
@@ -774,17 +774,17 @@ void mresidual(const Level& L, const MultiLevel& ML, const TB* b, const float* x
 
 void mrestrict(const Level& L, const MultiLevel& ML, float* bc, int mp, const int* stop, cudaStream_t s) {
   const int nr = L.R.n_rows;
-  if (L.kdim == 6 && L.bs == 3) mspmm<6, 3, float>(L.R32, ML.t.p, mp, ML.tR, EpiPutMF<6, false>{bc, nr, mp, stop}, s);
-  else if (L.kdim == 6) mspmm<6, 6, float>(L.R32, ML.t.p, mp, ML.tR, EpiPutMF<6, false>{bc, nr, mp, stop}, s);
-  else mspmm<3, 3, float>(L.R32, ML.t.p, mp, ML.tR, EpiPutMF<3, false>{bc, nr, mp, stop}, s);
+  if (L.kdim == 6 && L.bs == 3) mspmm<6, 3, float>(L.R32m, ML.t.p, mp, ML.tR, EpiPutMF<6, false>{bc, nr, mp, stop}, s);
+  else if (L.kdim == 6) mspmm<6, 6, float>(L.R32m, ML.t.p, mp, ML.tR, EpiPutMF<6, false>{bc, nr, mp, stop}, s);
+  else mspmm<3, 3, float>(L.R32m, ML.t.p, mp, ML.tR, EpiPutMF<3, false>{bc, nr, mp, stop}, s);
 }
 
 void mprolong(const Level& L, const MultiLevel& ML, const float* xc, float* x, int mp, const int* stop,
               cudaStream_t s) {
   const int nr = L.P.n_rows;
-  if (L.kdim == 6 && L.bs == 3) mspmm<3, 6, float>(L.P32, xc, mp, ML.tP, EpiPutMF<3, true>{x, nr, mp, stop}, s);
-  else if (L.kdim == 6) mspmm<6, 6, float>(L.P32, xc, mp, ML.tP, EpiPutMF<6, true>{x, nr, mp, stop}, s);
-  else mspmm<3, 3, float>(L.P32, xc, mp, ML.tP, EpiPutMF<3, true>{x, nr, mp, stop}, s);
+  if (L.kdim == 6 && L.bs == 3) mspmm<3, 6, float>(L.P32m, xc, mp, ML.tP, EpiPutMF<3, true>{x, nr, mp, stop}, s);
+  else if (L.kdim == 6) mspmm<6, 6, float>(L.P32m, xc, mp, ML.tP, EpiPutMF<6, true>{x, nr, mp, stop}, s);
+  else mspmm<3, 3, float>(L.P32m, xc, mp, ML.tP, EpiPutMF<3, true>{x, nr, mp, stop}, s);
 }
 
 template <typename TB, typename TO>
@@ -895,21 +895,21 @@ void autotune(tam_amg_s* H, cudaStream_t s) {
     Level& L = H->levels[l];
     MultiLevel& ML = MS.lv[l];
     MultiLevel& MC = MS.lv[l + 1];
-    ML.tA = pick_tile(mp, L.A32.op.lpr, [&](const MTile& t) {
+    ML.tA = pick_tile(mp, L.A32m.op.lpr, [&](const MTile& t) {
       if (L.bs == 3) level_mspmm<3>(L, ML.xa.p, mp, t, EpiPutMF<3, false>{ML.t.p, L.n_rows, mp, nullptr}, s);
       else level_mspmm<6>(L, ML.xa.p, mp, t, EpiPutMF<6, false>{ML.t.p, L.n_rows, mp, nullptr}, s);
     }, s);
-    ML.tR = pick_tile(mp, L.R32.op.lpr, [&](const MTile& t) {
+    ML.tR = pick_tile(mp, L.R32m.op.lpr, [&](const MTile& t) {
       const int nr = L.R.n_rows;
-      if (L.kdim == 6 && L.bs == 3) mspmm<6, 3, float>(L.R32, ML.t.p, mp, t, EpiPutMF<6, false>{MC.b.p, nr, mp, nullptr}, s);
-      else if (L.kdim == 6) mspmm<6, 6, float>(L.R32, ML.t.p, mp, t, EpiPutMF<6, false>{MC.b.p, nr, mp, nullptr}, s);
-      else mspmm<3, 3, float>(L.R32, ML.t.p, mp, t, EpiPutMF<3, false>{MC.b.p, nr, mp, nullptr}, s);
+      if (L.kdim == 6 && L.bs == 3) mspmm<6, 3, float>(L.R32m, ML.t.p, mp, t, EpiPutMF<6, false>{MC.b.p, nr, mp, nullptr}, s);
+      else if (L.kdim == 6) mspmm<6, 6, float>(L.R32m, ML.t.p, mp, t, EpiPutMF<6, false>{MC.b.p, nr, mp, nullptr}, s);
+      else mspmm<3, 3, float>(L.R32m, ML.t.p, mp, t, EpiPutMF<3, false>{MC.b.p, nr, mp, nullptr}, s);
     }, s);
-    ML.tP = pick_tile(mp, L.P32.op.lpr, [&](const MTile& t) {
+    ML.tP = pick_tile(mp, L.P32m.op.lpr, [&](const MTile& t) {
       const int nr = L.P.n_rows;
-      if (L.kdim == 6 && L.bs == 3) mspmm<3, 6, float>(L.P32, MC.y.p, mp, t, EpiPutMF<3, false>{ML.xb.p, nr, mp, nullptr}, s);
-      else if (L.kdim == 6) mspmm<6, 6, float>(L.P32, MC.y.p, mp, t, EpiPutMF<6, false>{ML.xb.p, nr, mp, nullptr}, s);
-      else mspmm<3, 3, float>(L.P32, MC.y.p, mp, t, EpiPutMF<3, false>{ML.xb.p, nr, mp, nullptr}, s);
+      if (L.kdim == 6 && L.bs == 3) mspmm<3, 6, float>(L.P32m, MC.y.p, mp, t, EpiPutMF<3, false>{ML.xb.p, nr, mp, nullptr}, s);
+      else if (L.kdim == 6) mspmm<6, 6, float>(L.P32m, MC.y.p, mp, t, EpiPutMF<6, false>{ML.xb.p, nr, mp, nullptr}, s);
+      else mspmm<3, 3, float>(L.P32m, MC.y.p, mp, t, EpiPutMF<3, false>{ML.xb.p, nr, mp, nullptr}, s);
     }, s);
   }
   MS.tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -917,6 +917,7 @@ void autotune(tam_amg_s* H, cudaStream_t s) {
 
 void ensure_multi(tam_amg_s* H, int mp, cudaStream_t s) {
   if (!H->levels[0].dinv32.p) build_low_precision(H, s);
+  if (!H->levels[0].A32m.vals && !H->levels[0].A16m.vals) build_batch_operators(H, s);
   if (H->multi && H->multi->mp == mp) return;
   static std::atomic<unsigned long long> serials{0};
   H->multi.reset(new MultiState());

@@ -1201,33 +1201,38 @@ __global__ void convert_kernel(const double* __restrict__ in, T* __restrict__ ou
     round_to(in[i], out[i]);
 }
 
-// SELL values (element-major slots) into packed slots
+// Slots (or groups) of `width` blocks, element-major, into packed ones
 template <typename T>
-__global__ void convert_slots_kernel(const double* __restrict__ in, T* __restrict__ out, long long n, int bb) {
-  const int slot = 32 * bb;
+__global__ void convert_slots_kernel(const double* __restrict__ in, T* __restrict__ out, long long n, int bb, int width) {
+  const int slot = width * bb;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const long long s0 = i / slot * slot;
     const int r = (int)(i - s0);
-    round_to(in[i], out[s0 + pack_pos(pack_of(sizeof(T)), 32, bb, r >> 5, r & 31)]);
+    round_to(in[i], out[s0 + pack_pos(pack_of(sizeof(T), width, bb), width, bb, r / width, r % width)]);
   }
 }
 
 template <typename T>
-void convert_values(const SpOp& op, DBuf<T>& out, cudaStream_t s) {
-  const bool sell = op.lpr == 0;
-  const int bb = sell ? op.S->br * op.S->bc : (int)op.B->block_elems();
-  const long long n = (sell ? op.S->n_slots * 32 : op.B->nnzb) * (long long)bb;
+void convert_values(const SpOp& op, DBuf<T>& out, cudaStream_t s, bool batch) {
+  const bool store = !batch && low_in_store(op);
+  const int bb = (int)op.B->block_elems();
+  const long long blocks = op.lpr == 0 ? op.S->n_slots * 32 : (store ? op.L->n_groups * op.L->lpr : op.B->nnzb);
+  const long long n = blocks * bb;
   out = DBuf<T>((size_t)std::max(1LL, n), s);
   if (n <= 0) return;
-  if (sell) convert_slots_kernel<T><<<stride_grid(n, 256, 16), 256, 0, s>>>(op.S->vals.p, out.p, n, bb);
-  else convert_kernel<T><<<stride_grid(n, 256, 16), 256, 0, s>>>(op.B->vals.p, out.p, n);
+  const unsigned g = stride_grid(n, 256, 16);
+  if (op.lpr == 0) convert_slots_kernel<T><<<g, 256, 0, s>>>(op.S->vals.p, out.p, n, bb, 32);
+  else if (store) convert_slots_kernel<T><<<g, 256, 0, s>>>(op.L->vals.p, out.p, n, bb, op.L->lpr);
+  else convert_kernel<T><<<g, 256, 0, s>>>(op.B->vals.p, out.p, n);
   TAM_LAUNCH_CHECK();
 }
 }  // namespace
 
-void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s) { convert_values<float>(op, out, s); }
-void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s) {
-  convert_values<__nv_bfloat16>(op, out, s);
+void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s, bool batch) {
+  convert_values<float>(op, out, s, batch);
+}
+void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s, bool batch) {
+  convert_values<__nv_bfloat16>(op, out, s, batch);
 }
 
 }  // namespace tam

@@ -183,8 +183,12 @@ struct Sell {
 // for one request (16 bytes: W = 2 float2, 4 float, 8 BF16): pack q of block j
 // at [(q * width + j) * W], the elements left over after the whole packs one by
 // one behind them.  Element by element a 3 x 3 slot took nine requests, and the
-// FP32 kernels stalled on the load queue rather than on memory.
-__host__ __device__ constexpr int pack_of(size_t value_bytes) { return (int)(16 / value_bytes); }
+// FP32 kernels stalled on the load queue rather than on memory.  A slot whose
+// size is not a multiple of 16 bytes (two lanes of 3 x 3 floats: 72) would put
+// every second one off the boundary: it stays element by element (W = 1).
+__host__ __device__ constexpr int pack_of(size_t value_bytes, int width, int bb) {
+  return value_bytes * width * bb % 16 == 0 ? (int)(16 / value_bytes) : 1;
+}
 __host__ __device__ constexpr int pack_pos(int W, int width, int bb, int e, int j) {
   return e < bb / W * W ? (e / W * width + j) * W + e % W : e * width + j;
 }
@@ -192,7 +196,7 @@ __host__ __device__ constexpr int pack_pos(int W, int width, int bb, int e, int 
 // Block j of a slot (or group) of `width` packed blocks.
 template <int BB, int WIDTH, typename V>
 __device__ __forceinline__ void slot_load(const V* __restrict__ slot, int j, V (&out)[BB]) {
-  constexpr int W = pack_of(sizeof(V)), Q = BB / W;
+  constexpr int W = pack_of(sizeof(V), WIDTH, BB), Q = W > 1 ? BB / W : 0;
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const float4 v = __ldg(reinterpret_cast<const float4*>(slot) + q * WIDTH + j);
@@ -1293,19 +1297,115 @@ bsr_vector_f32_kernel(int n_rows, const int* __restrict__ rp, const int* __restr
   epi((sub == 0 && row < n_rows) ? row : n_rows, acc, sh);
 }
 
-// A reduced-precision operator: the pattern of `op` with values `vals`
-// (same layout as op's FP64 values: SELL when op.lpr == 0, else Bsr).
+// The lanes-per-row and block-row kernels in FP32: the store and lane mapping
+// of lpr_spmv_kernel and blockrow_spmv_kernel (values packed, x in records).
+// A lane per 6 x 6 block over the block-CSR arrays spreads a warp's request
+// over 32 lines and keeps a lane's chain long; these read whole lines (the
+// 1.38M-DOF P2 disc, 8,416 and 1,280 coarse rows: a Chebyshev step 24 -> 19 and
+// 17 -> 7 us, the prolongation between them 20 -> 12).  The operators of whole-warp rows (restriction to the first
+// coarse level: 2,100 rows of hundreds of 6 x 3 blocks) stay on the block-CSR
+// arrays, a warp per row: 36 us against 52 through the 8-lane store, whose
+// FP64 form is bound by arithmetic instead.
+template <int BR, int BC, int LPR, typename TV, class Epi>
+__global__ void __launch_bounds__(SPMV_THREADS)
+lpr_spmv_f32_kernel(int n_rows, const int* __restrict__ gp, const int* __restrict__ cols, const TV* __restrict__ v,
+                    const float* __restrict__ x, Epi epi) {
+  __shared__ double sh[32];
+  if (epi.skip()) return;
+  constexpr int BB = BR * BC;
+  const int t = blockIdx.x * SPMV_THREADS + threadIdx.x;
+  const int row = t / LPR, sub = t % LPR;
+  float acc[BR];
+#pragma unroll
+  for (int r = 0; r < BR; ++r) acc[r] = 0.f;
+  if (row < n_rows) {
+    const int g0 = gp[row], g1 = gp[row + 1];
+    float xn[BC];  // the gather runs one group ahead
+    if (g0 < g1) gather_f32<BC>(x, __ldg(cols + (size_t)g0 * LPR + sub), xn);
+    for (int g = g0; g < g1; ++g) {
+      TV vv[BB];
+      slot_load<BB, LPR>(v + (size_t)g * BB * LPR, sub, vv);
+      float xv[BC];
+#pragma unroll
+      for (int j = 0; j < BC; ++j) xv[j] = xn[j];
+      if (g + 1 < g1) gather_f32<BC>(x, __ldg(cols + (size_t)(g + 1) * LPR + sub), xn);
+#pragma unroll
+      for (int r = 0; r < BR; ++r)
+#pragma unroll
+        for (int j = 0; j < BC; ++j) acc[r] = fmaf(to_f32(vv[r * BC + j]), xv[j], acc[r]);
+    }
+  }
+#pragma unroll
+  for (int o = LPR / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int r = 0; r < BR; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+  epi((sub == 0 && row < n_rows) ? row : n_rows, acc, sh);
+}
+
+template <int B, int WPR, typename TV, class Epi>
+__global__ void __launch_bounds__(BLOCKROW_THREADS)
+blockrow_f32_kernel(int n_rows, const int* __restrict__ rp, const int* __restrict__ ci, const TV* __restrict__ v,
+                    const float* __restrict__ x, Epi epi) {
+  constexpr int G = 32 / B, W = BLOCKROW_THREADS / 32, RPB = W / WPR, BB = B * B;
+  __shared__ double sh[32];
+  __shared__ float part[W][B];
+  if (epi.skip()) return;  // block-uniform (a device flag)
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = blockIdx.x * RPB + wid / WPR, wr = wid % WPR;
+  const int g = lane / B, r = lane - g * B;
+  float ad = 0.f;
+  if (row < n_rows && g < G) {
+    const int p1 = rp[row + 1];
+    float xn[B];  // the gather runs one step ahead (a group's lanes read one record)
+    int p = rp[row] + wr * G + g;
+    if (p < p1) gather_f32<B>(x, __ldg(ci + p), xn);
+    for (; p < p1; p += WPR * G) {
+      TV vv[B];
+      block_load_low<B>(v + (size_t)p * BB + r * B, vv);
+      float xv[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) xv[j] = xn[j];
+      if (p + WPR * G < p1) gather_f32<B>(x, __ldg(ci + p + WPR * G), xn);
+#pragma unroll
+      for (int j = 0; j < B; ++j) ad = fmaf(to_f32(vv[j]), xv[j], ad);
+    }
+  }
+  // groups of the warp, in order, into lanes 0 .. B-1
+  float sum = ad;
+#pragma unroll
+  for (int gg = 1; gg < G; ++gg) sum += __shfl_sync(0xffffffffu, ad, gg * B + r);
+  if constexpr (WPR > 1) {
+    if (lane < B) part[wid][lane] = sum;
+    __syncthreads();
+    if (wr == 0 && lane < B)
+#pragma unroll
+      for (int w = 1; w < WPR; ++w) sum += part[wid + w][lane];
+  }
+  float acc[B];
+#pragma unroll
+  for (int k = 0; k < B; ++k) acc[k] = __shfl_sync(0xffffffffu, sum, k);
+  epi((wr == 0 && lane == 0 && row < n_rows) ? row : n_rows, acc, sh);
+}
+
+// A reduced-precision operator: the pattern of `op` with values `vals` in the
+// order of the kernel that runs it -- SELL or lanes-per-row store (packed), or
+// the block-CSR arrays.  The batched solve's copies (`batch`) keep block-CSR
+// order wherever the operator is not SELL.
 template <typename TV>
 struct SpOpLow {
   SpOp op;
   const TV* vals = nullptr;
 };
 
+// Whether the values of op's reduced-precision copy follow its lanes-per-row store
+inline bool low_in_store(const SpOp& op) { return op.L && !op.tpr; }
+
 template <int BR, int BC, typename TV, class Epi>
 void spop_apply_f32(const SpOpLow<TV>& o, const float* x, Epi epi, cudaStream_t s) {
-  const unsigned g = spop_grid(o.op);
-  if (o.op.lpr == 0) {
-    const Sell& S = *o.op.S;
+  const SpOp& op = o.op;
+  const unsigned g = spop_grid(op);
+  if (op.lpr == 0) {
+    const Sell& S = *op.S;
     const int split = sell_split(S.n_slices);
     const unsigned grid = grid_for((long long)S.n_slices * 32 * split, SPMV_THREADS);
     if (split == 2)
@@ -1314,9 +1414,31 @@ void spop_apply_f32(const SpOpLow<TV>& o, const float* x, Epi epi, cudaStream_t 
     else
       sell_spmv_f32_kernel<BR, BC, TV, Epi, 1><<<grid, SPMV_THREADS, 0, s>>>(S.n_slices, S.slice_ptr.p, S.cols.p, o.vals,
                                                                              x, S.perm.p, S.n_rows, epi);
+  } else if (op.brw) {
+    const Bsr& B = *op.B;
+    if constexpr (BR == 6 && BC == 6 && std::is_same<TV, float>::value) {
+      const unsigned gb = grid_for(B.n_rows, (BLOCKROW_THREADS / 32) / op.brw);
+      switch (op.brw) {
+        case 1: blockrow_f32_kernel<6, 1, TV, Epi><<<gb, BLOCKROW_THREADS, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, epi); break;
+        case 2: blockrow_f32_kernel<6, 2, TV, Epi><<<gb, BLOCKROW_THREADS, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, epi); break;
+        case 4: blockrow_f32_kernel<6, 4, TV, Epi><<<gb, BLOCKROW_THREADS, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, epi); break;
+        case 8: blockrow_f32_kernel<6, 8, TV, Epi><<<gb, BLOCKROW_THREADS, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, epi); break;
+        default: throw Error(TAM_ERR_INTERNAL, "spmv: block-row lanes need 1, 2, 4 or 8 warps per row");
+      }
+    } else {
+      throw Error(TAM_ERR_INTERNAL, "spmv: FP32 block-row lanes are for 6x6 blocks");
+    }
+  } else if (low_in_store(op)) {
+    const LprStore& L = *op.L;
+    switch (L.lpr) {
+      case 2: lpr_spmv_f32_kernel<BR, BC, 2, TV, Epi><<<g, SPMV_THREADS, 0, s>>>(L.n_rows, L.grp_ptr.p, L.cols.p, o.vals, x, epi); break;
+      case 4: lpr_spmv_f32_kernel<BR, BC, 4, TV, Epi><<<g, SPMV_THREADS, 0, s>>>(L.n_rows, L.grp_ptr.p, L.cols.p, o.vals, x, epi); break;
+      case 8: lpr_spmv_f32_kernel<BR, BC, 8, TV, Epi><<<g, SPMV_THREADS, 0, s>>>(L.n_rows, L.grp_ptr.p, L.cols.p, o.vals, x, epi); break;
+      default: throw Error(TAM_ERR_INTERNAL, "spmv: the lanes-per-row store is for 2, 4 or 8 lanes");
+    }
   } else {
-    const Bsr& B = *o.op.B;
-    switch (o.op.lpr) {
+    const Bsr& B = *op.B;
+    switch (op.lpr) {
       case 2: bsr_vector_f32_kernel<BR, BC, 2, TV, Epi><<<g, SPMV_THREADS, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, epi); break;
       case 4: bsr_vector_f32_kernel<BR, BC, 4, TV, Epi><<<g, SPMV_THREADS, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, epi); break;
       case 8: bsr_vector_f32_kernel<BR, BC, 8, TV, Epi><<<g, SPMV_THREADS, 0, s>>>(B.n_rows, B.row_ptr.p, B.col_idx.p, o.vals, x, epi); break;
@@ -1327,9 +1449,9 @@ void spop_apply_f32(const SpOpLow<TV>& o, const float* x, Epi epi, cudaStream_t 
   TAM_LAUNCH_CHECK();
 }
 
-// Values of `op` (whichever layout it uses; SELL slots packed, see pack_pos) as a reduced-precision copy.
-void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s);
-void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s);
+// Values of `op` as a reduced-precision copy, in SpOpLow's order (batch: the batched solve's).
+void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s, bool batch = false);
+void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s, bool batch = false);
 
 // --- common epilogues ------------------------------------------------------
 struct NoStop {

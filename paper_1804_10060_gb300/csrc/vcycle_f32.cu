@@ -280,4 +280,23 @@ void build_low_precision(tam_amg_s* H, cudaStream_t s) {
   }
 }
 
+void build_batch_operators(tam_amg_s* H, cudaStream_t s) {
+  for (size_t l = 0; l + 1 < H->levels.size(); ++l) {
+    Level& L = H->levels[l];
+    auto own = [&](const SpOpLow<float>& o, DBuf<float>& v) {
+      if (!o.vals || !low_in_store(o.op)) return o;
+      convert_values_f32(o.op, v, s, true);
+      return SpOpLow<float>{o.op, v.p};
+    };
+    L.A32m = own(L.A32, L.A32mv);
+    L.P32m = own(L.P32, L.P32mv);
+    L.R32m = own(L.R32, L.R32mv);
+    L.A16m = L.A16;
+    if (L.A16.vals && low_in_store(L.A16.op)) {
+      convert_values_bf16(L.A16.op, L.A16mv, s, true);
+      L.A16m.vals = L.A16mv.p;
+    }
+  }
+}
+
 }  // namespace tam
