@@ -1301,7 +1301,7 @@ bsr_vector_f32_kernel(int n_rows, const int* __restrict__ rp, const int* __restr
 // of lpr_spmv_kernel and blockrow_spmv_kernel (values packed, x in records).
 // A lane per 6 x 6 block over the block-CSR arrays spreads a warp's request
 // over 32 lines and keeps a lane's chain long; these read whole lines (the
-// 1.38M-DOF P2 disc, 8,416 and 1,280 coarse rows: a Chebyshev step 24 -> 19 and
+// 1.38M-DOF P2 disc, 8,416 and 1,280 coarse rows: a Chebyshev step 24 -> 14 and
 // 17 -> 7 us, the prolongation between them 20 -> 12).  The operators of whole-warp rows (restriction to the first
 // coarse level: 2,100 rows of hundreds of 6 x 3 blocks) stay on the block-CSR
 // arrays, a warp per row: 36 us against 52 through the 8-lane store, whose
