@@ -1262,6 +1262,13 @@ tam_amg_s* amg_build(tam_matrix_s* K, const double* coords, const amg_params& pr
     H->r = DBuf<double>((size_t)n0 * 3, s);
     H->z = DBuf<double>((size_t)n0 * 3, s);
     H->p = DBuf<double>((size_t)n0 * 3, s);
+    if (K->A.br == 1)
+      for (Level& L : H->levels)
+        if (split_beforehand(L)) {
+          L.xsa = DBuf<float2>((size_t)L.n_rows, s);
+          L.xsb = DBuf<float2>((size_t)L.n_rows, s);
+        }
+    if (H->levels[0].xsa.p) H->ps = DBuf<float2>((size_t)n0, s);
     H->q = DBuf<double>((size_t)n0 * 3, s);
     H->sc = DBuf<PcgScalars>(1, s);
     if (prm.level_precision > 0) {

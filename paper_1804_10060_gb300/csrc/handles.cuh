@@ -66,6 +66,7 @@ struct Level {
   DBuf<__nv_bfloat16> A16v;
   SpOpLow<float> A32, P32, R32;
   SpOpLow<__nv_bfloat16> A16;
+  DBuf<float2> xsa, xsb;  // xa and xb split, where the level's products read them so (split_beforehand)
   // the batched solve's operators: the same copies, or block-CSR-ordered ones
   // of its own where the solve's follow a lanes-per-row store
   DBuf<float> A32mv, P32mv, R32mv;
@@ -125,6 +126,7 @@ struct tam_amg_s {
   tam::DBuf<double> coarse_inv;          // [n_coarse * n_coarse]
   // PCG workspace
   tam::DBuf<double> r, z, p, q;
+  tam::DBuf<float2> ps;                  // p split, where the products read it so (split_beforehand)
   tam::DBuf<double> bs, xs;              // b and x scaled by the solve's power of two
   tam::DBuf<double> hist;                // ||r_k||^2 of the last solve (scaled), k = 0 .. hist_len - 1
   long long hist_len = 0;
@@ -176,6 +178,11 @@ void vcycle_apply(tam_amg_s* H, const double* r, double* z, const int* stop, cud
 // The reduced-precision V-cycle (FP32 vectors and arithmetic; FP64 in/out on
 // level 0 and FP64 dense coarsest solve), and its set-up after amg_build.
 void vcycle_apply_low(tam_amg_s* H, const double* r, double* z, const int* stop, cudaStream_t s);
+// Whether a scalar level's products read x split beforehand (sell_spmv_pre):
+// double-float over SELL.
+inline bool split_beforehand(const Level& L) {
+  return L.bs == 1 && L.Aop.lpr == 0 && L.Aop.df && L.Aop.S && L.Aop.S->vals_df.p;
+}
 void build_low_precision(tam_amg_s* H, cudaStream_t s);
 // The batched solve's operators, after build_low_precision.
 void build_batch_operators(tam_amg_s* H, cudaStream_t s);

@@ -30,13 +30,15 @@ constexpr int TPB = 256;
 
 __global__ void cheb_first_zero_kernel(const double* __restrict__ b, const double* __restrict__ dinv,
                                        const double* __restrict__ consts, double* __restrict__ d,
-                                       double* __restrict__ x, long long N, const int* __restrict__ stop) {
+                                       double* __restrict__ x, float2* __restrict__ xs, long long N,
+                                       const int* __restrict__ stop) {
   if (stop && *stop) return;
   const double cr = consts[3];
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     double di = cr * dinv[i] * b[i];
     d[i] = di;
     x[i] = di;
+    if (xs) xs[i] = split_bits(di);
   }
 }
 
@@ -49,6 +51,7 @@ struct EpiCheb {
   const double* coef;  // (c_d, c_r) of this step
   double* d;
   double* xn;          // next iterate (other buffer)
+  float2* xns;         // BR = 1: the next iterate split, or null
   int n_rows;
   const int* stop;
   __device__ bool skip() const { return stop && *stop; }
@@ -77,6 +80,8 @@ struct EpiCheb {
     for (int r = 0; r < BR; ++r) {
       d[i0 + r] = dv[r];
       xn[i0 + r] = xv[r] + dv[r];
+      if constexpr (BR == 1)
+        if (xns) xns[row] = split_bits(xv[r] + dv[r]);
     }
   }
 };
@@ -180,14 +185,16 @@ struct EpiInitResidual {
 };
 
 // rho = r . z (> 0 for an SPD preconditioner);  first call also sets p = z
+// ps: p split, or null (as below)
 __global__ void pcg_rz_kernel(const double* __restrict__ r, const double* __restrict__ z, double* __restrict__ p,
-                              long long N, GridReduce gr, PcgScalars* sc, int first) {
+                              float2* __restrict__ ps, long long N, GridReduce gr, PcgScalars* sc, int first) {
   __shared__ double sh[32];
   if (sc->stop) return;
   double acc[1] = {0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     acc[0] += r[i] * z[i];
     if (first) p[i] = z[i];
+    if (first && ps) ps[i] = split_bits(z[i]);
   }
   double tot[1];
   if (grid_reduce<1>(gr, acc, tot, sh) && threadIdx.x == 0) {
@@ -251,12 +258,15 @@ __global__ void pcg_update_kernel(double* __restrict__ x, double* __restrict__ r
   }
 }
 
-__global__ void pcg_direction_kernel(const double* __restrict__ z, double* __restrict__ p, long long N,
-                                     const PcgScalars* sc) {
+__global__ void pcg_direction_kernel(const double* __restrict__ z, double* __restrict__ p, float2* __restrict__ ps,
+                                     long long N, const PcgScalars* sc) {
   if (sc->stop) return;
   const double beta = sc->beta;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-    p[i] = z[i] + beta * p[i];
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    const double v = z[i] + beta * p[i];
+    p[i] = v;
+    if (ps) ps[i] = split_bits(v);
+  }
 }
 
 // final ||b - K x||^2
@@ -293,22 +303,28 @@ __global__ void loop_control_kernel(cudaGraphConditionalHandle h, const int* __r
 // ---------------------------------------------------------------------------
 // Dispatch on block shapes (3x3, 6x6 for A; 3x6, 6x3, 6x6, 3x3 for P and R)
 // ---------------------------------------------------------------------------
+// xs, xns: x and xn split (scalar levels, split_beforehand) or null
 void cheb_step(const Level& L, const double* b, const double* x, double* d, double* xn, int step, const int* stop,
-               cudaStream_t s) {
+               cudaStream_t s, const float2* xs = nullptr, float2* xns = nullptr) {
   const double* coef = L.consts.p + 2 + 2 * step;
   if (L.bs == 3)
-    spop_apply<3, 3>(L.Aop, x, EpiCheb<3>{b, x, L.dinv.p, coef, d, xn, L.n_rows, stop}, s);
+    spop_apply<3, 3>(L.Aop, x, EpiCheb<3>{b, x, L.dinv.p, coef, d, xn, nullptr, L.n_rows, stop}, s);
   else if (L.bs == 6)
-    spop_apply<6, 6>(L.Aop, x, EpiCheb<6>{b, x, L.dinv.p, coef, d, xn, L.n_rows, stop}, s);
+    spop_apply<6, 6>(L.Aop, x, EpiCheb<6>{b, x, L.dinv.p, coef, d, xn, nullptr, L.n_rows, stop}, s);
+  else if (xs)
+    sell_spmv_pre<1, 1>(*L.Aop.S, xs, EpiCheb<1>{b, x, L.dinv.p, coef, d, xn, xns, L.n_rows, stop}, s);
   else
-    spop_apply<1, 1>(L.Aop, x, EpiCheb<1>{b, x, L.dinv.p, coef, d, xn, L.n_rows, stop}, s);
+    spop_apply<1, 1>(L.Aop, x, EpiCheb<1>{b, x, L.dinv.p, coef, d, xn, nullptr, L.n_rows, stop}, s);
 }
 
-void residual(const Level& L, const double* b, const double* x, double* t, const int* stop, cudaStream_t s) {
+void residual(const Level& L, const double* b, const double* x, double* t, const int* stop, cudaStream_t s,
+              const float2* xs = nullptr) {
   if (L.bs == 3)
     spop_apply<3, 3>(L.Aop, x, EpiResidual<3>{b, t, L.n_rows, stop}, s);
   else if (L.bs == 6)
     spop_apply<6, 6>(L.Aop, x, EpiResidual<6>{b, t, L.n_rows, stop}, s);
+  else if (xs)
+    sell_spmv_pre<1, 1>(*L.Aop.S, xs, EpiResidual<1>{b, t, L.n_rows, stop}, s);
   else
     spop_apply<1, 1>(L.Aop, x, EpiResidual<1>{b, t, L.n_rows, stop}, s);
 }
@@ -322,10 +338,26 @@ void restrict_to(const Level& L, const double* t, double* bc, const int* stop, c
   else spop_apply<3, 3>(L.Rop, t, EpiStore<3>{bc, nr, stop}, s);
 }
 
-void prolong_add(const Level& L, const double* xc, double* x, const int* stop, cudaStream_t s) {
+// x += A xc on a scalar level, and x split
+struct EpiAddSplit {
+  double* y;
+  float2* ys;
+  int n_rows;
+  const int* stop;
+  __device__ bool skip() const { return stop && *stop; }
+  __device__ void operator()(int row, const double (&acc)[1], double*) const {
+    if (row >= n_rows) return;
+    const double v = y[row] + acc[0];
+    y[row] = v;
+    ys[row] = split_bits(v);
+  }
+};
+
+void prolong_add(const Level& L, const double* xc, double* x, const int* stop, cudaStream_t s, float2* xs = nullptr) {
   const int nr = L.P.n_rows;
   if (L.kdim == 6 && L.bs == 3) spop_apply<3, 6>(L.Pop, xc, EpiAdd<3>{x, nr, stop}, s);
   else if (L.kdim == 6 && L.bs == 6) spop_apply<6, 6>(L.Pop, xc, EpiAdd<6>{x, nr, stop}, s);
+  else if (L.kdim == 1 && xs) spop_apply<1, 1>(L.Pop, xc, EpiAddSplit{x, xs, nr, stop}, s);
   else if (L.kdim == 1) spop_apply<1, 1>(L.Pop, xc, EpiAdd<1>{x, nr, stop}, s);
   else spop_apply<3, 3>(L.Pop, xc, EpiAdd<3>{x, nr, stop}, s);
 }
@@ -360,25 +392,32 @@ void vcycle_level(tam_amg_s* H, int l, const double* b, double* out, const int* 
   const int deg = L.deg;
   double* xa = L.xa.p;
   double* xb = L.xb.p;
+  const bool split = L.xsa.p && split_beforehand(L);
+  float2* sa = split ? L.xsa.p : nullptr;  // xa and xb split
+  float2* sb = split ? L.xsb.p : nullptr;
   // pre-smoothing from zero
-  cheb_first_zero_kernel<<<vec_grid(N), TPB, 0, s>>>(b, L.dinv.p, L.consts.p, L.d.p, xa, N, stop);
+  cheb_first_zero_kernel<<<vec_grid(N), TPB, 0, s>>>(b, L.dinv.p, L.consts.p, L.d.p, xa, sa, N, stop);
   TAM_LAUNCH_CHECK();
   for (int k = 1; k < deg; ++k) {
-    cheb_step(L, b, xa, L.d.p, xb, k, stop, s);
+    cheb_step(L, b, xa, L.d.p, xb, k, stop, s, sa, sb);
     std::swap(xa, xb);
+    std::swap(sa, sb);
   }
-  residual(L, b, xa, L.t.p, stop, s);
+  residual(L, b, xa, L.t.p, stop, s, sa);
   Level& C = H->levels[l + 1];
   restrict_to(L, L.t.p, C.b.p, stop, s);
   double* xc = C.y.p;
   vcycle_level(H, l + 1, C.b.p, xc, stop, s);
-  prolong_add(L, xc, xa, stop, s);
+  prolong_add(L, xc, xa, stop, s, sa);
   // post-smoothing from x
   for (int k = 0; k < deg; ++k) {
     double* dst = (k == deg - 1) ? out : xb;
-    cheb_step(L, b, xa, L.d.p, dst, k, stop, s);
+    float2* dst_s = (k == deg - 1) ? nullptr : sb;
+    cheb_step(L, b, xa, L.d.p, dst, k, stop, s, sa, dst_s);
     xb = xa;
     xa = dst;
+    sb = sa;
+    sa = dst_s;
   }
 }
 
@@ -410,7 +449,11 @@ void spmv_outer_pq(tam_amg_s* H, cudaStream_t s) {
   GridReduce gr{H->partials.p, H->ticket.p};
   by_block(H->K->A.br, [&](auto B) {
     constexpr int BR = decltype(B)::value;
-    spmv_outer<BR>(H, H->p.p, EpiPq<BR>{H->p.p, H->q.p, H->K->n_nodes, gr, H->sc.p}, s);
+    const EpiPq<BR> epi{H->p.p, H->q.p, H->K->n_nodes, gr, H->sc.p};
+    if constexpr (BR == 1) {
+      if (H->ps.p && split_beforehand(H->levels[0])) return sell_spmv_pre<1, 1, true>(H->K->S, H->ps.p, epi, s);
+    }
+    spmv_outer<BR>(H, H->p.p, epi, s);
   });
 }
 
@@ -423,9 +466,9 @@ void enqueue_iteration(tam_amg_s* H, double* x, cudaStream_t s) {
                                                 (int)H->hist.n);
   TAM_LAUNCH_CHECK();
   precondition(H, H->r.p, H->z.p, stop, s);
-  pcg_rz_kernel<<<vec_grid(N), TPB, 0, s>>>(H->r.p, H->z.p, H->p.p, N, gr, H->sc.p, 0);
+  pcg_rz_kernel<<<vec_grid(N), TPB, 0, s>>>(H->r.p, H->z.p, H->p.p, H->ps.p, N, gr, H->sc.p, 0);
   TAM_LAUNCH_CHECK();
-  pcg_direction_kernel<<<vec_grid(N), TPB, 0, s>>>(H->z.p, H->p.p, N, H->sc.p);
+  pcg_direction_kernel<<<vec_grid(N), TPB, 0, s>>>(H->z.p, H->p.p, H->ps.p, N, H->sc.p);
   TAM_LAUNCH_CHECK();
 }
 
@@ -539,7 +582,7 @@ int pcg_solve(tam_amg_s* H, const double* b, double* x, double rtol, double atol
     spmv_outer<BR>(H, x, EpiInitResidual<BR>{b, H->r.p, H->K->n_nodes, gr, sc, H->hist.p}, s);
   });
   precondition(H, H->r.p, H->z.p, &sc->stop, s);
-  pcg_rz_kernel<<<vec_grid(N), TPB, 0, s>>>(H->r.p, H->z.p, H->p.p, N, gr, sc, 1);
+  pcg_rz_kernel<<<vec_grid(N), TPB, 0, s>>>(H->r.p, H->z.p, H->p.p, H->ps.p, N, gr, sc, 1);
   TAM_LAUNCH_CHECK();
   // the iterations as one graph: a device-side WHILE loop over one iteration,
   // built on the first solve with this hierarchy, one launch per solve
@@ -607,7 +650,8 @@ void smooth_fine(tam_amg_s* H, const double* b, double* x, int degree, double lo
   for (int k = 0; k < degree; ++k) {
     by_block(L.bs, [&](auto B) {
       constexpr int BR = decltype(B)::value;
-      spop_apply<BR, BR>(L.Aop, cur, EpiCheb<BR>{b, cur, L.dinv.p, coef + 2 + 2 * k, L.d.p, nxt, L.n_rows, nullptr},
+      spop_apply<BR, BR>(L.Aop, cur, EpiCheb<BR>{b, cur, L.dinv.p, coef + 2 + 2 * k, L.d.p, nxt, nullptr, L.n_rows,
+                                                 nullptr},
                          s);
     });
     std::swap(cur, nxt);

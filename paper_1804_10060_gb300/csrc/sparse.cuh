@@ -325,10 +325,24 @@ __device__ __forceinline__ void gather_x(const double* __restrict__ x, int c, do
 
 // f(std::true_type) when x is 16-byte aligned, else f(std::false_type): one
 // uniform branch around a kernel's row loop.
+// A vector split beforehand (hi, lo), entry by entry
+template <int BC, bool AL>
+__device__ __forceinline__ void gather_x(const float2* __restrict__ x, int c, float2 (&v)[BC]) {
+#pragma unroll
+  for (int j = 0; j < BC; ++j) v[j] = __ldg(x + (size_t)c * BC + j);
+}
+
+__device__ __forceinline__ float2 as_split(double v) { return split_bits(v); }
+__device__ __forceinline__ float2 as_split(float2 v) { return v; }
+
 template <class F>
 __device__ __forceinline__ void by_alignment(const double* x, F&& f) {
   if ((reinterpret_cast<size_t>(x) & 15) == 0) f(std::true_type());
   else f(std::false_type());
+}
+template <class F>
+__device__ __forceinline__ void by_alignment(const float2*, F&& f) {
+  f(std::true_type());  // read entry by entry
 }
 
 
@@ -337,10 +351,18 @@ __device__ __forceinline__ void by_alignment(const double* x, F&& f) {
 // ones).  A row is a serial chain of its slots, and a mesh of a few thousand
 // slices (quadratic cells: 27 slots a row) leaves the chip with one or two
 // waves of long chains; see sell_split.
-template <int BR, int BC, class Epi, bool DF, bool ACC, int S>
+//
+// XT = float2: x comes split already.  The split of a gathered FP64 value takes
+// some 35 integer instructions, which a 1 x 1 block spreads over one product
+// (460k-unknown P2 disc: Chebyshev step 52 -> 40 us, the CG's product 74 ->
+// 57).  3 x 3 blocks are bound by their 72 bytes a block instead (as
+// 32-byte records for one sector a gather, the CG's product 225 -> 212 us on
+// the 1.38M-DOF disc and 230 -> 225 on the 3.26M-DOF box, which writing the
+// records took back): they split as they gather.
+template <int BR, int BC, class Epi, bool DF, bool ACC, int S, typename XT = double>
 __global__ void __launch_bounds__(SPMV_THREADS)
-sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
-  static_assert(DF || S == 1, "sell_spmv_kernel: FP64 rows are not split");
+sell_spmv_kernel(SellView A, const XT* __restrict__ x, Epi epi) {
+  static_assert(DF || (S == 1 && std::is_same<XT, double>::value), "sell_spmv_kernel: FP64 rows are not split");
   constexpr int SLICES = SPMV_THREADS / 32 / S;  // per block
   __shared__ double sh[32];
   [[maybe_unused]] __shared__ float2 part[S > 1 ? SLICES : 1][BR][32];
@@ -369,10 +391,10 @@ sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
       // to ~2^-45 on long P2 rows); FP32 work only (an FP64 sum every two
       // slots cost 1.5 FP64 adds per row and slot pair on GB300's slow FP64
       // pipe).
-      auto slot = [&](const float2 (&vv)[BR * BC], const double (&xg)[BC]) {
+      auto slot = [&](const float2 (&vv)[BR * BC], const XT (&xg)[BC]) {
         float2 xv[BC];
 #pragma unroll
-        for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
+        for (int j = 0; j < BC; ++j) xv[j] = as_split(xg[j]);
 #pragma unroll
         for (int r = 0; r < BR; ++r) {
           if constexpr (ACC) {
@@ -396,7 +418,7 @@ sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
         for (int k = k0; k < k1; k += S) {
           float2 vv[BR * BC];
           slot_load<BR * BC, 32>(vp, lane, vv);
-          double xg[BC];
+          XT xg[BC];
           gather_x<BC, AL>(x, c0, xg);
           c0 = c1;
           if (k + 2 * S < k1) c1 = __ldg(cp + 2 * S * 32);
@@ -414,11 +436,11 @@ sell_spmv_kernel(SellView A, const double* __restrict__ x, Epi epi) {
         for (int u = 0; u < U; ++u) cn[u] = k0 + u * S < k1 ? __ldg(cp + u * S * 32) : 0;
         for (int k = k0; k < k1; k += U * S) {
           float2 vv[U][1];
-          double xg[U][1];
+          XT xg[U][1];
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             vv[u][0] = make_float2(0.f, 0.f);
-            xg[u][0] = 0.0;
+            xg[u][0] = XT();
             if (u == 0 || k + u * S < k1) {
               vv[u][0] = __ldg(vp + u * S * 32 + lane);
               gather_x<1, AL>(x, cn[u], xg[u]);
@@ -485,6 +507,16 @@ void sell_spmv(const Sell& A, const double* x, Epi epi, cudaStream_t s, bool df 
   if (!use) sell_spmv_kernel<BR, BC, Epi, false, false, 1><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
   else if (split == 2) sell_spmv_kernel<BR, BC, Epi, true, ACC, 2><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
   else sell_spmv_kernel<BR, BC, Epi, true, ACC, 1><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
+  TAM_LAUNCH_CHECK();
+}
+
+// The same for an x split beforehand (A must have its split copy).
+template <int BR, int BC, bool ACC = false, class Epi>
+void sell_spmv_pre(const Sell& A, const float2* x, Epi epi, cudaStream_t s) {
+  const int split = sell_split(A.n_slices);
+  const unsigned grid = grid_for((long long)A.n_slices * 32 * split, SPMV_THREADS);
+  if (split == 2) sell_spmv_kernel<BR, BC, Epi, true, ACC, 2, float2><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
+  else sell_spmv_kernel<BR, BC, Epi, true, ACC, 1, float2><<<grid, SPMV_THREADS, 0, s>>>(view(A), x, epi);
   TAM_LAUNCH_CHECK();
 }
 
@@ -1320,15 +1352,26 @@ lpr_spmv_f32_kernel(int n_rows, const int* __restrict__ gp, const int* __restric
   for (int r = 0; r < BR; ++r) acc[r] = 0.f;
   if (row < n_rows) {
     const int g0 = gp[row], g1 = gp[row + 1];
-    float xn[BC];  // the gather runs one group ahead
-    if (g0 < g1) gather_f32<BC>(x, __ldg(cols + (size_t)g0 * LPR + sub), xn);
+    // one group ahead: its values and its gather (values loaded in their own
+    // turn: 21 us a level-1 step of the disc instead of 14)
+    TV vn[BB];
+    float xn[BC];
+    if (g0 < g1) {
+      slot_load<BB, LPR>(v + (size_t)g0 * BB * LPR, sub, vn);
+      gather_f32<BC>(x, __ldg(cols + (size_t)g0 * LPR + sub), xn);
+    }
     for (int g = g0; g < g1; ++g) {
       TV vv[BB];
-      slot_load<BB, LPR>(v + (size_t)g * BB * LPR, sub, vv);
       float xv[BC];
 #pragma unroll
+      for (int e = 0; e < BB; ++e) vv[e] = vn[e];
+#pragma unroll
       for (int j = 0; j < BC; ++j) xv[j] = xn[j];
-      if (g + 1 < g1) gather_f32<BC>(x, __ldg(cols + (size_t)(g + 1) * LPR + sub), xn);
+      if (g + 1 < g1) {
+        const int c = __ldg(cols + (size_t)(g + 1) * LPR + sub);
+        slot_load<BB, LPR>(v + (size_t)(g + 1) * BB * LPR, sub, vn);
+        gather_f32<BC>(x, c, xn);
+      }
 #pragma unroll
       for (int r = 0; r < BR; ++r)
 #pragma unroll
