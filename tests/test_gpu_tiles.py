@@ -219,3 +219,33 @@ def test_scan_lengths(n):
     K, _ = tam.fem_assemble_elasticity(**tam.problem_to_device(q))
     rp = tam.tam_matrix_export_bsr(K)[0].cpu().numpy()
     assert np.array_equal(np.diff(rp), np.r_[np.full(4, 4), np.ones(n, int)])
+
+
+@pytest.mark.parametrize("precision,tol", [(1, 1e-5), (2, 5e-2)])
+@pytest.mark.parametrize("hexes,degree", [((5, 4, 3), 1), ((24, 20, 18), 1), ((36, 30, 30), 1), ((44, 38, 38), 1), ((12, 12, 10), 2)])
+def test_low_precision_vcycle_lane_layouts(hexes, degree, precision, tol):
+    """One FP32 V-cycle against the FP64 one, for meshes whose levels take 2, 4, 8 and more lanes per row, block
+    rows and thread-per-row (FP32 rounding: 1e-5; BF16 finest values: 5e-2)."""
+    tam = need_gpu()
+    pb = meshgen.slab_box_problem(*hexes, degree=degree)
+    d = tam.problem_to_device(pb)
+    K, rhs = tam.fem_assemble_elasticity(**d)
+    r = torch.randn((pb.n_nodes, 3), dtype=torch.float64, device="cuda", generator=torch.Generator(device="cuda").manual_seed(2))
+    z = [tam.amg_vcycle(tam.amg_setup(K, d["coords"], tam.amg_params_default(level_precision=p, coarse_max_dofs=60)), r)
+         for p in (0, precision)]
+    assert float((z[1] - z[0]).norm() / z[0].norm()) <= tol
+
+
+@pytest.mark.parametrize("hexes,degree", [((24, 20, 18), 1), ((44, 38, 38), 1), ((20, 20, 20), 2)])
+def test_direction_split_beforehand(hexes, degree):
+    """The CG's products on rows of several lanes, thread-per-row and two warps per slice: the true residual (plain
+    double-float or FP64 product of the result) is what the recurrence says, to a few 2^-48 of its terms."""
+    tam = need_gpu()
+    pb = meshgen.slab_box_problem(*hexes, degree=degree)
+    d = tam.problem_to_device(pb)
+    K, rhs = tam.fem_assemble_elasticity(**d)
+    H = tam.amg_setup(K, d["coords"])
+    x = torch.zeros_like(rhs)
+    it, rel, st = tam.amg_pcg_solve(H, rhs, x, rtol=1e-8, max_iter=300)
+    true = tam.tam_matrix_residual_norm(K, rhs, x) / float(rhs.norm())
+    assert rel <= 1e-8 and abs(true - rel) <= 1e-2 * rel, (it, rel, true)
