@@ -1399,16 +1399,31 @@ blockrow_f32_kernel(int n_rows, const int* __restrict__ rp, const int* __restric
   float ad = 0.f;
   if (row < n_rows && g < G) {
     const int p1 = rp[row + 1];
-    float xn[B];  // the gather runs one step ahead (a group's lanes read one record)
-    int p = rp[row] + wr * G + g;
-    if (p < p1) gather_f32<B>(x, __ldg(ci + p), xn);
-    for (; p < p1; p += WPR * G) {
+    // values and x one step ahead, columns two (a group's lanes read one record;
+    // with x alone ahead 11.7 us instead of 10.7 for the disc's prolongation to
+    // level 1; the double-float kernel's long rows lose 2% that way)
+    constexpr int STEP = WPR * G;
+    TV vn[B];
+    float xn[B];
+    int p = rp[row] + wr * G + g, cn = 0;
+    if (p < p1) {
+      block_load_low<B>(v + (size_t)p * BB + r * B, vn);
+      gather_f32<B>(x, __ldg(ci + p), xn);
+      if (p + STEP < p1) cn = __ldg(ci + p + STEP);
+    }
+    for (; p < p1; p += STEP) {
       TV vv[B];
-      block_load_low<B>(v + (size_t)p * BB + r * B, vv);
       float xv[B];
 #pragma unroll
-      for (int j = 0; j < B; ++j) xv[j] = xn[j];
-      if (p + WPR * G < p1) gather_f32<B>(x, __ldg(ci + p + WPR * G), xn);
+      for (int j = 0; j < B; ++j) {
+        vv[j] = vn[j];
+        xv[j] = xn[j];
+      }
+      if (p + STEP < p1) {
+        block_load_low<B>(v + (size_t)(p + STEP) * BB + r * B, vn);
+        gather_f32<B>(x, cn, xn);
+        if (p + 2 * STEP < p1) cn = __ldg(ci + p + 2 * STEP);
+      }
 #pragma unroll
       for (int j = 0; j < B; ++j) ad = fmaf(to_f32(vv[j]), xv[j], ad);
     }
