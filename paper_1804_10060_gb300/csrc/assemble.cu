@@ -454,7 +454,7 @@ __device__ __forceinline__ double p2_moment(int c, int k) {
 // 32 x 9 values, so that a request covers 9 neighbouring values of a block
 // (3 sectors) instead of one value of 32 blocks (32 sectors).  15.3 -> 1.4 ms
 // on 331,776 cells (the operations alone: 1.1 ms at the measured FP64 rate);
-// the whole assembly 18.0 -> 4.1 ms.
+// the whole assembly 18.0 -> 3.8 ms.
 constexpr int P2_WARPS = 8, P2_CELLS = 32;
 
 struct P2Tile {
