@@ -503,7 +503,7 @@ dense_mma_kernel(const float* __restrict__ A, long long n, int K, int N, const _
 // written.  Same roundings, products and summation order as the layer-by-
 // layer kernel above, so the results are bitwise the same.  Bound by the
 // hidden layers' tanh (384 a row); the weight fragments come four registers a
-// request (468,864 rows of 8-128-128-128-3: 6.40 -> 6.25 ms).
+// request (11.6M rows of 8-128-128-128-3: 6.40 -> 6.25 ms).
 // ---------------------------------------------------------------------------
 constexpr int FUSED_WARPS = 8;
 constexpr int FUSED_MAX_LAYERS = 8;
