@@ -255,11 +255,9 @@ struct AsmArgs {
   int npc = 0;
 };
 
-// Does the element block (row na, column nb) contribute anything?  In
-// loads-only mode only Dirichlet columns with prescribed values do (lifting).
-__device__ __forceinline__ bool block_needed(const AsmArgs& A, int nb) {
-  return !A.loads_only || (A.dmask[nb] && A.ud);
-}
+// Whether the element blocks go into K's values: not in the deterministic
+// mode (slots of its own) nor for the loads alone.
+__device__ __forceinline__ bool fills_values(const AsmArgs& A) { return !A.ck && !A.loads_only; }
 
 // Scatter one 3x3 block (row node na, col node nb; local a, b of cell c) or
 // lift it into the load; in deterministic mode store it in its slot.
@@ -292,7 +290,7 @@ __device__ __forceinline__ void scatter_block(const AsmArgs& A, int c, int a, in
 // Dirichlet node.
 __device__ __forceinline__ int block_slot(const AsmArgs& A, int c, int a, int b, int na, int nb, bool fixed,
                                           const double (&k)[9]) {
-  if (A.ck || fixed || A.loads_only) {
+  if (fixed || !fills_values(A)) {
     scatter_block(A, c, a, b, na, nb, k);
     return -1;
   }
@@ -356,8 +354,12 @@ __global__ void __launch_bounds__(P1_THREADS) assemble_p1_kernel(AsmArgs A) {
   bool fixed[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) fixed[a] = A.dmask[v[a]] != 0;
-  // the loads alone need no stiffness unless a prescribed displacement is lifted
-  if (!A.loads_only || A.ud) {
+  // the loads alone need no stiffness unless a prescribed displacement is
+  // lifted: a warp without Dirichlet nodes skips it, the others the pairs that
+  // no lane needs (786,432 cells, one face of the box held: 677 -> 320 us; each
+  // pair of every cell otherwise)
+  const bool lifted = A.ud && (fixed[0] || fixed[1] || fixed[2] || fixed[3]);
+  if (!A.loads_only || __any_sync(0xffffffffu, lifted)) {
     // K_ab[i][j] = lg_a[i] g_b[j] + mg_a[j] g_b[i] + delta_ij (mg_a . g_b),
     // lg = lam vol g, mg = mu vol g; K_ba = K_ab^T
     const double lv = lam * vol, mv = mu * vol;
@@ -372,6 +374,9 @@ __global__ void __launch_bounds__(P1_THREADS) assemble_p1_kernel(AsmArgs A) {
       }
 #pragma unroll
       for (int b = a; b < 4; ++b) {
+        const bool ab = ok && !fixed[a] && (!A.loads_only || (fixed[b] && A.ud));
+        const bool ba = b != a && ok && !fixed[b] && (!A.loads_only || (fixed[a] && A.ud));
+        if (A.loads_only && !__any_sync(0xffffffffu, ab || ba)) continue;
         const double mgg = fma(mg[0], g[b][0], fma(mg[1], g[b][1], mg[2] * g[b][2]));
         double k[9];
 #pragma unroll
@@ -383,13 +388,13 @@ __global__ void __launch_bounds__(P1_THREADS) assemble_p1_kernel(AsmArgs A) {
             else k[3 * i + j] = i < j ? sg[i] * g[a][j] : k[3 * j + i];
           }
         int s = -1;
-        if (ok && !fixed[a] && block_needed(A, v[b])) s = block_slot(A, c, a, b, v[a], v[b], fixed[b], k);
-        scatter_run(A.vals, k, s, s_out[wid], s_slot[wid], lane);
+        if (ab) s = block_slot(A, c, a, b, v[a], v[b], fixed[b], k);
+        if (fills_values(A)) scatter_run(A.vals, k, s, s_out[wid], s_slot[wid], lane);
         if (b != a) {
           const double kt[9] = {k[0], k[3], k[6], k[1], k[4], k[7], k[2], k[5], k[8]};
           s = -1;
-          if (ok && !fixed[b] && block_needed(A, v[a])) s = block_slot(A, c, b, a, v[b], v[a], fixed[a], kt);
-          scatter_run(A.vals, kt, s, s_out[wid], s_slot[wid], lane);
+          if (ba) s = block_slot(A, c, b, a, v[b], v[a], fixed[a], kt);
+          if (fills_values(A)) scatter_run(A.vals, kt, s, s_out[wid], s_slot[wid], lane);
         }
       }
     }
@@ -589,12 +594,12 @@ __global__ void __launch_bounds__(P2_WARPS * 32) assemble_p2_kernel(AsmArgs A) {
       // the block to (a, b), then its transpose to (b, a)
       int slot = -1;
       if (ab) slot = block_slot(A, c, a, b, na, nb, db, k);
-      scatter_run(A.vals, k, slot, S.out[wid][0], S.slot[wid], lane);
+      if (fills_values(A)) scatter_run(A.vals, k, slot, S.out[wid][0], S.slot[wid], lane);
       if (a != b) {
         const double kt[9] = {k[0], k[3], k[6], k[1], k[4], k[7], k[2], k[5], k[8]};
         slot = -1;
         if (ba) slot = block_slot(A, c, b, a, nb, na, da, kt);
-        scatter_run(A.vals, kt, slot, S.out[wid][0], S.slot[wid], lane);
+        if (fills_values(A)) scatter_run(A.vals, kt, slot, S.out[wid][0], S.slot[wid], lane);
       }
     }
   // loads: f_a = kT vol int (T_h - T_ref) grad phi_a + vol int f_h phi_a
