@@ -382,7 +382,8 @@ int tam_mlp_set_params(tam_mlp mlp, const float* theta_host);
  * BF16-rounded activations on the tensor cores with FP32 accumulation, the
  * whole network in one kernel (activations never leave the SM; nets of at
  * most 8 layers of width <= 128, else layer by layer); 2: the same BF16
- * arithmetic one kernel per layer (bitwise the same results as 1). */
+ * arithmetic one kernel per layer (bitwise the same results as 1).  Y may
+ * overlap X, except in the one-kernel form. */
 int tam_mlp_forward(tam_mlp mlp, long long n, const float* X, float* Y, int bf16, void* stream);
 /* mean squared error of net(X) against Yt and its gradient (grad_host: n_params
  * floats, may be NULL); synchronising */

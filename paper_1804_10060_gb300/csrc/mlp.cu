@@ -16,6 +16,7 @@
 // weights.  Each FP32 dense layer is one tiled kernel (dense_kernel), its
 // weight gradient a split sum over row tiles (weight_grad_kernel).
 #include <cmath>
+#include <functional>
 #include <type_traits>
 #include <vector>
 
@@ -841,13 +842,22 @@ void mlp_forward_device(tam_mlp_s* M, long long n, const float* X, float* Y, int
   }
   if (bf16) ensure_bf16(M, s);
   ensure_workspace(M, std::min(n, PIECE), false, s);
+  // a piece's outputs over the inputs of later ones (a caller's Y may overlap
+  // its X): all outputs aside first
+  DBuf<float> aside;
+  float* out = Y;
+  if (n > PIECE && std::less<const float*>()(X, Y + n * M->n_out) && std::less<const float*>()(Y, X + n * M->n_in)) {
+    aside = DBuf<float>((size_t)n * M->n_out, s);
+    out = aside.p;
+  }
   for (long long r = 0; r < n; r += PIECE) {
     const long long m = std::min(PIECE, n - r);
     const float* Xr = X + r * M->n_in;
-    float* Yr = Y + r * M->n_out;
+    float* Yr = out + r * M->n_out;
     if (bf16) forward<__nv_bfloat16>(M, Xr, m, M->theta16.p, Yr, s);
     else forward<float>(M, Xr, m, M->theta.p, Yr, s);
   }
+  if (aside.p) TAM_CUDA(cudaMemcpyAsync(Y, aside.p, sizeof(float) * (size_t)n * M->n_out, cudaMemcpyDeviceToDevice, s));
 }
 int mlp_n_in(tam_mlp_s* M) { return M->n_in; }
 int mlp_n_out(tam_mlp_s* M) { return M->n_out; }
