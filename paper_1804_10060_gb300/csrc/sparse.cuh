@@ -298,8 +298,9 @@ constexpr int SPMV_THREADS = 128;
 // 16-byte boundary for even c, 8 bytes past one for odd c).  AL: x itself is
 // 16-byte aligned (a caller's vector need not be: gather_x with AL = false).
 // Measured: the accurate product of a 1.38M-DOF P2 mesh 288 -> 265 us, the
-// level-0 prolongation of the 3.26M-DOF box 143 -> 133 us.  The lanes-per-row
-// kernels keep single loads for BC = 3 (the restriction: 112 us, 119 in pairs).
+// level-0 prolongation of the 3.26M-DOF box 143 -> 133 us.  Single loads stay
+// for BC = 3 in the lanes-per-row kernels (the restriction: 112 us, 119 in
+// pairs) and in plain FP64 (gather_pairs).
 template <int BC, bool AL>
 __device__ __forceinline__ void gather_x(const double* __restrict__ x, int c, double (&v)[BC]) {
   const double* __restrict__ p = x + (size_t)c * BC;
@@ -323,8 +324,6 @@ __device__ __forceinline__ void gather_x(const double* __restrict__ x, int c, do
   }
 }
 
-// f(std::true_type) when x is 16-byte aligned, else f(std::false_type): one
-// uniform branch around a kernel's row loop.
 // A vector split beforehand (hi, lo), entry by entry
 template <int BC, bool AL>
 __device__ __forceinline__ void gather_x(const float2* __restrict__ x, int c, float2 (&v)[BC]) {
@@ -335,16 +334,32 @@ __device__ __forceinline__ void gather_x(const float2* __restrict__ x, int c, fl
 __device__ __forceinline__ float2 as_split(double v) { return split_bits(v); }
 __device__ __forceinline__ float2 as_split(float2 v) { return v; }
 
-template <class F>
+// BC = 3 in plain FP64: a row is one thread's chain of column, gather and
+// multiply-adds, and a pair's selects lengthen it (in pairs tam_matrix_spmv of
+// a 60,625-row P2 mesh took 123 us instead of 92, the FP64 V-cycle of one of
+// 116,281 rows 726 instead of 645) -- except in the SELL kernels whose epilogue
+// sums over the grid (a member gr): they get more registers, and the residual
+// norm of the larger mesh takes 137 us in pairs, 150 without.
+template <int BC, bool DF>
+constexpr bool gather_pairs = BC % 2 == 0 || DF;
+template <class Epi, class = void>
+struct sums_over_grid : std::false_type {};
+template <class Epi>
+struct sums_over_grid<Epi, std::void_t<decltype(Epi::gr)>> : std::true_type {};
+
+// f(std::true_type) when x is 16-byte aligned and PAIRS, else
+// f(std::false_type): one uniform branch around a kernel's row loop.
+template <bool PAIRS, class F>
 __device__ __forceinline__ void by_alignment(const double* x, F&& f) {
-  if ((reinterpret_cast<size_t>(x) & 15) == 0) f(std::true_type());
-  else f(std::false_type());
+  if constexpr (PAIRS) {
+    if ((reinterpret_cast<size_t>(x) & 15) == 0) return f(std::true_type());
+  }
+  f(std::false_type());
 }
-template <class F>
+template <bool PAIRS, class F>
 __device__ __forceinline__ void by_alignment(const float2*, F&& f) {
   f(std::true_type());  // read entry by entry
 }
-
 
 // S: warps per slice.  With S = 2 the slice's slots alternate between two
 // warps, whose row sums meet in shared memory (each row: even slots, then odd
@@ -376,7 +391,7 @@ sell_spmv_kernel(SellView A, const XT* __restrict__ x, Epi epi) {
   if constexpr (DF)
 #pragma unroll
     for (int r = 0; r < BR; ++r) run[r] = make_float2(0.f, 0.f);
-  by_alignment(x, [&](auto al) {
+  by_alignment<gather_pairs<BC, DF> || sums_over_grid<Epi>::value>(x, [&](auto al) {
     constexpr bool AL = decltype(al)::value;
     if (slice >= A.n_slices) return;
     const int k0 = A.slice_ptr[slice] + sub, k1 = A.slice_ptr[slice + 1];
@@ -577,7 +592,7 @@ bsr_vector_kernel(BsrView A, const double* __restrict__ x, Epi epi) {
   double acc[BR];
 #pragma unroll
   for (int r = 0; r < BR; ++r) acc[r] = 0.0;
-  by_alignment(x, [&](auto al) {
+  by_alignment<gather_pairs<BC, DF>>(x, [&](auto al) {
     constexpr bool AL = decltype(al)::value;
   if (row < A.n_rows) {
     const int pe = A.rp[row + 1];
@@ -667,7 +682,7 @@ lpr_spmv_kernel(LprView A, const double* __restrict__ x, Epi epi) {
   [[maybe_unused]] float2 ad[BR];
 #pragma unroll
   for (int r = 0; r < BR; ++r) ad[r] = make_float2(0.f, 0.f);
-  by_alignment(x, [&](auto al) {
+  by_alignment<BC % 2 == 0>(x, [&](auto al) {
     constexpr bool AL = decltype(al)::value;
   if (row < A.n_rows) {
     const int g0 = A.gp[row], g1 = A.gp[row + 1];
@@ -679,7 +694,7 @@ lpr_spmv_kernel(LprView A, const double* __restrict__ x, Epi epi) {
       double xg[BC];
       if (g0 < g1) {
         const int c = __ldg(A.cols + (size_t)g0 * LPR + sub);
-        gather_x<BC, AL && BC != 3>(x, c, xg);
+        gather_x<BC, AL>(x, c, xg);
       }
       for (int g = g0; g < g1; ++g) {
         float2 vv[BB];
@@ -689,7 +704,7 @@ lpr_spmv_kernel(LprView A, const double* __restrict__ x, Epi epi) {
         for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
         if (g + 1 < g1) {
           const int c = __ldg(A.cols + (size_t)(g + 1) * LPR + sub);
-          gather_x<BC, AL && BC != 3>(x, c, xg);
+          gather_x<BC, AL>(x, c, xg);
         }
 #pragma unroll
         for (int r = 0; r < BR; ++r)
@@ -704,7 +719,7 @@ lpr_spmv_kernel(LprView A, const double* __restrict__ x, Epi epi) {
         for (int e = 0; e < BB; ++e) vv[e] = __ldg(vb + e * LPR);
         const int c = __ldg(A.cols + (size_t)g * LPR + sub);
         double xv[BC];
-        gather_x<BC, AL && BC != 3>(x, c, xv);
+        gather_x<BC, AL>(x, c, xv);
 #pragma unroll
         for (int r = 0; r < BR; ++r)
 #pragma unroll
@@ -760,7 +775,7 @@ lpr_rows_kernel(LprView A, const double* __restrict__ x, Epi epi) {
     float2 ad[BR];
 #pragma unroll
     for (int r = 0; r < BR; ++r) ad[r] = make_float2(0.f, 0.f);
-    by_alignment(x, [&](auto al) {
+    by_alignment<gather_pairs<BC, DF>>(x, [&](auto al) {
       constexpr bool AL = decltype(al)::value;
     if (row < A.n_rows) {
       const int g1 = A.gp[row + 1];
@@ -802,7 +817,7 @@ lpr_rows_kernel(LprView A, const double* __restrict__ x, Epi epi) {
   } else {
 #pragma unroll
     for (int r = 0; r < BR; ++r) acc[r] = 0.0;
-    by_alignment(x, [&](auto al) {
+    by_alignment<gather_pairs<BC, DF>>(x, [&](auto al) {
       constexpr bool AL = decltype(al)::value;
     if (row < A.n_rows) {
       const int g1 = A.gp[row + 1];
