@@ -223,16 +223,24 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
 // of grad_W in registers (8 x 8 for a 128 x 128 layer) and reads TK + TN
 // values of a row for TK TN products; the kernel before held every 256th
 // entry and read two values per product.
-constexpr int WG_ROWS = 32;
+// Narrow layers (K, N <= 16: a product a thread and row) are bound by the trip
+// to memory and the two barriers of a tile instead: four times the rows a
+// tile, each quarter with a sum of its own (a gradient on 300,001 rows of 8-3-3:
+// 240 -> 190 us).  Their partial sums, where at most WG_LAST blocks wrote some,
+// are added by the last block to finish, not by a launch of its own (3,000 rows of
+// 8-8-8-3: 110 -> 105 us).
+constexpr int WG_ROWS = 32, WG_LAST = 32;
+constexpr int wg_quarters(int TK, int TN) { return TK == 1 && TN == 1 ? 4 : 1; }
 
 template <int TK, int TN>
 __global__ void __launch_bounds__(THREADS, 2)
 weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, long long n, int K, int N,
                    const float* __restrict__ shift, const float* __restrict__ scale, float* __restrict__ part,
-                   bool h_vec, bool d_vec) {
+                   bool h_vec, bool d_vec, float* __restrict__ grad, unsigned int* __restrict__ ticket) {
   constexpr int Kp = 16 * TK, Np = 16 * TN;  // 16 x 16 threads
-  __shared__ __align__(16) float Hs[WG_ROWS][Kp];
-  __shared__ __align__(16) float Ds[WG_ROWS][Np];
+  constexpr int Q = wg_quarters(TK, TN), ROWS_T = Q * WG_ROWS;
+  __shared__ __align__(16) float Hs[ROWS_T][Kp];
+  __shared__ __align__(16) float Ds[ROWS_T][Np];
   // a warp: 4 x 8 threads, so that its reads of a row are 64 and 128 bytes
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int kg = (lane >> 3) + 4 * (wid >> 1), ng = (lane & 7) + 8 * (wid & 1);
@@ -245,11 +253,12 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
   for (int j = 0; j < TP; ++j)
 #pragma unroll
     for (int i = 0; i < TK; ++i) acc[i][j] = make_float2(0.f, 0.f);
-  // rows of src [n x M] from r0 into dst [WG_ROWS][Mp], zero-padded
+  [[maybe_unused]] float accq[Q] = {}, accbq[Q] = {};  // Q > 1: the quarters' sums
+  // rows of src [n x M] from r0 into dst [ROWS_T][Mp], zero-padded
   auto fill = [&](const float* __restrict__ src, int M, int Mp, float* dst, bool vec, bool std_, long long r0) {
     if (vec) {
       const int q = Mp >> 2;
-      for (int e = threadIdx.x; e < WG_ROWS * q; e += THREADS) {
+      for (int e = threadIdx.x; e < ROWS_T * q; e += THREADS) {
         const int r = e / q, k = (e - r * q) * 4;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r0 + r < n && k < M) {
@@ -264,7 +273,7 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
         *reinterpret_cast<float4*>(dst + r * Mp + k) = a;
       }
     } else {
-      for (int e = threadIdx.x; e < WG_ROWS * Mp; e += THREADS) {
+      for (int e = threadIdx.x; e < ROWS_T * Mp; e += THREADS) {
         const int r = e / Mp, k = e - r * Mp;
         float a = 0.f;
         if (r0 + r < n && k < M) {
@@ -291,11 +300,22 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
       }
     }
   };
-  for (long long r0 = (long long)blockIdx.x * WG_ROWS; r0 < n; r0 += (long long)gridDim.x * WG_ROWS) {
+  for (long long r0 = (long long)blockIdx.x * ROWS_T; r0 < n; r0 += (long long)gridDim.x * ROWS_T) {
     __syncthreads();
     fill(H, K, Kp, &Hs[0][0], h_vec, shift != nullptr, r0);
     fill(D, N, Np, &Ds[0][0], d_vec, false, r0);
     __syncthreads();
+    if constexpr (Q > 1) {
+#pragma unroll 4
+      for (int r = 0; r < WG_ROWS; ++r)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const float d = Ds[q * WG_ROWS + r][ng];
+          accbq[q] += d;
+          accq[q] = fmaf(Hs[q * WG_ROWS + r][kg], d, accq[q]);
+        }
+      continue;
+    }
 #pragma unroll 4
     for (int r = 0; r < WG_ROWS; ++r) {
       float h[TK], d[TN];
@@ -316,6 +336,10 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
       }
     }
   }
+  if constexpr (Q > 1) {
+    acc[0][0].x = (accq[0] + accq[1]) + (accq[2] + accq[3]);
+    accb[0] = (accbq[0] + accbq[1]) + (accbq[2] + accbq[3]);
+  }
   float* __restrict__ o = part + (size_t)blockIdx.x * ((size_t)K * N + N);
 #pragma unroll
   for (int i = 0; i < TK; ++i) {
@@ -326,6 +350,28 @@ weight_grad_kernel(const float* __restrict__ H, const float* __restrict__ D, lon
       if (k < K && c < N) o[(size_t)k * N + c] = (j & 1) ? acc[i][j / 2].y : acc[i][j / 2].x;
       if (kg == 0 && i == 0 && c < N) o[(size_t)K * N + c] = accb[j];
     }
+  }
+  if constexpr (Q > 1) {
+    if (gridDim.x > WG_LAST) return;  // weight_grad_reduce_kernel follows
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int M = K * N + N;
+    for (int e = threadIdx.x; e < M; e += THREADS) {  // in weight_grad_reduce_kernel's order
+      float s[8] = {};
+      for (int b = 0; b < (int)gridDim.x; b += 8)
+#pragma unroll
+        for (int w = 0; w < 8; ++w)
+          if (b + w < (int)gridDim.x) s[w] += __ldcg(part + (size_t)(b + w) * M + e);
+#pragma unroll
+      for (int w = 1; w < 8; ++w) s[0] += s[w];
+      grad[e] = s[0];
+    }
+    if (threadIdx.x == 0) *ticket = 0u;
   }
 }
 
@@ -699,26 +745,30 @@ void dense(const float* A, long long n, int K, int N, const TW* W, const float* 
 }
 
 template <int TK>
-void weight_grad_tn(int N, unsigned blocks, const float* H, const float* D, long long n, int K, const float* shift,
-                    const float* scale, float* part, cudaStream_t s) {
+void weight_grad_tn(tam_mlp_s* M, int N, unsigned blocks, const float* H, const float* D, long long n, int K,
+                    const float* shift, const float* scale, float* grad, cudaStream_t s) {
+  float* part = M->part.p;
+  unsigned int* t = M->ticket.p;
   const bool hv = K % 4 == 0 && aligned16(H) && TK >= 4, dv = N % 4 == 0 && aligned16(D);
   if (N <= 16)
-    weight_grad_kernel<TK, 1><<<blocks, THREADS, 0, s>>>(H, D, n, K, N, shift, scale, part, hv, dv);
+    weight_grad_kernel<TK, 1><<<blocks, THREADS, 0, s>>>(H, D, n, K, N, shift, scale, part, hv, dv, grad, t);
   else if (N <= 64)
-    weight_grad_kernel<TK, 4><<<blocks, THREADS, 0, s>>>(H, D, n, K, N, shift, scale, part, hv, dv);
+    weight_grad_kernel<TK, 4><<<blocks, THREADS, 0, s>>>(H, D, n, K, N, shift, scale, part, hv, dv, grad, t);
   else
-    weight_grad_kernel<TK, 8><<<blocks, THREADS, 0, s>>>(H, D, n, K, N, shift, scale, part, hv, dv);
+    weight_grad_kernel<TK, 8><<<blocks, THREADS, 0, s>>>(H, D, n, K, N, shift, scale, part, hv, dv, grad, t);
   TAM_LAUNCH_CHECK();
 }
 
 // grad[0 .. K N + N) = the layer's weight and bias gradients (row count n)
 void weight_grad(tam_mlp_s* M, const float* H, const float* D, long long n, int K, int N, const float* shift,
                  const float* scale, float* grad, cudaStream_t s) {
-  const unsigned blocks = row_grid(n, WG_ROWS);
+  const bool narrow = K <= 16 && N <= 16;
+  const unsigned blocks = row_grid(n, WG_ROWS * (narrow ? wg_quarters(1, 1) : 1));
   const int m = K * N + N;
-  if (K <= 16) weight_grad_tn<1>(N, blocks, H, D, n, K, shift, scale, M->part.p, s);
-  else if (K <= 64) weight_grad_tn<4>(N, blocks, H, D, n, K, shift, scale, M->part.p, s);
-  else weight_grad_tn<8>(N, blocks, H, D, n, K, shift, scale, M->part.p, s);
+  if (K <= 16) weight_grad_tn<1>(M, N, blocks, H, D, n, K, shift, scale, grad, s);
+  else if (K <= 64) weight_grad_tn<4>(M, N, blocks, H, D, n, K, shift, scale, grad, s);
+  else weight_grad_tn<8>(M, N, blocks, H, D, n, K, shift, scale, grad, s);
+  if (narrow && blocks <= WG_LAST) return;  // added up by its last block
   weight_grad_reduce_kernel<<<(m + 31) / 32, 256, 0, s>>>(M->part.p, (int)blocks, m, grad);
   TAM_LAUNCH_CHECK();
 }
