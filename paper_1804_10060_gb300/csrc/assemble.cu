@@ -924,7 +924,12 @@ tam_matrix_s* assemble_elasticity(int n_nodes, const double* coords, int n_cells
     M->vmax_exp = range.max_exp;
     M->finite = range.finite;
     M->df_ok = M->finite && std::abs(M->vmax_exp) <= kDfExpLimit;
-    if (!M->df_ok) M->S.vals_df.reset();
+    if (!M->df_ok) {
+      M->S.vals_df.reset();
+    } else if (!M->S.vals_df.p) {  // memory was short: out of memory for good, or not
+      alloc_split(M->S, s);
+      sell_refresh_values(A, M->S, s);
+    }
     if (M->df_ok && choose_lpr(A) != 0) build_df_values(A, s);
     TAM_CUDA(cudaStreamSynchronize(s));
   } catch (...) {

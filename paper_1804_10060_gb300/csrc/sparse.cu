@@ -99,6 +99,10 @@ static void read_range(const DBuf<int>& out, ExponentRange* range, cudaStream_t 
   range->finite = bad == 0;
 }
 
+void alloc_split(Sell& S, cudaStream_t s) {
+  S.vals_df = DBuf<float2>((size_t)std::max(1LL, S.n_slots * 32 * (long long)S.br * S.bc), s);
+}
+
 void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df, ExponentRange* range) {
   TAM_CHECK(A.n_cols > 0, TAM_ERR_INTERNAL, "SELL of a matrix without columns");
   S.n_rows = A.n_rows;
@@ -124,7 +128,13 @@ void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df, ExponentRange* 
   }
   S.cols = DBuf<int>((size_t)S.n_slots * 32, s);
   S.vals = DBuf<double>((size_t)S.n_slots * 32 * A.block_elems(), s);
-  if (df) S.vals_df = DBuf<float2>((size_t)std::max(1LL, S.n_slots * 32 * (long long)A.block_elems()), s);
+  if (df) {
+    try {
+      alloc_split(S, s);
+    } catch (const Error& e) {
+      if (!range || e.code != TAM_ERR_OOM) throw;  // the caller may not need it, see assemble_elasticity
+    }
+  }
   DBuf<int> out;
   if (range) {
     out = DBuf<int>(2, s);

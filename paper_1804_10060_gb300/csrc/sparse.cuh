@@ -244,8 +244,10 @@ __device__ __forceinline__ int sell_row(const int* __restrict__ perm, int pos, i
 void build_df_values(Bsr& B, cudaStream_t s);
 
 // Builds the SELL-32 copy of a Bsr (pattern + values).
-// df: the split copy too; range: the values' exponent range (then synchronising)
+// df: the split copy too; range: the values' exponent range (then synchronising,
+// and the split copy is left out, not an error, when memory does not reach for it)
 void bsr_to_sell(const Bsr& A, Sell& S, cudaStream_t s, bool df = false, ExponentRange* range = nullptr);
+void alloc_split(Sell& S, cudaStream_t s);
 // Refreshes only the values of an existing SELL copy built from A (and its
 // split copy, when it has one).
 void sell_refresh_values(const Bsr& A, Sell& S, cudaStream_t s, ExponentRange* range = nullptr);
