@@ -773,15 +773,15 @@ gj_coop_kernel(double* __restrict__ D, int ld, double* __restrict__ cpan, double
   }
 }
 
-// The inverse out of the padded working matrix: rows and columns of inactive
-// unknowns zero; sym: tiles above the diagonal from below it.
-__global__ void dense_out_kernel(const double* __restrict__ W, int ld, int N, const unsigned char* __restrict__ inactive,
-                                 int sym, double* __restrict__ out) {
+// After the elimination, in place: rows and columns of inactive unknowns zero;
+// sym: tiles above the diagonal from below it (which only the zeros change).
+__global__ void dense_finish_kernel(double* __restrict__ D, int ld, int N, const unsigned char* __restrict__ inactive,
+                                    int sym) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   int i = blockIdx.y;
   if (j >= N) return;
-  const bool mirror = sym && j / GJB > i / GJB;
-  out[(size_t)i * N + j] = (inactive[i] || inactive[j]) ? 0.0 : (mirror ? W[(size_t)j * ld + i] : W[(size_t)i * ld + j]);
+  if (inactive[i] || inactive[j]) D[(size_t)i * ld + j] = 0.0;
+  else if (sym && j / GJB > i / GJB) D[(size_t)i * ld + j] = D[(size_t)j * ld + i];
 }
 
 }  // namespace
@@ -1014,8 +1014,9 @@ static void coarse_inverse(tam_amg_s* H, const Level& L, bool sym, cudaStream_t 
   const int N = L.n_rows * L.bs, ld = (N + GJB - 1) / GJB * GJB;
   TAM_CHECK(N <= 12000, TAM_ERR_UNSUPPORTED, "amg_setup: coarsest level too large for the dense solve");
   H->n_coarse = N;
-  H->coarse_inv = DBuf<double>((size_t)N * N, s);
-  DBuf<double> W((size_t)ld * ld, s);
+  H->coarse_ld = ld;  // the result stays in the padded matrix: a copy of 12,000 rows would be another 1.15 GB
+  H->coarse_inv = DBuf<double>((size_t)ld * ld, s);
+  DBuf<double>& W = H->coarse_inv;
   W.zero();
   const Bsr& A = *L.A;
   bsr_to_dense_kernel<<<grid_for((long long)L.n_rows * 32, TPB), TPB, 0, s>>>(A.row_ptr.p, A.col_idx.p, A.vals.p,
@@ -1041,7 +1042,7 @@ static void coarse_inverse(tam_amg_s* H, const Level& L, bool sym, cudaStream_t 
   void* args[] = {&wp, &ld_arg, &cp, &rp, &pp, &bp};
   TAM_CUDA(cudaLaunchCooperativeKernel(kern, dim3(sm_count()), dim3(GJ_THREADS), args, 0, s));
   TAM_LAUNCH_CHECK();
-  dense_out_kernel<<<dim3(grid_for(N, TPB), N), TPB, 0, s>>>(W.p, ld, N, inactive.p, sym ? 1 : 0, H->coarse_inv.p);
+  dense_finish_kernel<<<dim3(grid_for(N, TPB), N), TPB, 0, s>>>(W.p, ld, N, inactive.p, sym ? 1 : 0);
   TAM_LAUNCH_CHECK();
   TAM_CHECK(read_back_int(bad.p, s) == 0, TAM_ERR_INTERNAL, "amg_setup: coarsest operator is not positive definite");
 }

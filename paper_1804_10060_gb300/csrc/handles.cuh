@@ -123,7 +123,8 @@ struct tam_amg_s {
   amg_params prm{};
   std::vector<tam::Level> levels;
   int n_coarse = 0;                      // dense coarsest size (scalars)
-  tam::DBuf<double> coarse_inv;          // [n_coarse * n_coarse]
+  int coarse_ld = 0;                     // its inverse's leading dimension
+  tam::DBuf<double> coarse_inv;          // [coarse_ld * coarse_ld], rows and columns past n_coarse unused
   // PCG workspace
   tam::DBuf<double> r, z, p, q;
   tam::DBuf<float2> ps;                  // p split, where the products read it so (split_beforehand)

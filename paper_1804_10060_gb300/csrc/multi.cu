@@ -714,13 +714,13 @@ __global__ void mfirst_kernel(const TB* __restrict__ b, const float* __restrict_
 // columns (a thread per output walked N columns alone, one dependent FP64
 // multiply-add after the other).
 template <typename TI, typename TO>
-__global__ void mcoarse_kernel(const double* __restrict__ A, const TI* __restrict__ b, TO* __restrict__ y, int N, int mp,
-                               const int* __restrict__ stop) {
+__global__ void mcoarse_kernel(const double* __restrict__ A, const TI* __restrict__ b, TO* __restrict__ y, int N, int ld,
+                               int mp, const int* __restrict__ stop) {
   if (stop && *stop) return;
   const int i = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (i >= N) return;
   const int j0 = blockIdx.y * 8;
-  const double* __restrict__ a = A + (size_t)i * N;
+  const double* __restrict__ a = A + (size_t)i * ld;
   double s[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) s[k] = 0.0;
@@ -795,7 +795,7 @@ void mvcycle(tam_amg_s* H, int l, const TB* b, TO* out, const int* stop, cudaStr
   MultiLevel& ML = MS.lv[l];
   if (l == (int)H->levels.size() - 1) {
     mcoarse_kernel<TB, TO><<<dim3(grid_for((long long)H->n_coarse * 32, TPB), mp / 8), TPB, 0, s>>>(
-        H->coarse_inv.p, b, out, H->n_coarse, mp, stop);
+        H->coarse_inv.p, b, out, H->n_coarse, H->coarse_ld, mp, stop);
     TAM_LAUNCH_CHECK();
     return;
   }

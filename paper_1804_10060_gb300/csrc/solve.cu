@@ -88,11 +88,11 @@ struct EpiCheb {
 
 // y = Ainv b (dense), warp per row
 __global__ void dense_gemv_kernel(const double* __restrict__ A, const double* __restrict__ b, double* __restrict__ y,
-                                  int N, const int* __restrict__ stop) {
+                                  int N, int ld, const int* __restrict__ stop) {
   if (stop && *stop) return;
   int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= N) return;
-  const double* a = A + (size_t)row * N;
+  const double* a = A + (size_t)row * ld;
   double s = 0.0;
   for (int j = lane; j < N; j += 32) s = fma(a[j], b[j], s);
   s = warp_sum(s);
@@ -385,7 +385,7 @@ void vcycle_level(tam_amg_s* H, int l, const double* b, double* out, const int* 
   const long long N = (long long)L.n_rows * L.bs;
   if (l == (int)H->levels.size() - 1) {
     dense_gemv_kernel<<<grid_for((long long)H->n_coarse * 32, TPB), TPB, 0, s>>>(H->coarse_inv.p, b, out,
-                                                                                  H->n_coarse, stop);
+                                                                                  H->n_coarse, H->coarse_ld, stop);
     TAM_LAUNCH_CHECK();
     return;
   }

@@ -143,11 +143,11 @@ struct EpiAddF {
 // dot products; y: records of bs entries in FP32, packed in FP64
 template <typename TI, typename TO>
 __global__ void dense_gemv_mixed_kernel(const double* __restrict__ A, const TI* __restrict__ b, TO* __restrict__ y,
-                                        int N, int bs, const int* __restrict__ stop) {
+                                        int N, int ld, int bs, const int* __restrict__ stop) {
   if (stop && *stop) return;
   int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= N) return;
-  const double* a = A + (size_t)row * N;
+  const double* a = A + (size_t)row * ld;
   double s = 0.0;
   for (int j = lane; j < N; j += 32) s = fma(a[j], (double)b[j], s);
   s = warp_sum(s);
@@ -206,7 +206,7 @@ void vcycle_low(tam_amg_s* H, int l, const TB* b, TO* out, const int* stop, cuda
   Level& L = H->levels[l];
   if (l == (int)H->levels.size() - 1) {
     dense_gemv_mixed_kernel<TB, TO><<<grid_for((long long)H->n_coarse * 32, TPB), TPB, 0, s>>>(
-        H->coarse_inv.p, b, out, H->n_coarse, L.bs, stop);
+        H->coarse_inv.p, b, out, H->n_coarse, H->coarse_ld, L.bs, stop);
     TAM_LAUNCH_CHECK();
     return;
   }

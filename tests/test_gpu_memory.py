@@ -84,3 +84,33 @@ def test_matrix_outside_the_range_needs_no_split_copy():
 
     pools.limited(limit, short)
     pools.limited(peak + (1 << 28), lambda: assemble(d))
+
+
+@pytest.mark.parametrize("n_rhs", [0, 3])
+def test_coarsest_inverse_in_place(n_rhs):
+    """A hierarchy of one level of 5,202 unknowns: setup needs the 216 MB of its inverse and little else (K takes
+    8 MB), in the V-cycles of both precisions and in the batch."""
+    tam = need_gpu()
+    pools = Pools()
+    pb = meshgen.slab_box_problem(16, 16, 5)
+    d = tam.problem_to_device(pb)
+    K, rhs = tam.fem_assemble_elasticity(**d)
+    prm = tam.amg_params_default(coarse_max_dofs=6000, level_precision=1 if n_rhs else 0)
+    N = 3 * pb.n_nodes
+    hs = []
+    peak = pools.peak(lambda: hs.append(tam.amg_setup(K, d["coords"], prm)))
+    H = hs[0]
+    assert tam.amg_info(H)["n_levels"] == 1 and N > 5000
+    assert 8 * N * N <= peak <= 1.25 * 8 * N * N
+    free = d["dirichlet_mask"] == 0
+    r = torch.randn((pb.n_nodes, 3), dtype=torch.float64, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    r[~free] = 0.0
+    if n_rhs:
+        B = torch.stack([r.reshape(-1) * (k + 1) for k in range(n_rhs)])
+        X = torch.zeros_like(B)
+        its, _, _ = tam.amg_pcg_solve_batch([H], [B], [X], rtol=1e-10)
+        assert max(its) <= 2
+        z = (X[-1] / n_rhs).reshape(r.shape)
+    else:
+        z = tam.amg_vcycle(H, r)
+    assert tam.tam_matrix_residual_norm(K, r, z) <= 1e-8 * float(r.norm())
