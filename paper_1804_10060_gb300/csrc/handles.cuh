@@ -146,6 +146,8 @@ struct tam_amg_s {
   int smooth_deg = 0;
   double smooth_lo = 0.0, smooth_hi = 0.0;
   std::unique_ptr<tam::MultiState> multi;  // multi-RHS workspace (built on first use)
+  // whether every level's reduced-precision data, and the batched solve's operators, are there
+  bool low_ready = false, batch_ready = false;
   ~tam_amg_s();
 };
 
@@ -187,6 +189,9 @@ inline bool split_beforehand(const Level& L) {
 void build_low_precision(tam_amg_s* H, cudaStream_t s);
 // The batched solve's operators, after build_low_precision.
 void build_batch_operators(tam_amg_s* H, cudaStream_t s);
+// Both given back, whole or in part.
+void release_low_precision(tam_amg_s* H);
+void release_batch_operators(tam_amg_s* H);
 // x <- degree Chebyshev-Jacobi steps on K x = b from x over [lo, hi] * lambda_max(D^-1 K)
 void smooth_fine(tam_amg_s* H, const double* b, double* x, int degree, double lo, double hi, cudaStream_t s);
 

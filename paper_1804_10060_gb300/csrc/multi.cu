@@ -915,10 +915,8 @@ void autotune(tam_amg_s* H, cudaStream_t s) {
   MS.tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
 }
 
-void ensure_multi(tam_amg_s* H, int mp, cudaStream_t s) {
-  if (!H->levels[0].dinv32.p) build_low_precision(H, s);
-  if (!H->levels[0].A32m.vals && !H->levels[0].A16m.vals) build_batch_operators(H, s);
-  if (H->multi && H->multi->mp == mp) return;
+// The workspace of a batch of mp (padded) right-hand sides, and its tiles.
+void build_multi(tam_amg_s* H, int mp, cudaStream_t s) {
   static std::atomic<unsigned long long> serials{0};
   H->multi.reset(new MultiState());
   MultiState& MS = *H->multi;
@@ -947,6 +945,21 @@ void ensure_multi(tam_amg_s* H, int mp, cudaStream_t s) {
     }
   }
   autotune(H, s);
+}
+
+// A call that fails here (out of memory) leaves the hierarchy as it was.
+void ensure_multi(tam_amg_s* H, int mp, cudaStream_t s) {
+  const bool had_low = H->low_ready, had_batch = H->batch_ready;
+  try {
+    if (!had_low) build_low_precision(H, s);
+    if (!had_batch) build_batch_operators(H, s);
+    if (!H->multi || H->multi->mp != mp) build_multi(H, mp, s);
+  } catch (...) {
+    H->multi.reset();
+    if (!had_batch) release_batch_operators(H);
+    if (!had_low) release_low_precision(H);
+    throw;
+  }
 }
 
 void enqueue_multi_iteration(tam_amg_s* H, cudaStream_t s) {

@@ -278,6 +278,7 @@ void build_low_precision(tam_amg_s* H, cudaStream_t s) {
     convert_values_f32(L.Rop, L.R32v, s);
     L.R32 = SpOpLow<float>{L.Rop, L.R32v.p};
   }
+  H->low_ready = true;
 }
 
 void build_batch_operators(tam_amg_s* H, cudaStream_t s) {
@@ -297,6 +298,28 @@ void build_batch_operators(tam_amg_s* H, cudaStream_t s) {
       L.A16m.vals = L.A16mv.p;
     }
   }
+  H->batch_ready = true;
+}
+
+void release_low_precision(tam_amg_s* H) {
+  for (Level& L : H->levels) {
+    for (auto* v : {&L.dinv32, &L.consts32, &L.b32, &L.y32, &L.xa32, &L.xb32, &L.d32, &L.t32, &L.A32v, &L.P32v, &L.R32v})
+      v->reset();
+    L.A16v.reset();
+    L.A32 = L.P32 = L.R32 = SpOpLow<float>{};
+    L.A16 = SpOpLow<__nv_bfloat16>{};
+  }
+  H->low_ready = false;
+}
+
+void release_batch_operators(tam_amg_s* H) {
+  for (Level& L : H->levels) {
+    for (auto* v : {&L.A32mv, &L.P32mv, &L.R32mv}) v->reset();
+    L.A16mv.reset();
+    L.A32m = L.P32m = L.R32m = SpOpLow<float>{};
+    L.A16m = SpOpLow<__nv_bfloat16>{};
+  }
+  H->batch_ready = false;
 }
 
 }  // namespace tam

@@ -27,9 +27,9 @@ class Pools:
     def ok(self, r):
         assert r == 0, r
 
-    def get(self, attr):
+    def get(self, attr, pool=None):
         v = ctypes.c_uint64()
-        self.ok(self.cu.cuMemPoolGetAttribute(self.default, attr, ctypes.byref(v)))
+        self.ok(self.cu.cuMemPoolGetAttribute(pool or self.default, attr, ctypes.byref(v)))
         return v.value
 
     def peak(self, f):
@@ -51,7 +51,9 @@ class Pools:
             torch.cuda.synchronize()
         finally:
             self.ok(self.cu.cuDeviceSetMemPool(0, self.default))
-            self.ok(self.cu.cuMemPoolDestroy(pool))
+        torch.cuda.synchronize()
+        assert self.get(USED_CURRENT, pool) == 0  # whatever f() took is given back
+        self.ok(self.cu.cuMemPoolDestroy(pool))
 
 
 def test_matrix_outside_the_range_needs_no_split_copy():
@@ -114,3 +116,38 @@ def test_coarsest_inverse_in_place(n_rhs):
     else:
         z = tam.amg_vcycle(H, r)
     assert tam.tam_matrix_residual_norm(K, r, z) <= 1e-8 * float(r.norm())
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_batch_after_running_out_of_memory(precision):
+    """A batched solve that runs out of memory, at any stage of building its operators and workspace, says so and
+    gives back what it took; a later call with enough memory gives the solutions of a hierarchy that never did."""
+    tam = need_gpu()
+    pools = Pools()
+    pb = meshgen.slab_box_problem(96, 24, 24)
+    d = tam.problem_to_device(pb)
+    K, rhs = tam.fem_assemble_elasticity(**d)
+    prm = tam.amg_params_default(level_precision=precision)
+    B = torch.stack([rhs.reshape(-1) * (k + 1) for k in range(8)])
+
+    def solve(H):
+        X = torch.zeros_like(B)
+        tam.amg_pcg_solve_batch([H], [B], [X], rtol=1e-8)
+        return X
+
+    fresh = tam.amg_setup(K, d["coords"], prm)
+    ref = []
+    peak = pools.peak(lambda: ref.append(solve(fresh)))
+    fresh.destroy()
+    H = tam.amg_setup(K, d["coords"], prm)
+
+    def short():
+        with pytest.raises(tam.TamError) as e:
+            solve(H)
+            pytest.skip("the driver does not limit the pool")
+        assert e.value.code == -3, e.value  # TAM_ERR_OOM
+
+    for part in (0.05, 0.2, 0.35, 0.5, 0.65, 0.8):
+        pools.limited(int(part * peak), short)
+    X = solve(H)
+    assert float((X - ref[0]).norm()) <= 1e-6 * float(ref[0].norm())
