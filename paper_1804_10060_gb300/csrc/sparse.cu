@@ -1223,8 +1223,8 @@ __global__ void convert_slots_kernel(const double* __restrict__ in, T* __restric
 }
 
 template <typename T>
-void convert_values(const SpOp& op, DBuf<T>& out, cudaStream_t s, bool batch) {
-  const bool store = !batch && low_in_store(op);
+void convert_values(const SpOp& op, DBuf<T>& out, cudaStream_t s) {
+  const bool store = low_in_store(op);
   const int bb = (int)op.B->block_elems();
   const long long blocks = op.lpr == 0 ? op.S->n_slots * 32 : (store ? op.L->n_groups * op.L->lpr : op.B->nnzb);
   const long long n = blocks * bb;
@@ -1238,11 +1238,9 @@ void convert_values(const SpOp& op, DBuf<T>& out, cudaStream_t s, bool batch) {
 }
 }  // namespace
 
-void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s, bool batch) {
-  convert_values<float>(op, out, s, batch);
-}
-void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s, bool batch) {
-  convert_values<__nv_bfloat16>(op, out, s, batch);
+void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s) { convert_values<float>(op, out, s); }
+void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s) {
+  convert_values<__nv_bfloat16>(op, out, s);
 }
 
 }  // namespace tam

@@ -1464,8 +1464,8 @@ blockrow_f32_kernel(int n_rows, const int* __restrict__ rp, const int* __restric
 
 // A reduced-precision operator: the pattern of `op` with values `vals` in the
 // order of the kernel that runs it -- SELL or lanes-per-row store (packed), or
-// the block-CSR arrays.  The batched solve's copies (`batch`) keep block-CSR
-// order wherever the operator is not SELL.
+// the block-CSR arrays.  The batched solve's copies keep block-CSR order
+// wherever the operator is not SELL (in_block_csr).
 template <typename TV>
 struct SpOpLow {
   SpOp op;
@@ -1474,6 +1474,11 @@ struct SpOpLow {
 
 // Whether the values of op's reduced-precision copy follow its lanes-per-row store
 inline bool low_in_store(const SpOp& op) { return op.L && !op.tpr; }
+// op with a copy in block-CSR order instead of its lanes-per-row store's
+inline SpOp in_block_csr(SpOp op) {
+  if (low_in_store(op)) op.L = nullptr;
+  return op;
+}
 
 template <int BR, int BC, typename TV, class Epi>
 void spop_apply_f32(const SpOpLow<TV>& o, const float* x, Epi epi, cudaStream_t s) {
@@ -1524,9 +1529,9 @@ void spop_apply_f32(const SpOpLow<TV>& o, const float* x, Epi epi, cudaStream_t 
   TAM_LAUNCH_CHECK();
 }
 
-// Values of `op` as a reduced-precision copy, in SpOpLow's order (batch: the batched solve's).
-void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s, bool batch = false);
-void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s, bool batch = false);
+// Values of `op` as a reduced-precision copy, in SpOpLow's order.
+void convert_values_f32(const SpOp& op, DBuf<float>& out, cudaStream_t s);
+void convert_values_bf16(const SpOp& op, DBuf<__nv_bfloat16>& out, cudaStream_t s);
 
 // --- common epilogues ------------------------------------------------------
 struct NoStop {

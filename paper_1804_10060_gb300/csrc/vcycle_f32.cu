@@ -247,6 +247,12 @@ void vcycle_apply_low(tam_amg_s* H, const double* r, double* z, const int* stop,
 
 void build_low_precision(tam_amg_s* H, cudaStream_t s) {
   const int mode = H->prm.level_precision;
+  // level_precision 0: for the batched solve alone, which reads block-CSR order
+  auto order = [&](const SpOp& op) { return mode == 0 ? in_block_csr(op) : op; };
+  auto low_copy = [&](const SpOp& op, DBuf<float>& v) {
+    convert_values_f32(op, v, s);
+    return SpOpLow<float>{op, v.p};
+  };
   for (size_t l = 0; l < H->levels.size(); ++l) {
     Level& L = H->levels[l];
     const size_t N = (size_t)L.n_rows * L.bs;
@@ -270,13 +276,10 @@ void build_low_precision(tam_amg_s* H, cudaStream_t s) {
       convert_values_bf16(L.Aop, L.A16v, s);
       L.A16 = SpOpLow<__nv_bfloat16>{L.Aop, L.A16v.p};
     } else {
-      convert_values_f32(L.Aop, L.A32v, s);
-      L.A32 = SpOpLow<float>{L.Aop, L.A32v.p};
+      L.A32 = low_copy(order(L.Aop), L.A32v);
     }
-    convert_values_f32(L.Pop, L.P32v, s);
-    L.P32 = SpOpLow<float>{L.Pop, L.P32v.p};
-    convert_values_f32(L.Rop, L.R32v, s);
-    L.R32 = SpOpLow<float>{L.Rop, L.R32v.p};
+    L.P32 = low_copy(order(L.Pop), L.P32v);
+    L.R32 = low_copy(order(L.Rop), L.R32v);
   }
   H->low_ready = true;
 }
@@ -286,16 +289,16 @@ void build_batch_operators(tam_amg_s* H, cudaStream_t s) {
     Level& L = H->levels[l];
     auto own = [&](const SpOpLow<float>& o, DBuf<float>& v) {
       if (!o.vals || !low_in_store(o.op)) return o;
-      convert_values_f32(o.op, v, s, true);
-      return SpOpLow<float>{o.op, v.p};
+      convert_values_f32(in_block_csr(o.op), v, s);
+      return SpOpLow<float>{in_block_csr(o.op), v.p};
     };
     L.A32m = own(L.A32, L.A32mv);
     L.P32m = own(L.P32, L.P32mv);
     L.R32m = own(L.R32, L.R32mv);
     L.A16m = L.A16;
     if (L.A16.vals && low_in_store(L.A16.op)) {
-      convert_values_bf16(L.A16.op, L.A16mv, s, true);
-      L.A16m.vals = L.A16mv.p;
+      convert_values_bf16(in_block_csr(L.A16.op), L.A16mv, s);
+      L.A16m = SpOpLow<__nv_bfloat16>{in_block_csr(L.A16.op), L.A16mv.p};
     }
   }
   H->batch_ready = true;

@@ -151,3 +151,35 @@ def test_batch_after_running_out_of_memory(precision):
         pools.limited(int(part * peak), short)
     X = solve(H)
     assert float((X - ref[0]).norm()) <= 1e-6 * float(ref[0].norm())
+
+
+def test_batch_operators_are_not_kept_twice():
+    """The batched solve on an FP64 hierarchy keeps one FP32 copy of every operator.  Copies and workspace are those
+    of an FP32 hierarchy and its own batch, less the latter's second copies of the operators whose solves read a
+    lanes-per-row store (at least 100 MB on this machine, whose first restriction is one)."""
+    tam = need_gpu()
+    pools = Pools()
+    pb = meshgen.slab_box_problem(256, 64, 64)
+    d = tam.problem_to_device(pb)
+    K, rhs = tam.fem_assemble_elasticity(**d)
+    B = torch.stack([rhs.reshape(-1)] * 2)
+
+    def batch(H):
+        X = torch.zeros_like(B)
+        tam.amg_pcg_solve_batch([H], [B], [X], rtol=1e-8, max_iter=2, raise_on_error=False)
+
+    kept, extra = [], []
+    for precision in (0, 1):
+        before = pools.get(USED_CURRENT)
+        H = tam.amg_setup(K, d["coords"], tam.amg_params_default(level_precision=precision))
+        kept.append(pools.get(USED_CURRENT) - before)
+        extra.append(pools.peak(lambda: batch(H)))
+        twice = 0
+        for l in range(tam.amg_info(H)["n_levels"] - 1):
+            for which in range(3):  # A, P, R
+                if tam.amg_level_spmv_plan(H, l, which)["kind"] == 1:
+                    e = tam.amg_level_export(H, l, which)
+                    twice += 4 * e["nnzb"] * e["br"] * e["bc"]
+        H.destroy()
+    assert twice > 100e6
+    assert extra[0] <= kept[1] - kept[0] + extra[1] - 0.9 * twice
