@@ -596,42 +596,42 @@ bsr_vector_kernel(BsrView A, const double* __restrict__ x, Epi epi) {
   for (int r = 0; r < BR; ++r) acc[r] = 0.0;
   by_alignment<gather_pairs<BC, DF>>(x, [&](auto al) {
     constexpr bool AL = decltype(al)::value;
-  if (row < A.n_rows) {
-    const int pe = A.rp[row + 1];
-    if constexpr (DF) {
-      float2 ad[BR];
+    if (row < A.n_rows) {
+      const int pe = A.rp[row + 1];
+      if constexpr (DF) {
+        float2 ad[BR];
 #pragma unroll
-      for (int r = 0; r < BR; ++r) ad[r] = make_float2(0.f, 0.f);
-      for (int p = A.rp[row] + sub; p < pe; p += LPR) {
-        float2 vv[BR * BC];  // the whole block first (16-byte loads), then the gather
-        block_load<BR * BC>(A.v_df + (size_t)p * BR * BC, vv);
-        const int c = A.ci[p];
-        double xg[BC];
-        gather_x<BC, AL>(x, c, xg);
-        float2 xv[BC];
+        for (int r = 0; r < BR; ++r) ad[r] = make_float2(0.f, 0.f);
+        for (int p = A.rp[row] + sub; p < pe; p += LPR) {
+          float2 vv[BR * BC];  // the whole block first (16-byte loads), then the gather
+          block_load<BR * BC>(A.v_df + (size_t)p * BR * BC, vv);
+          const int c = A.ci[p];
+          double xg[BC];
+          gather_x<BC, AL>(x, c, xg);
+          float2 xv[BC];
 #pragma unroll
-        for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
+          for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
 #pragma unroll
-        for (int r = 0; r < BR; ++r)
+          for (int r = 0; r < BR; ++r)
 #pragma unroll
-          for (int j = 0; j < BC; ++j) df_fma(ad[r], vv[r * BC + j], xv[j]);
-      }
+            for (int j = 0; j < BC; ++j) df_fma(ad[r], vv[r * BC + j], xv[j]);
+        }
 #pragma unroll
-      for (int r = 0; r < BR; ++r) acc[r] = df_to_double(ad[r]);
-    } else {
-      for (int p = A.rp[row] + sub; p < pe; p += LPR) {
-        double vv[BR * BC];
-        block_load<BR * BC>(A.v + (size_t)p * BR * BC, vv);
-        const int c = A.ci[p];
-        double xv[BC];
-        gather_x<BC, AL>(x, c, xv);
+        for (int r = 0; r < BR; ++r) acc[r] = df_to_double(ad[r]);
+      } else {
+        for (int p = A.rp[row] + sub; p < pe; p += LPR) {
+          double vv[BR * BC];
+          block_load<BR * BC>(A.v + (size_t)p * BR * BC, vv);
+          const int c = A.ci[p];
+          double xv[BC];
+          gather_x<BC, AL>(x, c, xv);
 #pragma unroll
-        for (int r = 0; r < BR; ++r)
+          for (int r = 0; r < BR; ++r)
 #pragma unroll
-          for (int j = 0; j < BC; ++j) acc[r] = fma(vv[r * BC + j], xv[j], acc[r]);
+            for (int j = 0; j < BC; ++j) acc[r] = fma(vv[r * BC + j], xv[j], acc[r]);
+        }
       }
     }
-  }
   });
 #pragma unroll
   for (int o = LPR / 2; o > 0; o >>= 1)
@@ -686,49 +686,49 @@ lpr_spmv_kernel(LprView A, const double* __restrict__ x, Epi epi) {
   for (int r = 0; r < BR; ++r) ad[r] = make_float2(0.f, 0.f);
   by_alignment<BC % 2 == 0>(x, [&](auto al) {
     constexpr bool AL = decltype(al)::value;
-  if (row < A.n_rows) {
-    const int g0 = A.gp[row], g1 = A.gp[row + 1];
-    if constexpr (DF) {
-      // the x gather runs one group ahead: the next group's column and x
-      // entries are requested before this group's products, so that they
-      // arrive together with the next group's values (one memory round trip
-      // per group instead of values, then column and gather)
-      double xg[BC];
-      if (g0 < g1) {
-        const int c = __ldg(A.cols + (size_t)g0 * LPR + sub);
-        gather_x<BC, AL>(x, c, xg);
-      }
-      for (int g = g0; g < g1; ++g) {
-        float2 vv[BB];
-        slot_load<BB, LPR>(A.v_df + (size_t)g * BB * LPR, sub, vv);
-        float2 xv[BC];
-#pragma unroll
-        for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
-        if (g + 1 < g1) {
-          const int c = __ldg(A.cols + (size_t)(g + 1) * LPR + sub);
+    if (row < A.n_rows) {
+      const int g0 = A.gp[row], g1 = A.gp[row + 1];
+      if constexpr (DF) {
+        // the x gather runs one group ahead: the next group's column and x
+        // entries are requested before this group's products, so that they
+        // arrive together with the next group's values (one memory round trip
+        // per group instead of values, then column and gather)
+        double xg[BC];
+        if (g0 < g1) {
+          const int c = __ldg(A.cols + (size_t)g0 * LPR + sub);
           gather_x<BC, AL>(x, c, xg);
         }
+        for (int g = g0; g < g1; ++g) {
+          float2 vv[BB];
+          slot_load<BB, LPR>(A.v_df + (size_t)g * BB * LPR, sub, vv);
+          float2 xv[BC];
 #pragma unroll
-        for (int r = 0; r < BR; ++r)
+          for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
+          if (g + 1 < g1) {
+            const int c = __ldg(A.cols + (size_t)(g + 1) * LPR + sub);
+            gather_x<BC, AL>(x, c, xg);
+          }
 #pragma unroll
-          for (int j = 0; j < BC; ++j) df_fma(ad[r], vv[r * BC + j], xv[j]);
-      }
-    } else {
-      for (int g = g0; g < g1; ++g) {
-        const double* __restrict__ vb = A.v + (size_t)g * BB * LPR + sub;
-        double vv[BB];
+          for (int r = 0; r < BR; ++r)
 #pragma unroll
-        for (int e = 0; e < BB; ++e) vv[e] = __ldg(vb + e * LPR);
-        const int c = __ldg(A.cols + (size_t)g * LPR + sub);
-        double xv[BC];
-        gather_x<BC, AL>(x, c, xv);
+            for (int j = 0; j < BC; ++j) df_fma(ad[r], vv[r * BC + j], xv[j]);
+        }
+      } else {
+        for (int g = g0; g < g1; ++g) {
+          const double* __restrict__ vb = A.v + (size_t)g * BB * LPR + sub;
+          double vv[BB];
 #pragma unroll
-        for (int r = 0; r < BR; ++r)
+          for (int e = 0; e < BB; ++e) vv[e] = __ldg(vb + e * LPR);
+          const int c = __ldg(A.cols + (size_t)g * LPR + sub);
+          double xv[BC];
+          gather_x<BC, AL>(x, c, xv);
 #pragma unroll
-          for (int j = 0; j < BC; ++j) acc[r] = fma(vv[r * BC + j], xv[j], acc[r]);
+          for (int r = 0; r < BR; ++r)
+#pragma unroll
+            for (int j = 0; j < BC; ++j) acc[r] = fma(vv[r * BC + j], xv[j], acc[r]);
+        }
       }
     }
-  }
   });
   if constexpr (DF) {
     // the lanes' partial sums combined in double-float (FP32 work: an FP64
@@ -779,23 +779,23 @@ lpr_rows_kernel(LprView A, const double* __restrict__ x, Epi epi) {
     for (int r = 0; r < BR; ++r) ad[r] = make_float2(0.f, 0.f);
     by_alignment<gather_pairs<BC, DF>>(x, [&](auto al) {
       constexpr bool AL = decltype(al)::value;
-    if (row < A.n_rows) {
-      const int g1 = A.gp[row + 1];
-      for (int g = A.gp[row] + sub / ROWS_LPR; g < g1; g += GS) {
-        float2 vv[BB];
-        slot_load<BB, ROWS_LPR>(A.v_df + (size_t)g * BB * ROWS_LPR, ln, vv);
-        const int c = __ldg(A.cols + (size_t)g * ROWS_LPR + ln);
-        double xg[BC];
-        gather_x<BC, AL>(x, c, xg);
-        float2 xv[BC];
+      if (row < A.n_rows) {
+        const int g1 = A.gp[row + 1];
+        for (int g = A.gp[row] + sub / ROWS_LPR; g < g1; g += GS) {
+          float2 vv[BB];
+          slot_load<BB, ROWS_LPR>(A.v_df + (size_t)g * BB * ROWS_LPR, ln, vv);
+          const int c = __ldg(A.cols + (size_t)g * ROWS_LPR + ln);
+          double xg[BC];
+          gather_x<BC, AL>(x, c, xg);
+          float2 xv[BC];
 #pragma unroll
-        for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
+          for (int j = 0; j < BC; ++j) xv[j] = split_bits(xg[j]);
 #pragma unroll
-        for (int r = 0; r < BR; ++r)
+          for (int r = 0; r < BR; ++r)
 #pragma unroll
-          for (int j = 0; j < BC; ++j) df_fma(ad[r], vv[r * BC + j], xv[j]);
+            for (int j = 0; j < BC; ++j) df_fma(ad[r], vv[r * BC + j], xv[j]);
+        }
       }
-    }
     });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
@@ -821,22 +821,22 @@ lpr_rows_kernel(LprView A, const double* __restrict__ x, Epi epi) {
     for (int r = 0; r < BR; ++r) acc[r] = 0.0;
     by_alignment<gather_pairs<BC, DF>>(x, [&](auto al) {
       constexpr bool AL = decltype(al)::value;
-    if (row < A.n_rows) {
-      const int g1 = A.gp[row + 1];
-      for (int g = A.gp[row] + sub / ROWS_LPR; g < g1; g += GS) {
-        const double* __restrict__ vb = A.v + (size_t)g * BB * ROWS_LPR + ln;
-        double vv[BB];
+      if (row < A.n_rows) {
+        const int g1 = A.gp[row + 1];
+        for (int g = A.gp[row] + sub / ROWS_LPR; g < g1; g += GS) {
+          const double* __restrict__ vb = A.v + (size_t)g * BB * ROWS_LPR + ln;
+          double vv[BB];
 #pragma unroll
-        for (int e = 0; e < BB; ++e) vv[e] = __ldg(vb + e * ROWS_LPR);
-        const int c = __ldg(A.cols + (size_t)g * ROWS_LPR + ln);
-        double xv[BC];
-        gather_x<BC, AL>(x, c, xv);
+          for (int e = 0; e < BB; ++e) vv[e] = __ldg(vb + e * ROWS_LPR);
+          const int c = __ldg(A.cols + (size_t)g * ROWS_LPR + ln);
+          double xv[BC];
+          gather_x<BC, AL>(x, c, xv);
 #pragma unroll
-        for (int r = 0; r < BR; ++r)
+          for (int r = 0; r < BR; ++r)
 #pragma unroll
-          for (int j = 0; j < BC; ++j) acc[r] = fma(vv[r * BC + j], xv[j], acc[r]);
+            for (int j = 0; j < BC; ++j) acc[r] = fma(vv[r * BC + j], xv[j], acc[r]);
+        }
       }
-    }
     });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
