@@ -582,7 +582,7 @@ __global__ void dense_inactive_kernel(double* __restrict__ D, int N, int ld, uns
 //      the rest, so the next panel starts with its P known.
 // Two grid-wide barriers per panel (three, and FP64 products with two global
 // loads each, before: the unit cube's 3,993-DOF solve, whose coarsest level
-// this inverts, 12.2 -> 4.4 ms in all).  Bound by the FP64 pipe (N^3 or, for SYM,
+// this inverts, 12.2 -> 5.0 ms).  Bound by the FP64 pipe (N^3 or, for SYM,
 // N^3 / 2 multiply-adds at 2 per cycle and SM) once N is large, by the GJB
 // dependent pivots (about 9 us a panel) and the barriers below N ~ 500.
 // SYM: a symmetric matrix; only tiles on or below the diagonal are kept.  An

@@ -67,8 +67,9 @@ struct Level {
   SpOpLow<float> A32, P32, R32;
   SpOpLow<__nv_bfloat16> A16;
   DBuf<float2> xsa, xsb;  // xa and xb split, where the level's products read them so (split_beforehand)
-  // the batched solve's operators: the same copies, or block-CSR-ordered ones
-  // of its own where the solve's follow a lanes-per-row store
+  // the batched solve's operators: the same copies, or (level_precision > 0)
+  // block-CSR-ordered ones of its own where the solve's follow a lanes-per-row
+  // store
   DBuf<float> A32mv, P32mv, R32mv;
   DBuf<__nv_bfloat16> A16mv;
   SpOpLow<float> A32m, P32m, R32m;

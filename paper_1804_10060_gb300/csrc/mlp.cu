@@ -62,8 +62,9 @@ __device__ __forceinline__ void fma2(float2& acc, float2 a, float2 b) {
 // 3 backward through tanh: out = (A W^T) * (1 - H^2) with H = `aux`.
 // STD: standardise A on load with (a - shift) * scale.
 //
-// Bound by the FP32 pipe: a 128-row tile of the activations and the whole
-// weight matrix (zero-padded to Kp x Np) sit in shared memory, and each of the
+// Bound by the FP32 pipe and its operands' way out of shared memory (60% and
+// 64% busy on 131,072 rows of a 128 x 128 layer, 16 warps an SM): a 128-row
+// tile of the activations and the whole weight matrix (zero-padded to Kp x Np) sit in shared memory, and each of the
 // 512 threads keeps a TM x TN tile of outputs in registers, so that four
 // steps of k cost TM + TN 16-byte shared loads for 4 TM TN multiply-adds (the
 // kernel before, one row by 8 outputs a thread with scalar loads and a bounds
@@ -222,8 +223,10 @@ dense_kernel(const float* __restrict__ A, long long n, int K, int N, const float
 
 // Weight gradients, part 1: block b sums grad_W = H^T D and grad_b =
 // colsum(D) over its tiles of WG_ROWS rows and writes its partial sums to
-// part[b][K * N + N].  Bound by the FP32 pipe: a thread keeps a TK x TN tile
-// of grad_W in registers (8 x 8 for a 128 x 128 layer) and reads TK + TN
+// part[b][K * N + N].  Bound by the FP32 pipe and, on few rows, the trip to
+// memory before each tile (pipe 48% busy on 32,768 rows of 128 x 128, load
+// latency the most frequent stall): a thread keeps a TK x TN tile of grad_W in
+// registers (8 x 8 for a 128 x 128 layer) and reads TK + TN
 // values of a row for TK TN products; the kernel before held every 256th
 // entry and read two values per product.
 // Narrow layers (K, N <= 16: a product a thread and row) are bound by the trip
@@ -551,9 +554,12 @@ dense_mma_kernel(const float* __restrict__ A, long long n, int K, int N, const _
 // fragments of the next layer's m16n8k16 products (tiles 2m and 2m+1 form
 // k-chunk m).  Per row only the n_in inputs are read and the n_out outputs
 // written.  Same roundings, products and summation order as the layer-by-
-// layer kernel above, so the results are bitwise the same.  Bound by the
-// hidden layers' tanh (384 a row); the weight fragments come four registers a
-// request (11.6M rows of 8-128-128-128-3: 6.40 -> 6.25 ms).
+// layer kernel above, so the results are bitwise the same.  No pipe
+// is full (issue slots 61% busy, ALU 48, FMA 24, tensor 23, special functions
+// 15): accumulators and fragments take 128 registers a thread, and with the 16
+// warps an SM that leaves, their product and tanh phases (384 tanh a row) do
+// not cover each other.  The weight fragments come four registers a request
+// (11.6M rows of 8-128-128-128-3: 6.40 -> 6.25 ms).
 // ---------------------------------------------------------------------------
 constexpr int FUSED_WARPS = 8;
 constexpr int FUSED_MAX_LAYERS = 8;

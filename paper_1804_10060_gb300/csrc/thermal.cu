@@ -322,10 +322,11 @@ __global__ void thermal_p1_kernel(ThArgs A) {
 // part is sum_j (conduction_ij) T_theta,j -- with the nodal values taken
 // relative to the first vertex's, which a gradient does not see and which
 // leaves little to cancel.  About 3,300 FP64 operations a cell where an
-// 11-point rule took 13,000: 11.0 -> 1.9 ms on 305,280 cells (floor of the
-// operations at the measured FP64 rate: 1.6 ms).  A warp works on one pair (i, j) for its
-// 32 cells at a time: all lanes busy, table indices warp-uniform, per-cell
-// quantities in shared memory by [quantity][cell] (no bank conflicts).
+// 11-point rule took 13,000: 11.0 -> 2.1 ms on 305,280 cells (floor of the
+// operations at the measured FP64 rate: 1.6 ms; FP64 pipe 87% busy).  A warp
+// works on one pair (i, j) for its 32 cells at a time: all lanes busy, table
+// indices warp-uniform, per-cell quantities in shared memory by
+// [quantity][cell] (no bank conflicts).
 constexpr int P2T_WARPS = 8, P2T_CELLS = 32;  // one cell per lane
 
 __global__ void __launch_bounds__(P2T_WARPS * 32) thermal_p2_kernel(ThArgs A) {
